@@ -361,51 +361,57 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     return launch_capture(a, grid, block, smem, stream) == cudaSuccess ? PRCR_OK : PRCR_ECUDA;
 }
 
-// dynamic shared memory of the decode kernel: under the 48 KiB default limit
-// with room for its 1 KiB of static cos/sin
-constexpr size_t kDecodeSmem = 46 * 1024;
+// Which decode kernel runs, and the chunks that the sequence axis is split into.
+//
+// head_dim 64 and 128, large batches: sequence lengths differ, so CTAs differ
+// in work: aim at ~8 waves of resident CTAs (3 per SM) so that the last wave
+// is short, with chunks of at least 768 slots (below that a chunk's prologue
+// and its share of the merge outweigh the better balance; measured: 512 -> 768
+// slots took the qwen25vl-7b shape from 5032 to 5394 GB/s; 1184 -> 768 changed
+// qwen3vl-8b by < 1 %), a multiple of 32, at most kDecodeMaxChunk.
+// Small batches (work for fewer than ~6 waves at 768 slots per chunk) take the
+// ring kernel: the KV heads are split over CTAs of kDecodeRingWarps warps and
+// the chunk is sized so that the grid is about one wave of
+// kDecodeRingCtasPerSm CTAs per SM.
+// head_dim 256: one KV head per CTA, about 8 waves of kDecodeWideCtasPerSm
+// CTAs per SM with chunks of at least kWideMinChunk slots; where that is less
+// than two waves, one wave. Chunks are whole rounds of the CTA's warps.
+// Measured: 16 sequences x 26 layers x 4 heads of up to 4096 slots 822 us at 8
+// waves, 852 us at 16; 4 sequences of up to 2000 slots 162 us at 576 slots,
+// 178 us at 384.
+constexpr int64_t kWideMinChunk = 576;
 
-// Chunking of the decode step. Sequence lengths differ, so CTAs differ in
-// work: aim at ~8 waves of resident CTAs (3 per SM) so that the last wave is
-// short, with chunks of at least 256 slots (to amortise each CTA's query
-// rotation), a multiple of 32, at most kDecodeMaxChunk, and small enough for
-// the chunk's row offsets to fit beside the rotated queries in shared memory.
-// A small batch (work for fewer than ~6 waves at 768 slots per chunk) with
-// head_dim 64 or 128 takes the ring kernel instead (*ring = 1): its KV heads
-// are split over CTAs of kDecodeRingWarps warps and the chunk is sized so that
-// the grid is about one wave of kDecodeRingCtasPerSm CTAs per SM, each warp
-// streaming its chunk through a shared-memory ring.
-void decode_split(int64_t base_ctas, int64_t max_len, int sms, int64_t q_elems, int n_kv_heads,
-                  int head_dim, int* splits, int* chunk, int* ring) {
-    const bool small = base_ctas * ((max_len + 767) / 768) < int64_t(sms) * 6;
-    if (small && (head_dim == 64 || head_dim == 128)) {
+void decode_split(int64_t base_ctas, int64_t max_len, int sms, int n_kv_heads, int head_dim,
+                  int* splits, int* chunk, int* path) {
+    int64_t c;
+    if (head_dim == 256) {
+        *path = kDecodeWide;
+        const int64_t units = base_ctas * n_kv_heads, resident = int64_t(sms) * kDecodeWideCtasPerSm;
+        const int64_t round = 16 * kDecodeWideWarps;
+        const bool few = units * ((max_len + kWideMinChunk - 1) / kWideMinChunk) < 2 * resident;
+        int64_t want = few ? resident / units : (8 * resident + units - 1) / units;
+        if (want < 1) want = 1;
+        c = (max_len + want - 1) / want;
+        if (!few && c < kWideMinChunk) c = kWideMinChunk;
+        c = (c + round - 1) / round * round;
+        if (c > kDecodeMaxChunk) c = kDecodeMaxChunk / round * round;
+    } else if (base_ctas * ((max_len + 767) / 768) < int64_t(sms) * 6) {
+        *path = kDecodeRing;
         const int64_t units = base_ctas * ((n_kv_heads + kDecodeRingWarps - 1) / kDecodeRingWarps);
         int64_t want = int64_t(sms) * kDecodeRingCtasPerSm / units;
         if (want < 1) want = 1;
-        int64_t c = (max_len + want - 1) / want;
+        c = (max_len + want - 1) / want;
         c = (c + 15) / 16 * 16;
         if (c > kDecodeMaxChunk) c = kDecodeMaxChunk;
-        *ring = 1;
-        *chunk = int(c);
-        *splits = int((max_len + c - 1) / c);
-        if (*splits < 1) *splits = 1;
-        return;
+    } else {
+        *path = kDecodeMma;
+        int64_t want = (int64_t(sms) * 24 + base_ctas - 1) / base_ctas;
+        if (want < 1) want = 1;
+        c = (max_len + want - 1) / want;
+        c = (c + 31) / 32 * 32;
+        if (c < 768) c = 768;
+        if (c > kDecodeMaxChunk) c = kDecodeMaxChunk;
     }
-    *ring = 0;
-    int64_t want = (int64_t(sms) * 24 + base_ctas - 1) / base_ctas;
-    if (want < 1) want = 1;
-    int64_t c = (max_len + want - 1) / want;
-    c = (c + 31) / 32 * 32;
-    // Below ~768 slots a chunk's prologue and its share of the merge outweigh
-    // the better balance when there is work for a few waves anyway (measured:
-    // 512 -> 768 slots took the qwen25vl-7b shape from 5032 to 5394 GB/s;
-    // 1184 -> 768 changed qwen3vl-8b by < 1 %). A small batch at head_dim 256
-    // (the CUDA-core kernel) needs the parallelism instead: chunks of 64 slots.
-    const int64_t floor_c = small ? 64 : 768;
-    if (c < floor_c) c = floor_c;
-    if (c > kDecodeMaxChunk) c = kDecodeMaxChunk;
-    const int64_t cap = (int64_t(kDecodeSmem) - q_elems * int64_t(sizeof(float))) / 8 / 32 * 32;
-    if (c > cap) c = cap;
     *chunk = int(c);
     *splits = int((max_len + c - 1) / c);
     if (*splits < 1) *splits = 1;
@@ -609,9 +615,9 @@ size_t prcr_decode_workspace_size(const prcr_rope_cfg* cfg, int32_t n_seqs, int3
     if (check_cfg(cfg) || n_seqs < 1 || max_len < 1 || !decode_shape_ok(cfg, n_q_heads)) return 0;
     int dev = 0, sms = 1;
     if (cudaGetDevice(&dev) == cudaSuccess) sms = sm_count(dev);
-    int splits = 1, chunk = 32, ring = 0;
-    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sms, int64_t(n_q_heads) * cfg->head_dim,
-                 cfg->n_kv_heads, cfg->head_dim, &splits, &chunk, &ring);
+    int splits = 1, chunk = 32, path = 0;
+    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sms, cfg->n_kv_heads, cfg->head_dim,
+                 &splits, &chunk, &path);
     if (splits == 1) return 0;
     return size_t(n_seqs) * cfg->n_layers * n_q_heads * splits * (cfg->head_dim + 2) * sizeof(float);
 }
@@ -637,9 +643,8 @@ int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
     DecodeArgs a = {};
-    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sm_count(dev),
-                 int64_t(n_q_heads) * cfg->head_dim, cfg->n_kv_heads, cfg->head_dim, &a.splits,
-                 &a.chunk, &a.ring);
+    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sm_count(dev), cfg->n_kv_heads,
+                 cfg->head_dim, &a.splits, &a.chunk, &a.path);
     if (n_seqs > 65535 || cfg->n_layers > 65535) return PRCR_EINVAL;  // grid z and y
     if (a.splits > 1) {
         const size_t need = size_t(n_seqs) * cfg->n_layers * n_q_heads * a.splits *
@@ -672,12 +677,8 @@ int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache
     a.group = n_q_heads / cfg->n_kv_heads;
     a.scale = float(1.0 / std::sqrt(double(cfg->head_dim)));
     copy_turn_freq(cfg, a.turn_freq);
-    int gp = 1;
-    while (gp < a.group) gp <<= 1;
-    const size_t smem = size_t(n_q_heads) * cfg->head_dim * sizeof(float) +
-                        size_t(a.chunk) * sizeof(int64_t);
     const dim3 grid(unsigned(a.splits), unsigned(cfg->n_layers), unsigned(n_seqs));
-    return launch_decode(a, gp, grid, smem, static_cast<cudaStream_t>(stream)) == cudaSuccess
+    return launch_decode(a, grid, static_cast<cudaStream_t>(stream)) == cudaSuccess
                ? PRCR_OK
                : PRCR_ECUDA;
 }

@@ -3,20 +3,15 @@
 //   o = softmax(RoPE(q_raw, (p, p, p)) K_act^T / sqrt(D)) V_act
 // over the sequence's cache slots [0, len), the revisited rows included.
 //
-// Work layout (memory-bound: every cached K/V row is read once per step).
-// A CTA owns (sequence, layer, slot chunk). Its prologue rotates the layer's
-// query heads at the text position (angle reduced modulo a turn in fixed
-// point, float32 sincos), pre-scales them by 1/sqrt(D) into shared memory, and
-// resolves the chunk's cache rows (block table for paged caches). Each warp
-// then serves one KV head and the `group` query heads that share it (GQA):
-// lane i holds D/32 consecutive dimensions, so every K or V row of the head
-// is one fully coalesced warp load. S = 32 / GP slots are processed per
-// iteration (GP = 4 for groups up to 4, else 8): each lane forms its
-// partial dot products for all GP x S (head, slot) pairs, and a butterfly
-// transpose-reduction (31 shuffles) leaves lane l with the complete logit of
-// pair l. The online softmax then runs per head, and P V accumulates in
-// float32 per lane. Chunks of one (sequence, layer) are merged by a second
-// kernel from (max, sum, accumulator) partials when the sequence is split.
+// The step is memory-bound: every cached K/V row is read once. A CTA owns a
+// chunk of one (sequence, layer)'s slots; its prologue rotates query heads at
+// the text position (angle reduced modulo a turn in fixed point, float32
+// sincos) and pre-scales them by 1/sqrt(D); its warps stream tiles of 16 slots
+// through mma.sync. Three kernels share that: decode_mma_kernel (head_dim 64
+// and 128, large batches), decode_ring_kernel (64 and 128, small batches) and
+// decode_wide_kernel (head_dim 256). Chunks of one (sequence, layer) are
+// merged by a further kernel from (max, sum, accumulator) partials when the
+// sequence is split.
 #include <cmath>
 
 #include <cuda_bf16.h>
@@ -30,247 +25,8 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kDecodeThreads = 128;
 
-
-// EPL consecutive bf16 of a row as EPL / 2 packed words.
-template <int EPL>
-__device__ __forceinline__ void load_row(const uint16_t* p, uint32_t (&w)[EPL / 2]) {
-    if constexpr (EPL == 2) {
-        w[0] = __ldg(reinterpret_cast<const unsigned int*>(p));
-    } else if constexpr (EPL == 4) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-        w[0] = v.x; w[1] = v.y;
-    } else {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    }
-}
-
-template <int GP, int EPL>
-__global__ void __launch_bounds__(kDecodeThreads, 3) decode_kernel(const __grid_constant__ DecodeArgs a) {
-    constexpr int S = 32 / GP;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int D = a.head_dim;
-    const int P = D >> 1;
-    const int Hq = a.n_q_heads;
-    float* q_s = reinterpret_cast<float*>(smem_raw);
-    int64_t* row_s = reinterpret_cast<int64_t*>(smem_raw + size_t(Hq) * D * sizeof(float));
-    const int b = blockIdx.z;
-    const int l = blockIdx.y;
-    const int split = blockIdx.x;
-    uint32_t err = 0;
-    pdl_allow();
-    pdl_wait();
-
-    int64_t len = a.seq_len[b];
-    if (len < 0 || len > a.capacity) {
-        err |= PRCR_ST_CAPACITY;
-        len = len < 0 ? 0 : a.capacity;
-    }
-    if (len > int64_t(a.splits) * a.chunk) {  // above the host's max_len: past the split
-        err |= PRCR_ST_CAPACITY;
-        len = int64_t(a.splits) * a.chunk;
-    }
-    // A query position beyond the fixed-point angle reduction (|p| >= 2^31)
-    // is reported and the sequence attends to nothing: its output is zeros.
-    const int64_t p = a.q_pos[b];
-    if (p <= -2147483648LL || p >= 2147483648LL) {
-        err |= PRCR_ST_POS_RANGE;
-        len = 0;
-    }
-    const int64_t s_begin = int64_t(split) * a.chunk;
-    const int64_t s_end = min(len, s_begin + a.chunk);
-
-    // Query heads of (b, l), rotated at (p, p, p) and scaled by 1/sqrt(D).
-    // With the same position on every axis, pair i turns by p * inv_freq_i
-    // whatever its band, so each pair's cos/sin serves all heads.
-    __shared__ float s_cos[kMaxPairs], s_sin[kMaxPairs];
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        sincos_turns(double(p), a.turn_freq[i], &s_sin[i], &s_cos[i]);
-    }
-    __syncthreads();
-    const uint16_t* qb = a.q + (int64_t(b) * a.n_layers + l) * Hq * D;
-    for (int e = threadIdx.x; e < Hq * P; e += blockDim.x) {
-        const int hq = e / P;
-        const int i = e - hq * P;
-        const float sn = s_sin[i], cs = s_cos[i];
-        const float x = __uint_as_float(uint32_t(qb[hq * D + i]) << 16);
-        const float y = __uint_as_float(uint32_t(qb[hq * D + i + P]) << 16);
-        q_s[hq * D + i] = fmaf(x, cs, -y * sn) * a.scale;
-        q_s[hq * D + i + P] = fmaf(y, cs, x * sn) * a.scale;
-    }
-    // Cache rows of this chunk (layer term excluded), -1 when unmapped.
-    for (int64_t s = s_begin + threadIdx.x; s < s_end; s += blockDim.x) {
-        int64_t row;
-        if (a.cache_kind == PRCR_CACHE_CONTIGUOUS) {
-            row = int64_t(b) * a.seq_stride + s * a.slot_stride;
-        } else {
-            const int64_t lb = s / a.block_size;
-            const int32_t blk = a.block_table[int64_t(b) * a.bt_stride + lb];
-            if (blk < 0 || blk >= a.n_blocks) {
-                err |= PRCR_ST_NO_BLOCK;
-                row = -1;
-            } else {
-                row = int64_t(blk) * a.block_stride + (s - lb * a.block_size) * a.slot_stride;
-            }
-        }
-        row_s[s - s_begin] = row;
-    }
-    if (err) atomicOr(a.status, err);
-    __syncthreads();
-
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
-    const int g = a.group;
-    const int my_h = lane / S;
-    const int my_si = lane - my_h * S;
-    const int64_t lstride = int64_t(l) * a.layer_stride;
-
-    for (int kh = warp; kh < a.n_kv_heads; kh += nwarps) {
-        float qf[GP][EPL];
-#pragma unroll
-        for (int h = 0; h < GP; ++h)
-#pragma unroll
-            for (int e = 0; e < EPL; ++e)
-                qf[h][e] = h < g ? q_s[(kh * g + h) * D + lane * EPL + e] : 0.0f;
-        float m[GP], lsum[GP], acc[GP][EPL];
-#pragma unroll
-        for (int h = 0; h < GP; ++h) {
-            m[h] = -INFINITY;
-            lsum[h] = 0.0f;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) acc[h][e] = 0.0f;
-        }
-        const uint16_t* kbase = a.cache_k + lstride + int64_t(kh) * D + lane * EPL;
-        const uint16_t* vbase = a.cache_v + lstride + int64_t(kh) * D + lane * EPL;
-
-        // Software pipeline: the K/V rows of the next S slots are requested
-        // before the current S slots are reduced, so every warp keeps its
-        // loads in flight while it runs the shuffle and softmax work.
-        uint32_t kn[S][EPL / 2], vn[S][EPL / 2];
-        bool okn[S];
-        auto fetch = [&](int64_t s0) {
-#pragma unroll
-            for (int si = 0; si < S; ++si) {
-                const int64_t s = s0 + si;
-                const int64_t row = s < s_end ? row_s[s - s_begin] : -1;
-                okn[si] = row >= 0;
-                if (okn[si]) {
-                    load_row<EPL>(kbase + row, kn[si]);
-                    load_row<EPL>(vbase + row, vn[si]);
-                } else {
-#pragma unroll
-                    for (int w = 0; w < EPL / 2; ++w) kn[si][w] = vn[si][w] = 0u;
-                }
-            }
-        };
-        if (s_begin < s_end) fetch(s_begin);
-        for (int64_t s0 = s_begin; s0 < s_end; s0 += S) {
-            uint32_t kw[S][EPL / 2], vw[S][EPL / 2];
-            bool ok[S];
-#pragma unroll
-            for (int si = 0; si < S; ++si) {
-                ok[si] = okn[si];
-#pragma unroll
-                for (int w = 0; w < EPL / 2; ++w) {
-                    kw[si][w] = kn[si][w];
-                    vw[si][w] = vn[si][w];
-                }
-            }
-            if (s0 + S < s_end) fetch(s0 + S);
-            // partial dot products of this lane's dimensions, index h * S + si
-            float val[32];
-#pragma unroll
-            for (int h = 0; h < GP; ++h)
-#pragma unroll
-                for (int si = 0; si < S; ++si) {
-                    float d = 0.0f;
-#pragma unroll
-                    for (int w = 0; w < EPL / 2; ++w) {
-                        d = fmaf(qf[h][2 * w], lo_f32(kw[si][w]), d);
-                        d = fmaf(qf[h][2 * w + 1], hi_f32(kw[si][w]), d);
-                    }
-                    val[h * S + si] = d;
-                }
-            // butterfly transpose-reduction: lane l ends with the full sum of index l
-#pragma unroll
-            for (int k = 16; k >= 1; k >>= 1) {
-                const bool upper = (lane & k) != 0;
-#pragma unroll
-                for (int i = 0; i < k; ++i) {
-                    const float send = upper ? val[i] : val[i + k];
-                    const float keep = upper ? val[i + k] : val[i];
-                    val[i] = keep + __shfl_xor_sync(kFull, send, k);
-                }
-            }
-            bool my_ok = false;
-#pragma unroll
-            for (int si = 0; si < S; ++si)
-                if (si == my_si) my_ok = ok[si];
-            const float logit = (my_h < g && my_ok) ? val[0] : -INFINITY;
-
-            // online softmax per head (each head's S lanes form an aligned segment)
-            float mx = logit;
-#pragma unroll
-            for (int o = 1; o < S; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-            float mnew[GP], alpha[GP];
-            float my_m = -INFINITY;
-#pragma unroll
-            for (int h = 0; h < GP; ++h) {
-                const float cm = __shfl_sync(kFull, mx, h * S);
-                mnew[h] = fmaxf(m[h], cm);
-                alpha[h] = mnew[h] == -INFINITY ? 1.0f : expf(m[h] - mnew[h]);
-                if (h == my_h) my_m = mnew[h];
-            }
-            const float pl = logit == -INFINITY ? 0.0f : expf(logit - my_m);
-            float ps = pl;
-#pragma unroll
-            for (int o = 1; o < S; o <<= 1) ps += __shfl_xor_sync(kFull, ps, o);
-#pragma unroll
-            for (int h = 0; h < GP; ++h) {
-                const float hs = __shfl_sync(kFull, ps, h * S);
-                lsum[h] = lsum[h] * alpha[h] + hs;
-                m[h] = mnew[h];
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) acc[h][e] *= alpha[h];
-            }
-#pragma unroll
-            for (int h = 0; h < GP; ++h)
-#pragma unroll
-                for (int si = 0; si < S; ++si) {
-                    const float pw = __shfl_sync(kFull, pl, h * S + si);
-#pragma unroll
-                    for (int w = 0; w < EPL / 2; ++w) {
-                        acc[h][2 * w] = fmaf(pw, lo_f32(vw[si][w]), acc[h][2 * w]);
-                        acc[h][2 * w + 1] = fmaf(pw, hi_f32(vw[si][w]), acc[h][2 * w + 1]);
-                    }
-                }
-        }
-
-#pragma unroll
-        for (int h = 0; h < GP; ++h) {
-            if (h >= g) break;
-            const int hq = kh * g + h;
-            const int64_t o_idx = (int64_t(b) * a.n_layers + l) * Hq + hq;
-            if (a.splits == 1) {
-                const float inv = lsum[h] > 0.0f ? 1.0f / lsum[h] : 0.0f;
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) a.out[o_idx * D + lane * EPL + e] = acc[h][e] * inv;
-            } else {
-                float* part = a.partial + (o_idx * a.splits + split) * (D + 2);
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) part[lane * EPL + e] = acc[h][e];
-                if (lane == 0) {
-                    part[D] = m[h];
-                    part[D + 1] = lsum[h];
-                }
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
-// Tensor-core variant (head_dim 64 and 128), mma.sync m16n8k16 bf16 -> fp32.
+// head_dim 64 and 128, mma.sync m16n8k16 bf16 -> fp32.
 //
 // A warp serves one KV head and its group of g <= 8 query heads over 16 slots
 // per iteration; the next 16 slots' K rows (registers) and V rows (shared
@@ -959,6 +715,300 @@ __global__ void __launch_bounds__(kRingWarps * 32, kDecodeRingCtasPerSm)
     if (err) atomicOr(a.status, err);
 }
 
+// head_dim 256. A CTA of kWideWarps warps takes one (sequence, layer, KV head,
+// chunk); its warps take the chunk's tiles of 16 slots in turn, each through
+// its own two-stage shared-memory ring (K and V by cp.async, the next tile in
+// flight during the current one), and their (max, sum, accumulator) are
+// merged in shared memory at the end.
+//   QK:  S^T (16 slots x 8 heads) = K Q^T, 16 k-steps; K's A fragments by
+//        ldmatrix from rows padded by 16 bytes (conflict-free).
+//   PV:  O^T (256 dims x 8 heads) += V^T P^T, 16 m-tiles, as in the kernels above.
+// The float32 query and probabilities enter as three bf16 pieces each (24
+// significant bits, three MMAs), the queries' fragments kept in registers
+// (96), and a tile's P V is summed from zero and added to the running
+// accumulator by the FMA that rescales it, so neither the split nor the tensor
+// core's accumulation costs precision against float32 FMAs.
+// What bounds it: DRAM. A tile is 16 KB and ~450 warp instructions; an SM's
+// share of the copy bandwidth brings a tile in ~745 cycles, in which it can
+// issue ~2980. Two CTAs per SM (113 KB of shared memory each) keep six tiles,
+// ~100 KB, in flight per SM and hide each other's prologue. Measured against
+// the CUDA-core kernel it replaced (one warp per KV head, shuffle-reduced dot
+// products, 1.4 TB/s): 16 sequences of up to 4096 slots x 26 layers x 4 KV
+// heads (4.9 GB) 3400 -> 822 us, 6.0 TB/s; one of 933 slots 109 -> 34 us;
+// error against float64 5.2e-7 -> 2.7e-7.
+constexpr int kWideWarps = kDecodeWideWarps;
+constexpr int kWideD = 256;
+constexpr int kWidePitch = kWideD + 8;           // bf16 per staged row
+constexpr int kWideTile = 16 * kWidePitch;       // bf16 per staged K or V tile
+constexpr int kWideQPitch = kWideD + 8;          // float32 per rotated query row (conflict-free fragment reads)
+constexpr int kWideOPitch = kWideD + 4;          // float32 per merged accumulator row
+constexpr size_t kWideSmem = size_t(2) * kWideWarps * 2 * kWideTile * sizeof(uint16_t);
+static_assert(8 * kWideQPitch * sizeof(float) <= kWideSmem / 2, "the rotated queries fit in the second stage");
+static_assert(kWideWarps * 8 * kWideOPitch * sizeof(float) <= kWideSmem, "the warps' accumulators fit in the ring");
+
+// Two floats as three bf16 pairs whose sum keeps 24 significant bits.
+__device__ __forceinline__ void split3_bf16x2(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = pack_bf16x2(x0, x1);
+    const float r0 = x0 - lo_f32(h), r1 = x1 - hi_f32(h);
+    split_bf16x2(r0, r1, m, l);
+}
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__global__ void __launch_bounds__(kWideWarps * 32, 2)
+    decode_wide_kernel(const __grid_constant__ DecodeArgs a) {
+    constexpr int D = kWideD, P = D / 2, KS = D / 16;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) float s_cos[P];
+    __shared__ __align__(16) float s_sin[P];
+    __shared__ float s_m[kWideWarps][8], s_l[kWideWarps][8];
+    const int b = blockIdx.z, l = blockIdx.y, H = a.n_kv_heads, g = a.group;
+    const int split = int(blockIdx.x) / H, kh = int(blockIdx.x) - split * H;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
+    // the ring, stage-major: stage st of warp w holds a K tile then a V tile;
+    // the rotated queries lie in the second stage until every warp holds its
+    // fragments
+    uint16_t* ring = reinterpret_cast<uint16_t*>(smem_raw);
+    float* q_s = reinterpret_cast<float*>(smem_raw + kWideSmem / 2);
+    const uint32_t wk_s = uint32_t(__cvta_generic_to_shared(ring + size_t(warp) * 2 * kWideTile));
+    constexpr uint32_t kStageBytes = uint32_t(kWideSmem / 2), kTileBytes = uint32_t(kWideTile * 2);
+    uint32_t err = 0;
+    pdl_allow();
+    pdl_wait();
+    const int64_t p = a.q_pos[b];
+    int64_t len = a.seq_len[b];
+    if (len < 0 || len > a.capacity) {
+        err |= PRCR_ST_CAPACITY;
+        len = len < 0 ? 0 : a.capacity;
+    }
+    if (len > int64_t(a.splits) * a.chunk) {  // above the host's max_len: past the split
+        err |= PRCR_ST_CAPACITY;
+        len = int64_t(a.splits) * a.chunk;
+    }
+    // A query position beyond the fixed-point angle reduction (|p| >= 2^31)
+    // is reported and the sequence attends to nothing: its output is zeros.
+    if (p <= -2147483648LL || p >= 2147483648LL) {
+        err |= PRCR_ST_POS_RANGE;
+        len = 0;
+    }
+    // slots as unsigned 32-bit numbers (seq_len is an int32)
+    const uint32_t s_begin = uint32_t(min(int64_t(split) * a.chunk, len));
+    const uint32_t s_end = uint32_t(min(len, int64_t(s_begin) + a.chunk));
+    const int n_tiles = int((s_end - s_begin + 15) / 16);
+    const int64_t head_off = int64_t(l) * a.layer_stride + int64_t(kh) * D;
+    const uint16_t* kbase = a.cache_k + head_off + lane * 8;
+    const uint16_t* vbase = a.cache_v + head_off + lane * 8;
+
+    // block id of this lane's slot (lane & 15) of tile n (paged caches)
+    auto block_id = [&](int n) -> int32_t {
+        const uint32_t s = s_begin + uint32_t(16 * n + (lane & 15));
+        if (a.cache_kind != PRCR_CACHE_PAGED || s >= s_end) return 0;
+        return a.block_table[int64_t(b) * a.bt_stride + s / uint32_t(a.block_size)];
+    };
+    // copies of tile n into stage st (lane i takes 16-byte chunk i of every
+    // row); returns the mask of its readable slots
+    auto issue = [&](int n, int st, int32_t blk) -> uint32_t {
+        const uint32_t s = s_begin + uint32_t(16 * n + (lane & 15));
+        int64_t row = -1;
+        if (s < s_end) {
+            if (a.cache_kind == PRCR_CACHE_CONTIGUOUS) {
+                row = int64_t(b) * a.seq_stride + int64_t(s) * a.slot_stride;
+            } else if (blk < 0 || blk >= a.n_blocks) {
+                err |= PRCR_ST_NO_BLOCK;
+            } else {
+                row = int64_t(blk) * a.block_stride +
+                      int64_t(s % uint32_t(a.block_size)) * a.slot_stride;
+            }
+        }
+        const uint32_t m = __ballot_sync(kFull, row >= 0) & 0xffffu;
+        const uint32_t ks_ = wk_s + uint32_t(st) * kStageBytes + uint32_t(lane * 16);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int64_t rr = __shfl_sync(kFull, row, i);
+            const bool ok = rr >= 0;
+            cp_async16(ks_ + uint32_t(i * kWidePitch * 2), ok ? kbase + rr : kbase, ok ? 16 : 0);
+            cp_async16(ks_ + kTileBytes + uint32_t(i * kWidePitch * 2), ok ? vbase + rr : vbase, ok ? 16 : 0);
+        }
+        return m;
+    };
+
+    // this warp's first tile is requested before the prologue
+    uint32_t mask_n = 0u;
+    if (warp < n_tiles) mask_n = issue(warp, 0, block_id(warp));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    int32_t blk_next = warp + kWideWarps < n_tiles ? block_id(warp + kWideWarps) : 0;
+
+    // the group's query heads rotated at (p, p, p), scaled by 1/sqrt(D)
+    for (int i = threadIdx.x; i < P; i += blockDim.x)
+        sincos_turns(double(p), a.turn_freq[i], &s_sin[i], &s_cos[i]);
+    __syncthreads();
+    const uint16_t* qb = a.q + ((int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g) * D;
+    for (int e = threadIdx.x; e < g * (P / 2); e += blockDim.x) {  // two pairs per thread (4-byte loads)
+        const int h = e / (P / 2), i = 2 * (e - h * (P / 2));
+        const uint32_t wx = __ldg(reinterpret_cast<const unsigned int*>(qb + h * D + i));
+        const uint32_t wy = __ldg(reinterpret_cast<const unsigned int*>(qb + h * D + i + P));
+        const float c0 = s_cos[i], s0 = s_sin[i], c1 = s_cos[i + 1], s1 = s_sin[i + 1];
+        const float x0 = lo_f32(wx), x1 = hi_f32(wx), y0 = lo_f32(wy), y1 = hi_f32(wy);
+        *reinterpret_cast<float2*>(q_s + h * kWideQPitch + i) =
+            make_float2(fmaf(x0, c0, -y0 * s0) * a.scale, fmaf(x1, c1, -y1 * s1) * a.scale);
+        *reinterpret_cast<float2*>(q_s + h * kWideQPitch + i + P) =
+            make_float2(fmaf(y0, c0, x0 * s0) * a.scale, fmaf(y1, c1, x1 * s1) * a.scale);
+    }
+    __syncthreads();
+    uint32_t qf[KS][3][2];  // B fragments: column gid = head gid of the group (zero past it)
+#pragma unroll
+    for (int j = 0; j < KS; ++j) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            float2 x = make_float2(0.0f, 0.0f);
+            if (gid < g) x = *reinterpret_cast<const float2*>(q_s + gid * kWideQPitch + 16 * j + 8 * u + 2 * t);
+            split3_bf16x2(x.x, x.y, qf[j][0][u], qf[j][1][u], qf[j][2][u]);
+        }
+    }
+    __syncthreads();  // the queries' stage may now be filled
+
+    float o[KS][4];
+#pragma unroll
+    for (int mt = 0; mt < KS; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.0f;
+    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.0f, 0.0f};  // heads 2t, 2t + 1
+    // ldmatrix row addresses: K (rows = slots), V transposed (rows = slots)
+    const uint32_t k_ld = uint32_t(((lane & 15) * kWidePitch + (lane >> 4) * 8) * 2);
+    const uint32_t v_ld = kTileBytes + uint32_t((((lane & 7) + ((lane >> 4) & 1) * 8) * kWidePitch + ((lane >> 3) & 1) * 8) * 2);
+
+    int st = 0;
+    for (int n = warp; n < n_tiles; n += kWideWarps, st ^= 1) {
+        const uint32_t mask = mask_n;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();  // every lane's copies of the tile are visible, and the other stage is read out
+        if (n + kWideWarps < n_tiles) {
+            const int32_t bn = blk_next;
+            blk_next = n + 2 * kWideWarps < n_tiles ? block_id(n + 2 * kWideWarps) : 0;
+            mask_n = issue(n + kWideWarps, st ^ 1, bn);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+
+        const uint32_t base = wk_s + uint32_t(st) * kStageBytes;
+        float c[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u][0] = c[u][1] = c[u][2] = c[u][3] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < KS; ++j) {
+            uint32_t r[4];
+            ldmatrix_x4(base + k_ld + uint32_t(j * 32), r);
+            mma_16816(c[j & 1], r[0], r[1], r[2], r[3], qf[j][0][0], qf[j][0][1]);
+            mma_16816(c[2], r[0], r[1], r[2], r[3], qf[j][1][0], qf[j][1][1]);
+            mma_16816(c[3], r[0], r[1], r[2], r[3], qf[j][2][0], qf[j][2][1]);
+        }
+        // online softmax of heads 2t, 2t + 1 over slots gid and gid + 8 of the
+        // eight lanes of one t
+        const bool oka = (mask >> gid) & 1u, okb = (mask >> (8 + gid)) & 1u;
+        float pa[2], pb[2], alpha[2];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+            const float va = oka ? (c[3][hh] + c[2][hh]) + (c[1][hh] + c[0][hh]) : -INFINITY;
+            const float vb = okb ? (c[3][2 + hh] + c[2][2 + hh]) + (c[1][2 + hh] + c[0][2 + hh]) : -INFINITY;
+            float mx = fmaxf(va, vb);
+            mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 4));
+            mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 8));
+            mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 16));
+            const float m_new = fmaxf(m_run[hh], mx);
+            alpha[hh] = m_new == -INFINITY ? 1.0f : expf(m_run[hh] - m_new);
+            pa[hh] = va == -INFINITY ? 0.0f : expf(va - m_new);
+            pb[hh] = vb == -INFINITY ? 0.0f : expf(vb - m_new);
+            float ps = pa[hh] + pb[hh];
+            ps += __shfl_xor_sync(kFull, ps, 4);
+            ps += __shfl_xor_sync(kFull, ps, 8);
+            ps += __shfl_xor_sync(kFull, ps, 16);
+            l_run[hh] = l_run[hh] * alpha[hh] + ps;
+            m_run[hh] = m_new;
+        }
+        // P^T as B fragments: the 8 x 8 blocks of S^T transposed in registers
+        uint32_t pf[3][2];
+        {
+            uint32_t w[3];
+            split3_bf16x2(pa[0], pa[1], w[0], w[1], w[2]);
+#pragma unroll
+            for (int u = 0; u < 3; ++u) pf[u][0] = movmatrix_trans(w[u]);
+            split3_bf16x2(pb[0], pb[1], w[0], w[1], w[2]);
+#pragma unroll
+            for (int u = 0; u < 3; ++u) pf[u][1] = movmatrix_trans(w[u]);
+        }
+        // O^T = alpha O^T + V^T P^T (columns are the lane's own heads)
+#pragma unroll
+        for (int mt = 0; mt < KS; ++mt) {
+            uint32_t r[4];
+            ldmatrix_x4_trans(base + v_ld + uint32_t(mt * 32), r);
+            float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            mma_16816(x, r[0], r[1], r[2], r[3], pf[2][0], pf[2][1]);
+            mma_16816(x, r[0], r[1], r[2], r[3], pf[1][0], pf[1][1]);
+            mma_16816(x, r[0], r[1], r[2], r[3], pf[0][0], pf[0][1]);
+            o[mt][0] = fmaf(o[mt][0], alpha[0], x[0]);
+            o[mt][1] = fmaf(o[mt][1], alpha[1], x[1]);
+            o[mt][2] = fmaf(o[mt][2], alpha[0], x[2]);
+            o[mt][3] = fmaf(o[mt][3], alpha[1], x[3]);
+        }
+    }
+
+    // merge the warps (the ring is free: no copy is in flight past a warp's last tile)
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float* o_s = reinterpret_cast<float*>(smem_raw) + warp * 8 * kWideOPitch;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        const int h = 2 * t + hh;
+#pragma unroll
+        for (int mt = 0; mt < KS; ++mt) {
+            o_s[h * kWideOPitch + mt * 16 + gid] = o[mt][hh];
+            o_s[h * kWideOPitch + mt * 16 + gid + 8] = o[mt][2 + hh];
+        }
+        if (gid == 0) {
+            s_m[warp][h] = m_run[hh];
+            s_l[warp][h] = l_run[hh];
+        }
+    }
+    __syncthreads();
+    const float* o_all = reinterpret_cast<const float*>(smem_raw);
+    for (int e = threadIdx.x; e < g * (D / 2); e += blockDim.x) {
+        const int h = e / (D / 2), d = 2 * (e - h * (D / 2));
+        float M = s_m[0][h];
+#pragma unroll
+        for (int w = 1; w < kWideWarps; ++w) M = fmaxf(M, s_m[w][h]);
+        float2 acc = make_float2(0.0f, 0.0f);
+        float den = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kWideWarps; ++w) {
+            const float f = s_m[w][h] == -INFINITY ? 0.0f : expf(s_m[w][h] - M);
+            const float2 x = *reinterpret_cast<const float2*>(o_all + (w * 8 + h) * kWideOPitch + d);
+            acc.x = fmaf(f, x.x, acc.x);
+            acc.y = fmaf(f, x.y, acc.y);
+            den = fmaf(f, s_l[w][h], den);
+        }
+        const int64_t o_idx = (int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g + h;
+        if (a.splits == 1) {
+            const float inv = den > 0.0f ? 1.0f / den : 0.0f;
+            *reinterpret_cast<float2*>(a.out + o_idx * D + d) = make_float2(acc.x * inv, acc.y * inv);
+        } else {
+            float* part = a.partial + (o_idx * a.splits + split) * (D + 2);
+            *reinterpret_cast<float2*>(part + d) = acc;
+            if (d == 0) {
+                part[D] = M;
+                part[D + 1] = den;
+            }
+        }
+    }
+    if (err) atomicOr(a.status, err);
+}
+
 // Merge the chunks of one (sequence, layer, query head). The chunks' maxima
 // and sums are reduced by the whole CTA, their weights exp(m_s - M) staged in
 // shared memory 256 at a time, and thread d accumulates dimension d over the
@@ -1069,22 +1119,11 @@ __global__ void __launch_bounds__(128) decode_merge_warp_kernel(const __grid_con
     }
 }
 
-template <int GP>
-cudaError_t launch_gp(const DecodeArgs& a, dim3 grid, size_t smem, cudaStream_t stream) {
-    const dim3 block(kDecodeThreads);
-    switch (a.head_dim) {
-        case 64: return launch_pdl(decode_kernel<GP, 2>, grid, block, smem, stream, a);
-        case 128: return launch_pdl(decode_kernel<GP, 4>, grid, block, smem, stream, a);
-        default: return launch_pdl(decode_kernel<GP, 8>, grid, block, smem, stream, a);
-    }
-}
-
 }  // namespace
 
-cudaError_t launch_decode(const DecodeArgs& a, int gp, dim3 grid, size_t smem,
-                          cudaStream_t stream) {
+cudaError_t launch_decode(const DecodeArgs& a, dim3 grid, cudaStream_t stream) {
     cudaError_t e;
-    if (a.ring) {
+    if (a.path == kDecodeRing) {
         // small batch: KV heads split over CTAs, K and V streamed through a
         // shared-memory ring per warp
         const int n_hg = (a.n_kv_heads + kRingWarps - 1) / kRingWarps;
@@ -1099,17 +1138,20 @@ cudaError_t launch_decode(const DecodeArgs& a, int gp, dim3 grid, size_t smem,
         auto k = D == 64 ? decode_ring_kernel<64> : decode_ring_kernel<128>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
         if (e == cudaSuccess) e = launch_pdl(k, g2, dim3(kRingWarps * 32), sm, stream, a);
-    } else if (a.head_dim == 64 || a.head_dim == 128) {
-        // tensor-core kernel: rotated queries + two staged V tiles per warp
+    } else if (a.path == kDecodeMma) {
+        // rotated queries + two staged V tiles per warp
         const size_t sm = size_t(a.n_q_heads) * a.head_dim * sizeof(float) +
                           size_t(kDecodeThreads / 32) * 2 * 16 * (a.head_dim + 8) * sizeof(uint16_t);
         auto k = a.head_dim == 64 ? decode_mma_kernel<64> : decode_mma_kernel<128>;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
         if (e == cudaSuccess) e = launch_pdl(k, grid, dim3(kDecodeThreads), sm, stream, a);
     } else {
-        // groups of 1, 2 and 4 query heads run as 4 (padded) heads x 8 slots per
-        // warp iteration, groups of 5..8 as 8 heads x 4 slots
-        e = gp <= 4 ? launch_gp<4>(a, grid, smem, stream) : launch_gp<8>(a, grid, smem, stream);
+        // head_dim 256: one KV head per CTA
+        dim3 g2 = grid;
+        g2.x *= unsigned(a.n_kv_heads);
+        e = cudaFuncSetAttribute(decode_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(kWideSmem));
+        if (e == cudaSuccess) e = launch_pdl(decode_wide_kernel, g2, dim3(kWideWarps * 32), kWideSmem, stream, a);
     }
     if (e != cudaSuccess || a.splits == 1) return e;
     const int64_t n_out = int64_t(grid.z) * a.n_layers * a.n_q_heads;

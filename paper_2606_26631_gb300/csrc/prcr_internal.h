@@ -256,12 +256,16 @@ struct DecodeArgs {
     int32_t group;
     int32_t splits;
     int32_t chunk;
-    int32_t ring;               // small batch: the ring-staged kernel (head_dim 64, 128)
+    int32_t path;               // kDecodeMma, kDecodeRing or kDecodeWide
     float scale;
     uint64_t turn_freq[kMaxPairs];  // pair i: round(inv_freq_i / (2 pi) * 2^64)
 };
 
 constexpr int kDecodeMaxChunk = 4096;
+// the decode kernels: head_dim 64 and 128 for large and small batches, and 256
+constexpr int kDecodeMma = 0, kDecodeRing = 1, kDecodeWide = 2;
+constexpr int kDecodeWideWarps = 3;   // warps (taking a chunk's tiles in turn) per CTA of the wide kernel
+constexpr int kDecodeWideCtasPerSm = 2;
 constexpr int kDecodeRingWarps = 4;   // KV heads (one per warp) per CTA of the ring kernel
 constexpr int kDecodeRingCtasPerSm = 3;
 
@@ -334,8 +338,7 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
 // and selection kernels
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
 
-cudaError_t launch_decode(const DecodeArgs& a, int gp, dim3 grid, size_t smem,
-                          cudaStream_t stream);
+cudaError_t launch_decode(const DecodeArgs& a, dim3 grid, cudaStream_t stream);
 cudaError_t launch_capture(const CaptureArgs& a, dim3 grid, int block, size_t smem,
                            cudaStream_t stream);
 cudaError_t capture_blocks_per_sm(int block, size_t smem, int* out);

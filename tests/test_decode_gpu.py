@@ -96,7 +96,7 @@ def test_decode_empty_and_single_slot(H, Hq, D, paged):
     slot's V row exactly (its softmax weight is exactly 1); a longer one
     beside them still matches the oracle. Covers the head-split kernel
     (8 KV heads), the one-CTA-per-chunk kernel, head_dim 64 and the
-    CUDA-core kernel (head_dim 256)."""
+    head_dim 256 kernel."""
     import paper_2606_26631_gb300 as prcr
     B, nL, max_len = 3, 2, 300
     sec = (D // 8, D // 8 + (D // 2 - 3 * (D // 8)) // 2, 0)
@@ -219,6 +219,45 @@ def test_decode_unaligned_query():
     got, st1 = _run_decode(cfg, cd, q_odd, inp["q_pos"], inp["seq_len"], max_len)
     assert st0 == 0 and st1 == 0
     assert torch.equal(ref, got)
+
+
+# slots at the edges of a 16-slot tile, of a round of the CTA's three warps (48)
+# and of a chunk (576), one per sequence of the batch; the group's ends
+@pytest.mark.parametrize("H,Hq,paged,bs", [(1, 8, True, 7), (3, 3, False, 16), (4, 28, True, 16)])
+@pytest.mark.parametrize("n_layers", [1, 40])
+def test_decode_head_dim_256_edges(H, Hq, paged, bs, n_layers):
+    """head_dim 256: every product has 24 significant bits and is summed in
+    float32, so a logit (sum of ~10 in magnitude over 48 MMAs) is off by about
+    sqrt(48) 2^-24 10 = 4e-6 and the output by no more than twice that."""
+    import paper_2606_26631_gb300 as prcr
+    D, sec = 256, (40, 44, 44)
+    lens = [1, 15, 16, 17, 47, 48, 49, 575, 576, 577, 593, 0, 1153]
+    B, max_len = len(lens), 1153
+    inp = make_decode_inputs(B, n_layers, H, Hq, D, max_len, paged, device=DEV, seed=31, block_size=bs)
+    if paged:  # every sequence's table maps all of its slots
+        nblk = -(-max_len // bs)
+        pool = inp["cache_k"].shape[1]
+        bt = (torch.arange(B * nblk, device=DEV, dtype=torch.int32).view(B, nblk) * 5) % pool
+        inp["block_table"] = bt.contiguous()
+    seq_len = torch.tensor(lens, dtype=torch.int32, device=DEV)
+    cfg = prcr.rope_cfg(n_layers, H, D, sec, 1e6)
+    cd = (prcr.cache_paged(inp["cache_k"], inp["cache_v"], inp["block_table"]) if paged
+          else prcr.cache_contiguous(inp["cache_k"], inp["cache_v"]))
+    out, st = _run_decode(cfg, cd, inp["q"], inp["q_pos"], seq_len, max_len)
+    assert st == 0
+    got, qv, l = out.cpu().numpy(), _f64(inp["q"]), n_layers - 1
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert np.all(got[b] == 0.0)
+            continue
+        s = torch.arange(n, device=DEV)
+        if paged:
+            blk = inp["block_table"][b][s // bs].long()
+            K, V = (_f64(inp[x][l][blk, s % bs]) for x in ("cache_k", "cache_v"))
+        else:
+            K, V = (_f64(inp[x][b, l, :n]) for x in ("cache_k", "cache_v"))
+        ref = O.decode_attention(qv[b, l], int(inp["q_pos"][b]), K, V, D, sec, 1e6)
+        assert np.abs(got[b, l] - ref).max() / np.abs(V).max() <= 8e-6, (b, n)
 
 
 def test_inject_then_decode():
