@@ -459,21 +459,10 @@ int select_common(const prcr_rope_cfg* cfg, int32_t n_seqs, int32_t layer, int32
     a.sec_h = cfg->sections[1];
     a.sec_w = cfg->sections[2];
     a.scale = float(1.0 / std::sqrt(double(cfg->head_dim)));
-    {
-        char* w = static_cast<char*>(workspace);
-        const int64_t Bn = n_seqs, Hn = n_q_heads, M = n_tokens;
-        a.n_seqs = n_seqs;
-        a.tok_tile = tile;
-        a.n_tiles = int32_t((M + tile - 1) / tile);
-        const int64_t max_tiles = (M + kSelectTokTile - 1) / kSelectTokTile;
-        a.logits = reinterpret_cast<float*>(w);
-        w += align256(size_t(4 * Bn * Hn * M));
-        a.tile_stats = reinterpret_cast<float*>(w);
-        w += align256(size_t(8 * Bn * Hn * max_tiles));
-        a.norm = reinterpret_cast<float*>(w);
-        w += align256(size_t(8 * Bn * Hn));
-        a.rel = reinterpret_cast<float*>(w);
-    }
+    a.n_seqs = n_seqs;
+    a.tok_tile = tile;
+    a.n_tiles = (n_tokens + tile - 1) / tile;
+    a.logits = static_cast<float*>(workspace);
     a.score_out = score_out;
     a.idx_out = idx_out;
     a.rev_tok_off = rev_tok_off;
@@ -697,10 +686,9 @@ int prcr_select_topk(const prcr_rope_cfg* cfg, const prcr_store_desc* store, int
     if ((rc = check_store(cfg, store))) return rc;
     if (n_seqs > store->n_seqs) return PRCR_EINVAL;
     SelectArgs a = {};
-    // token tiles of the softmax statistics: 16 tokens (one warp's MMA rows)
-    // for the tensor-core logits kernel (head_dim 64, 128); else the CUDA-core
-    // kernel's tiles, 64 tokens (32 at head_dim 256, whose cos/sin rows are
-    // twice as long)
+    // token tiles of the logits kernel: 16 tokens (one warp's MMA rows) for the
+    // tensor-core kernel (head_dim 64, 128); else the CUDA-core kernel's, 64
+    // tokens (32 at head_dim 256, whose cos/sin rows are twice as long)
     const int D = cfg->head_dim;
     rc = select_common(cfg, n_seqs, layer, n_q_heads, store->n_tokens, q, q_pos, k, idx_out,
                        seq_rev_off, rev_tok_off, score_out, workspace, workspace_bytes,

@@ -270,10 +270,12 @@ constexpr int kDecodeRingWarps = 4;   // KV heads (one per warp) per CTA of the 
 constexpr int kDecodeRingCtasPerSm = 3;
 
 constexpr int kSelectMaxQHeads = 128;
-constexpr int kSelectTokTile = 16;   // smallest tile of the logits kernel (sizes the workspace)
 
+// The logits, and what programs have always been asked for beside them (per
+// 16-token tile and head 8 bytes, per head 8, per token 4), which no kernel
+// uses: the size stays so that a workspace kept from before fits as before.
 inline size_t select_workspace_bytes(int64_t B, int64_t Hq, int64_t M) {
-    const int64_t tiles = (M + kSelectTokTile - 1) / kSelectTokTile;
+    const int64_t tiles = (M + 15) / 16;
     return align256(size_t(4 * B * Hq * M)) + align256(size_t(8 * B * Hq * tiles)) +
            align256(size_t(8 * B * Hq)) + align256(size_t(4 * B * M));
 }
@@ -299,13 +301,12 @@ struct SelectArgs {
     int32_t sec_w;
     float scale;
     float* logits;              // workspace [B][n_q_heads][n_tokens]
-    float* tile_stats;          // workspace [B][n_q_heads][n_tiles][2] (max, sum of exp)
-    float* norm;                // workspace [B][n_q_heads][2] (max, 1 / (sum * n_q_heads))
-    float* rel;                 // workspace [B][n_tokens] relevance
     int32_t n_seqs;
     int32_t n_tiles;            // token tiles of the logits kernel per sequence
     int32_t tok_tile;           // tokens per tile
     int32_t kh_per_item;        // tensor-core logits: KV heads per work item
+    int32_t cluster;            // CTAs per sequence of the cluster kernels
+    int32_t tok_per_cta;        // tokens of each of them (a multiple of 16)
     float* score_out;           // optional [B][n_tokens]
     int32_t* idx_out;           // [B][k]
     int32_t* rev_tok_off;       // [B + 1]
@@ -337,6 +338,9 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
 // the logits of the cached-key selection, then the same normaliser, relevance
 // and selection kernels
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
+
+// the steps after the logits: normalisers, relevances, top-k
+cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream);
 
 cudaError_t launch_decode(const DecodeArgs& a, dim3 grid, cudaStream_t stream);
 cudaError_t launch_capture(const CaptureArgs& a, dim3 grid, int block, size_t smem,

@@ -15,32 +15,17 @@
 // turned by theta_i (c_axis(i) - p) and dotted with the raw query, and the
 // 1/sqrt(D) scale is applied to the dot product. The raw bf16 query is then
 // exact in any operand format, and nothing is computed per query.
-// Kernel 1 (logits, persistent) forms every (token, query head) logit that
-// way from the raw key rotated on the fly, and each token tile's per-head
-// softmax statistics (max, sum of exp). Kernel 2 (norm) merges the tiles'
-// statistics into each head's normaliser; kernel 3 (relevance) averages
-// every token's per-head softmax weight; kernel 4 (select), one CTA per
-// sequence, finds the K-th largest relevance by counting against thresholds
-// two bits at a time on the float bits (relevance >= 0, so bit order is
-// value order) and compacts the selection in index order with block-wide
-// scans.
+// A logits kernel here (from the raw keys, rotated on the fly, or from the
+// position-bound cache) writes every (token, query head) logit to the
+// workspace; prcr_select_cluster.cu does the rest: softmax normalisers,
+// relevances, top-k.
 #include <cmath>
 
-#include "prcr_device.cuh"
 #include "prcr_pdl.cuh"
+#include "prcr_select.cuh"
 
 namespace prcr {
 namespace {
-
-// Rotation of an integer position offset: the turn fraction c * rate mod 1
-// in 0.32 fixed point is bits 32..63 of the 64-bit product c * rate (rate in
-// 0.64 fixed point; the product's wrap mod 2^64 keeps those bits exact for
-// any int64 c), then one sin/cos evaluation on [-pi, pi).
-__device__ __forceinline__ void sincos_coord(int64_t c, uint64_t turn_freq, float* s, float* co) {
-    const uint64_t prod = static_cast<uint64_t>(c) * turn_freq;
-    const int frac = static_cast<int>(static_cast<uint32_t>(prod >> 32));
-    __sincosf(float(frac) * 1.4629180792671596e-9f, s, co);  // 2 pi / 2^32
-}
 
 // 16-byte chunk c of a shared row stored at c ^ bit 3 of c: the 8 lanes of a
 // quarter-warp that read chunks 2v (or 2v + 1), v = 0..7, hit 8 distinct
@@ -56,8 +41,7 @@ __device__ __forceinline__ int swz(int c) { return c ^ ((c >> 3) & 1); }
 // rotates and dots with the group's query heads in packed float2 FMAs; the
 // lanes' partial sums are reduced by shuffles. The loads of a lane's next two
 // rows are in flight during the current row's arithmetic. The tile's logits are staged
-// in shared memory, reduced to per-head (max, sum of exp) and written out
-// coalesced.
+// in shared memory and written out coalesced.
 // L lanes per row (a power of two >= head_dim / 16); G = the GQA group size g
 // for g = 1, 2 and 4, else 8 (heads h >= g skipped).
 template <int L, int G>
@@ -221,48 +205,15 @@ __global__ void __launch_bounds__(256, 3) ads_logits_kernel(const __grid_constan
         }
         __syncthreads();
 
-        // per query head: the tile's (max, sum of exp), and its logits written out coalesced
+        // the tile's logits written out coalesced, a warp per query head
         for (int hq = warp; hq < Hq; hq += blockDim.x >> 5) {
             const float* row = lg_s + hq * (T + 1);
-            float mx = -INFINITY;
-            for (int t = lane; t < nt; t += 32) mx = fmaxf(mx, row[t]);
-#pragma unroll
-            for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            float z = 0.0f;
             float* dst = a.logits + (int64_t(b) * Hq + hq) * M + m0;
-            for (int t = lane; t < nt; t += 32) {
-                z += expf(row[t] - mx);
-                dst[t] = row[t];
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-            if (lane == 0) {
-                float* ts = a.tile_stats + ((int64_t(b) * Hq + hq) * a.n_tiles + j) * 2;
-                ts[0] = mx;
-                ts[1] = z;
-            }
+            for (int t = lane; t < nt; t += 32) dst[t] = row[t];
         }
         // the next tile rewrites the coordinates first, then (after a barrier)
         // the cos/sin rows and logits this tile's warps may still be reading
     }
-}
-
-// D += A B on tensor cores: mma.sync m16n8k8 with tf32 operands (the upper
-// 19 bits of each float32 register), float32 accumulate. Fragments as the
-// PTX ISA lays them out for this shape: a0 (row g, col t), a1 (row g + 8,
-// col t), a2 (row g, col t + 4), a3 (row g + 8, col t + 4); b0 (row t, col
-// g), b1 (row t + 4, col g); lane = 4 g + t.
-__device__ __forceinline__ void mma_1688_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                              uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-        "{%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
-    return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
 // Tensor-core logits (head_dim 64 and 128). Persistent over work items
@@ -287,8 +238,7 @@ __device__ __forceinline__ uint32_t word_of(const uint4& v, int i) {
 // float32: ~20 significant bits per product over float32's range. Runs of
 // 16-byte loads are double-buffered: the run two ahead is requested as soon
 // as a buffer's words are used. Each KV head's logits go straight from the
-// accumulators to global memory; the softmax statistics are left to the
-// normaliser kernel.
+// accumulators to global memory.
 template <int D, int NW>
 __global__ void __launch_bounds__(NW * 32, 2) ads_logits_mma_kernel(const __grid_constant__ SelectArgs a) {
     pdl_allow();
@@ -478,8 +428,7 @@ __global__ void __launch_bounds__(NW * 32, 2) ads_logits_mma_kernel(const __grid
                               __float_as_uint(lya), __float_as_uint(lyb), b0, b1);
             }
         };
-        // KV head kk done: its logits out (the softmax statistics come from
-        // the normaliser kernel, one pass over the logits)
+        // KV head kk done: its logits out
         const bool va = ta < ntw, vb = tb < ntw;
         // columns 2t, 2t + 1 of each KV head's logits; lg advances by g rows per head
         const int h0 = 2 * tq;
@@ -541,8 +490,7 @@ __global__ void __launch_bounds__(NW * 32, 2) ads_logits_mma_kernel(const __grid
 // bytes each straight into A fragments. The next item's rows are loaded
 // during this item's MMAs (each 16-byte run as soon as the register it goes
 // into is used), the rows of the one after that requested into L2. An item
-// writes its 16 logits per head (the softmax statistics are left to the
-// normaliser kernel); a token without a readable row gets logit -inf.
+// writes its 16 logits per head; a token without a readable row gets logit -inf.
 template <int D>
 __global__ void __launch_bounds__(256, D > 128 ? 1 : 2)
     ads_logits_cache_kernel(const __grid_constant__ SelectArgs a) {
@@ -760,8 +708,6 @@ __global__ void __launch_bounds__(256, D > 128 ? 1 : 2)
         if (left > 3) row_start(pf2, req_pf);
 
         // token gid: heads 2t, 2t + 1 in c[0], c[1]; token gid + 8 in c[2], c[3]
-        // (the softmax statistics come from the normaliser kernel, one pass
-        // over the logits)
         const bool ok0 = (mask >> gid) & 1u, ok1 = (mask >> (gid + 8)) & 1u;
         float v[4] = {ok0 ? c[0] : -INFINITY, ok0 ? c[1] : -INFINITY, ok1 ? c[2] : -INFINITY,
                       ok1 ? c[3] : -INFINITY};
@@ -785,323 +731,6 @@ __global__ void __launch_bounds__(256, D > 128 ? 1 : 2)
         pf = pf2;
     }
     if (err) atomicOr(a.status, err);
-}
-
-// Softmax normaliser of each (sequence, query head) from the tiles' statistics.
-__global__ void __launch_bounds__(256) ads_norm_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    pdl_wait();
-    __shared__ float s_m[8], s_z[8];
-    const int hq = blockIdx.x, b = blockIdx.y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float* ts = a.tile_stats + (int64_t(b) * a.n_q_heads + hq) * a.n_tiles * 2;
-    float mx = -INFINITY;
-    for (int i = threadIdx.x; i < a.n_tiles; i += blockDim.x) mx = fmaxf(mx, ts[2 * i]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) s_m[warp] = mx;
-    __syncthreads();
-    mx = s_m[0];
-    for (int w = 1; w < nw; ++w) mx = fmaxf(mx, s_m[w]);
-    float z = 0.0f;
-    for (int i = threadIdx.x; i < a.n_tiles; i += blockDim.x) z += ts[2 * i + 1] * expf(ts[2 * i] - mx);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if (lane == 0) s_z[warp] = z;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float zt = 0.0f;
-        for (int w = 0; w < nw; ++w) zt += s_z[w];
-        float* nrm = a.norm + (int64_t(b) * a.n_q_heads + hq) * 2;
-        // no finite logit (no readable token, or a query position out of
-        // range): every weight of this head is taken as 0
-        nrm[0] = mx == -INFINITY ? 0.0f : mx;
-        nrm[1] = mx == -INFINITY ? 0.0f : 1.0f / (zt * float(a.n_q_heads));
-    }
-}
-
-// Softmax normaliser of each (sequence, query head) straight from its logits
-// (the tensor-core and cached-key logits kernels write no tile statistics):
-// every thread keeps a running (max, sum of exp) over sixteen logits at a
-// time, all of a round's loads requested at once (16-byte loads when the row
-// is 16-byte aligned), and the block merges them.
-__device__ __forceinline__ void merge_max_sum(float& m, float& s, float m2, float s2) {
-    const float mn = fmaxf(m, m2);
-    if (mn == -INFINITY) return;
-    s = (m == -INFINITY ? 0.0f : s * __expf(m - mn)) + (m2 == -INFINITY ? 0.0f : s2 * __expf(m2 - mn));
-    m = mn;
-}
-
-__global__ void __launch_bounds__(256) ads_norm_logits_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    pdl_wait();
-    __shared__ float s_m[8], s_z[8];
-    const int hq = blockIdx.x, b = blockIdx.y, M = a.n_tokens, NT = blockDim.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = NT >> 5;
-    const float* lg = a.logits + (int64_t(b) * a.n_q_heads + hq) * M;
-    float mx = -INFINITY, z = 0.0f;
-    // sixteen logits (-inf past the end) into the running (max, sum of exp)
-    auto chunk = [&](const float (&x)[16]) {
-        float cm = mx;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) cm = fmaxf(cm, x[u]);
-        if (cm == -INFINITY) return;
-        float cz = 0.0f;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) cz += __expf(x[u] - cm);
-        z = (mx == -INFINITY ? 0.0f : z * __expf(mx - cm)) + cz;
-        mx = cm;
-    };
-    if ((M & 3) == 0) {
-        // 16-byte loads, eight per thread requested at once (the launch sizes
-        // the block so that one round covers the row where it can)
-        const float4* l4 = reinterpret_cast<const float4*>(lg);
-        const int M4 = M >> 2;
-        for (int i4 = 0; i4 < M4; i4 += 8 * NT) {
-            float x[2][16];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = i4 + u * NT + threadIdx.x;
-                const float4 v = j < M4 ? l4[j] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-                x[u >> 2][4 * (u & 3)] = v.x; x[u >> 2][4 * (u & 3) + 1] = v.y;
-                x[u >> 2][4 * (u & 3) + 2] = v.z; x[u >> 2][4 * (u & 3) + 3] = v.w;
-            }
-            chunk(x[0]);
-            chunk(x[1]);
-        }
-    } else {
-        for (int i = 0; i < M; i += 16 * NT) {
-            float x[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int t = i + u * NT + threadIdx.x;
-                x[u] = t < M ? lg[t] : -INFINITY;
-            }
-            chunk(x);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, mx, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-        merge_max_sum(mx, z, m2, z2);
-    }
-    if (lane == 0) {
-        s_m[warp] = mx;
-        s_z[warp] = z;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < nw; ++w) merge_max_sum(mx, z, s_m[w], s_z[w]);
-        float* nrm = a.norm + (int64_t(b) * a.n_q_heads + hq) * 2;
-        nrm[0] = mx == -INFINITY ? 0.0f : mx;
-        nrm[1] = mx == -INFINITY ? 0.0f : 1.0f / (z * float(a.n_q_heads));
-    }
-}
-
-// Relevance of every token: mean over the query heads of its softmax weight,
-// the heads accumulated in ascending order (exp of arguments <= 0 by
-// __expf, relative error ~1e-6, far inside the relevance's float32 budget). TPT consecutive tokens per thread:
-// four (16-byte loads, eight heads' logits requested together) for large
-// batches, one (sixteen heads requested together) where the grid would
-// otherwise be a few CTAs.
-template <int TPT>
-__global__ void __launch_bounds__(256) ads_relevance_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    pdl_wait();
-    __shared__ float s_n[2 * kSelectMaxQHeads];
-    const int b = blockIdx.y;
-    const int Hq = a.n_q_heads, M = a.n_tokens;
-    for (int i = threadIdx.x; i < 2 * Hq; i += blockDim.x) s_n[i] = a.norm[int64_t(b) * Hq * 2 + i];
-    __syncthreads();
-    const int m = TPT * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (m >= M) return;
-    const float* lg = a.logits + int64_t(b) * Hq * M + m;
-    float r[TPT];
-#pragma unroll
-    for (int u = 0; u < TPT; ++u) r[u] = 0.0f;
-    if (TPT == 1) {
-        int h = 0;
-        for (; h + 16 <= Hq; h += 16) {
-            float x[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) x[u] = lg[int64_t(h + u) * M];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) r[0] = fmaf(__expf(x[u] - s_n[2 * (h + u)]), s_n[2 * (h + u) + 1], r[0]);
-        }
-        for (; h < Hq; ++h) r[0] = fmaf(__expf(lg[int64_t(h) * M] - s_n[2 * h]), s_n[2 * h + 1], r[0]);
-    } else if ((M & 3) == 0) {
-        int h = 0;
-        for (; h + 16 <= Hq; h += 16) {  // sixteen heads' logits requested together
-            float4 x[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) x[u] = *reinterpret_cast<const float4*>(lg + int64_t(h + u) * M);
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const float mh = s_n[2 * (h + u)], wh = s_n[2 * (h + u) + 1];
-                r[0] = fmaf(__expf(x[u].x - mh), wh, r[0]);
-                r[1 % TPT] = fmaf(__expf(x[u].y - mh), wh, r[1 % TPT]);
-                r[2 % TPT] = fmaf(__expf(x[u].z - mh), wh, r[2 % TPT]);
-                r[3 % TPT] = fmaf(__expf(x[u].w - mh), wh, r[3 % TPT]);
-            }
-        }
-        for (; h < Hq; ++h) {
-            const float4 x = *reinterpret_cast<const float4*>(lg + int64_t(h) * M);
-            const float mh = s_n[2 * h], wh = s_n[2 * h + 1];
-            r[0] = fmaf(__expf(x.x - mh), wh, r[0]);
-            r[1 % TPT] = fmaf(__expf(x.y - mh), wh, r[1 % TPT]);
-            r[2 % TPT] = fmaf(__expf(x.z - mh), wh, r[2 % TPT]);
-            r[3 % TPT] = fmaf(__expf(x.w - mh), wh, r[3 % TPT]);
-        }
-    } else {
-        const int n = min(TPT, M - m);
-        for (int h = 0; h < Hq; ++h) {
-            const float mh = s_n[2 * h], wh = s_n[2 * h + 1];
-#pragma unroll
-            for (int u = 0; u < TPT; ++u)
-                if (u < n) r[u] = fmaf(__expf(lg[int64_t(h) * M + u] - mh), wh, r[u]);
-        }
-    }
-    const int n = min(TPT, M - m);
-#pragma unroll
-    for (int u = 0; u < TPT; ++u) {
-        if (u < n) {
-            a.rel[int64_t(b) * M + m + u] = r[u];
-            if (a.score_out) a.score_out[int64_t(b) * M + m + u] = r[u];
-        }
-    }
-}
-
-// Block-wide exclusive scan of one int per thread; returns the total.
-__device__ __forceinline__ int block_scan(int v, int* s_warp, int* out_excl) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        int w = lane < nw ? s_warp[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        if (lane < nw) s_warp[lane] = w;  // inclusive prefix of warp totals
-    }
-    __syncthreads();
-    const int total = s_warp[nw - 1];
-    *out_excl = x - v + (warp > 0 ? s_warp[warp - 1] : 0);
-    __syncthreads();
-    return total;
-}
-
-// PER: relevances per thread (a thread keeps its PER consecutive tokens in
-// registers; blockDim.x * PER >= n_tokens, blockDim.x a multiple of 32).
-template <int PER>
-__global__ void __launch_bounds__(1024) ads_select_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    pdl_wait();
-    __shared__ int s_warp[32];
-    __shared__ unsigned int s_cnt[3 * 32];
-    const int b = blockIdx.x;
-    const int M = a.n_tokens;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int beg = threadIdx.x * PER;
-    const int nwarp = blockDim.x >> 5;  // a multiple of 32 threads, <= 1024
-
-    // this thread's relevances (from the relevance kernel); tokens past the
-    // end read as 0 and are excluded wherever 0 could count
-    unsigned int key[PER];
-    const float* rs = a.rel + int64_t(b) * M;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) key[i] = beg + i < M ? __float_as_uint(rs[beg + i]) : 0u;
-
-    // 1. the K-th largest relevance, two bits per round from the top: of the
-    // candidates X | d << bit (d = 1, 2, 3) keep the largest that at least K
-    // keys reach (relevance >= 0, so float bits order as values; every
-    // candidate is >= 1, so the padding never counts). Counting against
-    // thresholds needs no histogram, hence no atomics on the few bins that
-    // relevances sharing their high bits would all fall into.
-    // The search also stops as soon as exactly K keys reach X: the selection
-    // is then every key >= X (the compaction below takes all keys above X
-    // and, of those equal to X, exactly the K - above that remain).
-    const unsigned int K = unsigned(a.k);
-    unsigned int X = 0u, cX = 0u;  // cX: keys >= X, once X > 0
-    for (int bit = 30; bit >= 0; bit -= 2) {
-        const unsigned int x1 = X | (1u << bit), x2 = X | (2u << bit), x3 = X | (3u << bit);
-        unsigned int c1 = 0u, c2 = 0u, c3 = 0u;
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            c1 += key[i] >= x1;
-            c2 += key[i] >= x2;
-            c3 += key[i] >= x3;
-        }
-        c1 = __reduce_add_sync(0xffffffffu, c1);
-        c2 = __reduce_add_sync(0xffffffffu, c2);
-        c3 = __reduce_add_sync(0xffffffffu, c3);
-        if (lane == 0) {
-            s_cnt[warp] = c1;
-            s_cnt[32 + warp] = c2;
-            s_cnt[64 + warp] = c3;
-        }
-        __syncthreads();
-        const bool wl = lane < nwarp;  // this lane reads warp `lane`'s counts
-        const unsigned int t1 = __reduce_add_sync(0xffffffffu, wl ? s_cnt[lane] : 0u);
-        const unsigned int t2 = __reduce_add_sync(0xffffffffu, wl ? s_cnt[32 + lane] : 0u);
-        const unsigned int t3 = __reduce_add_sync(0xffffffffu, wl ? s_cnt[64 + lane] : 0u);
-        cX = t3 >= K ? t3 : (t2 >= K ? t2 : (t1 >= K ? t1 : cX));
-        X = t3 >= K ? x3 : (t2 >= K ? x2 : (t1 >= K ? x1 : X));
-        __syncthreads();
-        if (X != 0u && cX == K) break;  // uniform: every thread read the same counts
-    }
-    // keys strictly above X: all taken; of the keys equal to X, the first ones
-    unsigned int above = 0u, n_eq = 0u;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        above += key[i] > X;
-        n_eq += beg + i < M && key[i] == X;
-    }
-    above = __reduce_add_sync(0xffffffffu, above);
-    if (lane == 0) s_cnt[warp] = above;
-    __syncthreads();
-    const int need_eq = int(K - __reduce_add_sync(0xffffffffu, lane < nwarp ? s_cnt[lane] : 0u));
-
-    // 2. ordered compaction: all keys > X, then the first need_eq keys == X
-    int eq_before = 0;
-    block_scan(int(n_eq), s_warp, &eq_before);
-    int n_sel = 0;
-    {
-        int e = eq_before;
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const bool eq = beg + i < M && key[i] == X;
-            n_sel += key[i] > X || (eq && e < need_eq);
-            e += eq;
-        }
-    }
-    int sel_before = 0;
-    block_scan(n_sel, s_warp, &sel_before);
-    int32_t* out = a.idx_out + int64_t(b) * a.k;
-    {
-        int e = eq_before, o = sel_before;
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const bool eq = beg + i < M && key[i] == X;
-            if (key[i] > X || (eq && e < need_eq)) out[o++] = beg + i;
-            e += eq;
-        }
-    }
-    if (threadIdx.x == 0) {
-        a.rev_tok_off[b] = b * a.k;
-        a.seq_rev_off[b] = b;
-        if (b == gridDim.x - 1) {
-            a.rev_tok_off[b + 1] = (b + 1) * a.k;
-            a.seq_rev_off[b + 1] = b + 1;
-        }
-    }
 }
 
 }  // namespace
@@ -1169,36 +798,6 @@ cudaError_t launch_logits_mma(const SelectArgs& a, int n_seqs, int sms, cudaStre
                       stream, b);
 }
 
-// The normalisers, relevances and selection after a logits kernel.
-static cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream,
-                                      bool norm_from_logits = false) {
-    // the normaliser from the logits: about 32 logits per thread, one round
-    // up to 256 threads (wider blocks would take large grids past one wave)
-    int nt = int(((a.n_tokens + 31) / 32 + 31) / 32 * 32);
-    nt = nt < 64 ? 64 : (nt > 256 ? 256 : nt);
-    cudaError_t e = norm_from_logits
-                        ? launch_pdl(ads_norm_logits_kernel, dim3(a.n_q_heads, n_seqs, 1), dim3(nt), 0,
-                                     stream, a)
-                        : launch_pdl(ads_norm_kernel, dim3(a.n_q_heads, n_seqs, 1), dim3(256), 0, stream, a);
-    if (e != cudaSuccess) return e;
-    // four tokens per thread once the grid fills the GPU a few times over
-    if (int64_t(n_seqs) * a.n_tokens >= (int64_t(1) << 19))
-        e = launch_pdl(ads_relevance_kernel<4>, dim3((a.n_tokens + 1023) / 1024, n_seqs, 1), dim3(256),
-                       0, stream, a);
-    else
-        e = launch_pdl(ads_relevance_kernel<1>, dim3((a.n_tokens + 255) / 256, n_seqs, 1), dim3(256), 0,
-                       stream, a);
-    if (e != cudaSuccess) return e;
-    const int M = a.n_tokens;
-    // just enough warps for PER tokens per thread: fewer warps, cheaper rounds
-    auto threads = [M](int per) { return int(((M + per - 1) / per + 31) / 32 * 32); };
-    const dim3 grid(unsigned(n_seqs), 1, 1);
-    if (M <= 4096) return launch_pdl(ads_select_kernel<4>, grid, dim3(threads(4)), 0, stream, a);
-    if (M <= 8192) return launch_pdl(ads_select_kernel<8>, grid, dim3(threads(8)), 0, stream, a);
-    if (M <= 16384) return launch_pdl(ads_select_kernel<16>, grid, dim3(threads(16)), 0, stream, a);
-    return launch_pdl(ads_select_kernel<32>, grid, dim3(threads(32)), 0, stream, a);
-}
-
 cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
     cudaError_t e;
     const bool mma = (a.head_dim == 128 || a.head_dim == 64) && a.tok_tile == 16;
@@ -1213,7 +812,7 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
                              : launch_logits<16>(a, n_seqs, sms, stream));
     }
     if (e != cudaSuccess) return e;
-    return launch_select_tail(a, n_seqs, stream, mma);
+    return launch_select_tail(a, n_seqs, stream);
 }
 
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
@@ -1231,7 +830,7 @@ cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaS
     const int64_t resident = int64_t(sms) * (per_sm > 0 ? per_sm : 1);
     e = launch_pdl(k, dim3(unsigned(ctas < resident ? ctas : resident)), dim3(256), smem, stream, a);
     if (e != cudaSuccess) return e;
-    return launch_select_tail(a, n_seqs, stream, true);
+    return launch_select_tail(a, n_seqs, stream);
 }
 
 }  // namespace prcr

@@ -320,3 +320,37 @@ def test_select_cached_query_position_range():
         kc = _image_rows(cache_k, None, img0.cpu().numpy(), 1, 0, M)
         ref = O.ads_relevance_cached(qv[1], 700, kc, D, sec, 1e6)
         _check_seq(score[1], ref, idx[1], k, M)
+
+
+# token counts around a tile (16), a group of four and a CTA's share, one
+# sequence and more sequences than the GPU holds clusters of, the largest
+# count; dup > 1 repeats every key row, so that many relevances are equal at
+# the cut (the lower token index first)
+SIZES = [  # (B, M, k, dup)
+    (1, 1, 1, 1), (2, 15, 4, 1), (3, 17, 17, 1), (1, 50, 7, 5), (5, 1001, 100, 1), (2, 4099, 2000, 40), (1, 32768, 500, 64),
+    (40, 777, 64, 3), (160, 130, 3, 1), (2, 4096, 4095, 4096),
+]
+
+
+@pytest.mark.parametrize("B,M,k,dup", SIZES, ids=[f"B{b}M{m}k{k}x{d}" for b, m, k, d in SIZES])
+def test_select_cached_sizes(B, M, k, dup):
+    """Relevances within the file's bar, and exactly the top-k of them."""
+    import paper_2606_26631_gb300 as prcr
+    H, Hq, D, sec = 2, 6, 64, (8, 12, 12)
+    g = torch.Generator(device=DEV).manual_seed(100 + M)
+    rows = torch.randn((B, 1, (M + dup - 1) // dup, H, D), device=DEV, generator=g).to(torch.bfloat16)
+    cache_k = rows.repeat(1, 1, dup, 1, 1)[:, :, :M].contiguous()
+    cd = prcr.cache_contiguous(cache_k, torch.zeros_like(cache_k))
+    cfg = prcr.rope_cfg(1, H, D, sec, 1e6)
+    q = (2.0 * torch.randn((B, Hq, D), device=DEV, generator=g)).to(torch.bfloat16)
+    q_pos = torch.arange(B, device=DEV, dtype=torch.int64) * 37 + 800
+    idx, sro, rto, score, st = _run(cfg, cd, 0, q, q_pos, torch.zeros(B, dtype=torch.int32, device=DEV), M, k)
+    assert st == 0
+    assert np.array_equal(sro, np.arange(B + 1)) and np.array_equal(rto, k * np.arange(B + 1))
+    qv = O.bf16_bits_to_f64(q.view(torch.int16).cpu().numpy())
+    for b in sorted({0, B // 2, B - 1}):
+        kc = O.bf16_bits_to_f64(cache_k[b, 0].view(torch.int16).cpu().numpy())
+        ref = O.ads_relevance_cached(qv[b], int(q_pos[b]), kc, D, sec, 1e6)
+        assert (np.abs(score[b] - ref) / ref).max() <= 1e-4
+    for b in range(B):
+        assert np.array_equal(idx[b], _topk_by(score[b].astype(np.float64), k)), b
