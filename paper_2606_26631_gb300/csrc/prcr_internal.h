@@ -339,6 +339,9 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
 // and selection kernels
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
 
+// the whole selection in one kernel, where that is the faster path (else
+// *done = false and nothing is launched)
+cudaError_t launch_select_fused(const SelectArgs& a, bool cached, int n_seqs, int sms, cudaStream_t stream, bool* done);
 // the steps after the logits: normalisers, relevances, top-k
 cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream);
 

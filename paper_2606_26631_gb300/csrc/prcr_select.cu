@@ -799,7 +799,9 @@ cudaError_t launch_logits_mma(const SelectArgs& a, int n_seqs, int sms, cudaStre
 }
 
 cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
-    cudaError_t e;
+    bool done = false;
+    cudaError_t e = launch_select_fused(a, false, n_seqs, sms, stream, &done);
+    if (e != cudaSuccess || done) return e;
     const bool mma = (a.head_dim == 128 || a.head_dim == 64) && a.tok_tile == 16;
     if (a.head_dim == 128 && mma) {
         e = launch_logits_mma<128>(a, n_seqs, sms, stream);
@@ -816,12 +818,15 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
 }
 
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
+    bool done = false;
+    cudaError_t e = launch_select_fused(a, true, n_seqs, sms, stream, &done);
+    if (e != cudaSuccess || done) return e;
     const int g = a.n_q_heads / a.n_kv_heads;
     const size_t smem = size_t(8) * g * a.head_dim * sizeof(float);  // 8 warps
     auto k = a.head_dim == 64 ? ads_logits_cache_kernel<64>
              : a.head_dim == 128 ? ads_logits_cache_kernel<128>
                                  : ads_logits_cache_kernel<256>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
     if (e != cudaSuccess) return e;

@@ -1,5 +1,7 @@
-// The selection's steps after the logits, on clusters of CTAs, one cluster per
-// sequence.
+// The selection on clusters of CTAs, one cluster per sequence: in one kernel
+// from the keys to the indices where the logits fit in the cluster's shared
+// memory (select_fused_kernel), else everything after a logits kernel
+// (select_tail_kernel).
 //
 // Rank r of a cluster of C CTAs takes the tokens r * T .. r * T + T - 1 of its
 // sequence (T = tok_per_cta). Two exchanges through distributed shared memory
@@ -398,6 +400,342 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
     select_topk<NT>(a, b, C, m_beg, nt, keys, lo, hi, sh);
 }
 
+// The whole selection in one kernel. The CTA's logits stay in shared memory;
+// their computation is that of ads_logits_mma_kernel (raw keys turned by the
+// offsets of their coordinates, CACHED = false) or of ads_logits_cache_kernel
+// (position-bound rows against the turned query, CACHED = true), as work items
+// of (16 tokens, KV head) that the CTA's warps take in turn. The queries'
+// fragments, and the raw keys' cos/sin (a pass of 1024 / D tiles at a time),
+// are computed once per CTA; an item's rows are loaded during the item before.
+// Small calls are a chain of latencies, which one kernel shortens by three
+// launches: 768 tokens x 8 KV heads in a cluster of 16, ~20k cycles: queries
+// and first rows 2.7k, cos/sin and MMAs 5.5k, statistics and their exchange
+// 4.8k, relevances and theirs 5k, search and output 2.7k. Measured with its
+// launches 20.9 -> 12.5 us (four kernels before), 8 sequences 20.6 -> 13.6 us,
+// 4 of 1000 tokens at head_dim 256 29.6 -> 13.9 us (CUDA cores before).
+constexpr int kFusedThreads = 512;
+
+// Shared memory of the fused kernel, in the order of its sections.
+struct FusedLayout {
+    int pitch;  // floats per head's row of logits: 4 mod 32, free of bank conflicts for the MMA's accumulators
+    size_t trig, tok, query, logits, keys, total;
+};
+
+__host__ __device__ inline FusedLayout fused_layout(int D, bool cached, int H, int Hq, int T, int C) {
+    FusedLayout f;
+    f.pitch = (T + 31) / 32 * 32 + 4;
+    f.trig = size_t(H) * D * 32;  // after the queries' fragments [H][D / 16][32] uint4
+    const int tiles = T / 16 < 1024 / D ? T / 16 : 1024 / D;
+    f.tok = f.trig + (cached ? 0 : size_t(tiles) * D * 64);          // [tiles][D / 8][32] float4
+    f.query = f.tok + (size_t(T) * (cached ? 8 : 12) + 15) / 16 * 16;  // rows (int64) or coordinates (3 int32)
+    f.logits = f.query + (cached ? size_t(Hq) * (D + 8) * 2 : 0);      // the raw queries
+    f.keys = f.logits + size_t(Hq) * f.pitch * 4;
+    f.total = f.keys + size_t(C) * T * 4;
+    return f;
+}
+
+template <int D, bool CACHED>
+__global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __grid_constant__ SelectArgs a) {
+    constexpr int NT = kFusedThreads, NW = NT / 32, P = D / 2;
+    constexpr int KQ = D / 16;                  // 16-byte fragment entries per lane of a KV head's queries
+    constexpr int NR = CACHED ? D / 32 : D / 64;  // groups of 16-byte loads of an item, refilled as they are used
+    constexpr int RL = CACHED ? 2 : 4;            // loads per group
+    constexpr int TP = 1024 / D;                // tiles of a pass (raw keys)
+    constexpr int QP = D + 8;                   // bf16 per staged query row
+    __shared__ SelectShared sh;
+    __shared__ uint64_t tf_s[P];
+    __shared__ __align__(16) float2 cs_s[CACHED ? P : 1];  // (cos, sin) of the query's turn
+    __shared__ uint8_t ax_s[P];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_allow();
+    const int C = a.cluster, b = int(blockIdx.x) / C, rank = int(cluster_rank()), T = a.tok_per_cta;
+    const int M = a.n_tokens, Hq = a.n_q_heads, H = a.n_kv_heads, g = Hq / H;
+    const int m_beg = rank * T, nt = max(0, min(T, M - m_beg)), n_tiles = (nt + 15) / 16;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tq = lane & 3;
+    const FusedLayout f = fused_layout(D, CACHED, H, Hq, T, C);
+    uint4* qf_s = reinterpret_cast<uint4*>(smem_raw);
+    float4* tr_s = reinterpret_cast<float4*>(smem_raw + f.trig);
+    int* crd_s = reinterpret_cast<int*>(smem_raw + f.tok);
+    int64_t* row_s = reinterpret_cast<int64_t*>(smem_raw + f.tok);
+    uint32_t* q_s = reinterpret_cast<uint32_t*>(smem_raw + f.query);
+    float* lg_s = reinterpret_cast<float*>(smem_raw + f.logits);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + f.keys);
+    for (int i = tid; i < P; i += NT) {
+        tf_s[i] = a.turn_freq[i];
+        ax_s[i] = uint8_t(pair_axis(i, a.layout, a.sec_t, a.sec_h, a.sec_w));
+    }
+    uint32_t err = 0;
+    pdl_wait();
+    const int64_t p = a.q_pos[b];
+    const uint16_t* qs = a.q + int64_t(b) * Hq * D;
+
+    // the items of this warp: warp, warp + NW, ... of (tile, KV head), heads fastest
+    uint4 k[NR][RL];
+    const uint16_t* kb = CACHED ? a.cache_k + int64_t(a.layer) * a.cache_layer_stride + tq * (D / 4)
+                                : a.store_k + int64_t(b) * a.store_seq_stride + int64_t(m_beg) * a.store_token_stride +
+                                      int64_t(a.layer) * a.store_layer_stride + 8 * tq;
+    // this lane's two token rows (gid and gid + 8 of the tile) at KV head kh; a
+    // token past the end reads the last one, one without a row the cache's
+    // first row (their logits are not stored, or are -inf)
+    auto rows = [&](int tile, int kh, const uint16_t* (&r)[2]) {
+        const int ta = min(16 * tile + gid, nt - 1), tb = min(16 * tile + gid + 8, nt - 1);
+        if constexpr (CACHED) {
+            const int64_t ra = row_s[ta], rb = row_s[tb];
+            r[0] = kb + (ra < 0 ? 0 : ra) + kh * D;
+            r[1] = kb + (rb < 0 ? 0 : rb) + kh * D;
+        } else {
+            r[0] = kb + int64_t(ta) * a.store_token_stride + kh * D;
+            r[1] = kb + int64_t(tb) * a.store_token_stride + kh * D;
+        }
+    };
+    auto fetch = [&](uint4 (&x)[RL], const uint16_t* ra, const uint16_t* rb, int u) {
+        if constexpr (CACHED) {
+            x[0] = ld_stream(ra + 8 * u);
+            x[1] = ld_stream(rb + 8 * u);
+        } else {
+            x[0] = ld_stream(ra + 32 * u);
+            x[1] = ld_stream(ra + 32 * u + P);
+            x[2] = ld_stream(rb + 32 * u);
+            x[3] = ld_stream(rb + 32 * u + P);
+        }
+    };
+    const int n_items = n_tiles * H;
+    const uint16_t* r_n[2];
+    auto first = [&]() {
+        if (warp < n_items) {
+            rows(warp / H, warp % H, r_n);
+#pragma unroll
+            for (int u = 0; u < NR; ++u) fetch(k[u], r_n[0], r_n[1], u);
+        }
+    };
+    const uint32_t* q_src = reinterpret_cast<const uint32_t*>(qs);  // 4-byte loads: the ABI's alignment
+    // B fragments of the groups' query heads: one entry per (KV head, j, head of
+    // the group, lane group t); those past the group's heads stay zero
+    auto each_fragment = [&](auto&& make) {
+        if (g < 8)
+            for (int e = tid; e < H * KQ * 32; e += NT)
+                if (gid >= g) qf_s[e] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 4
+        for (int e = tid; e < H * KQ * g * 4; e += NT) {
+            const int t = e & 3, h = (e >> 2) % g, kj = (e >> 2) / g;
+            const int kh = kj / KQ, j = kj % KQ;
+            qf_s[kj * 32 + 4 * h + t] = make(kh * g + h, j, t);
+        }
+    };
+    bool q_ok = true;
+    if constexpr (CACHED) {
+        // the query rows into shared memory, the cache rows of the CTA's tokens
+        // (-1: none), and the query's turn
+#pragma unroll 4
+        for (int i = tid; i < Hq * P; i += NT) q_s[(i / P) * (QP / 2) + i % P] = __ldg(q_src + i);
+        const int64_t s0 = a.img_slot0[b];
+        for (int t = tid; t < nt; t += NT) {
+            const int64_t slot = s0 + m_beg + t;
+            int64_t row = -1;
+            if (slot < 0 || slot >= a.cache_capacity) {
+                err |= PRCR_ST_CAPACITY;
+            } else if (a.cache_kind == PRCR_CACHE_CONTIGUOUS) {
+                row = int64_t(b) * a.cache_seq_stride + slot * a.cache_slot_stride;
+            } else {
+                const int64_t lb = slot <= INT32_MAX ? int64_t(uint32_t(slot) / uint32_t(a.block_size))
+                                                     : slot / a.block_size;
+                const int32_t blk = a.block_table[int64_t(b) * a.bt_stride + lb];
+                if (blk < 0 || blk >= a.n_blocks) err |= PRCR_ST_NO_BLOCK;
+                else row = int64_t(blk) * a.cache_block_stride + (slot - lb * a.block_size) * a.cache_slot_stride;
+            }
+            row_s[t] = row;
+        }
+        // a query position beyond the fixed-point angle reduction is reported
+        // and the sequence's logits are all -inf (relevance 0)
+        q_ok = p > -2147483648LL && p < 2147483648LL;
+        if (!q_ok) err |= PRCR_ST_POS_RANGE;
+        for (int i = tid; i < P; i += NT) {
+            float sn, cs;
+            sincos_fixed(q_ok ? static_cast<long long>(p) * (1ll << 32) : 0ll, tf_s[i], &sn, &cs);
+            cs_s[i] = make_float2(cs, sn);
+        }
+        __syncthreads();
+        first();
+        // dimensions t D/4 + 4j .. + 3 (those that the lane's key loads hold),
+        // turned at (p, p, p) and scaled, a bf16 head and remainder each
+        each_fragment([&](int hq, int j, int t) {
+            const uint32_t* q0 = q_s + hq * (QP / 2);
+            const int d = t * (D / 4) + 4 * j, dp = d < P ? d + P : d - P, i = d < P ? d : dp;
+            const uint2 x = *reinterpret_cast<const uint2*>(q0 + d / 2), y = *reinterpret_cast<const uint2*>(q0 + dp / 2);
+            const float4 ca = *reinterpret_cast<const float4*>(cs_s + i), cb = *reinterpret_cast<const float4*>(cs_s + i + 2);
+            const float sg = d < P ? -1.0f : 1.0f;
+            uint4 o;
+            split_bf16x2(fmaf(lo_f32(x.x), ca.x, sg * lo_f32(y.x) * ca.y) * a.scale,
+                         fmaf(hi_f32(x.x), ca.z, sg * hi_f32(y.x) * ca.w) * a.scale, o.x, o.z);
+            split_bf16x2(fmaf(lo_f32(x.y), cb.x, sg * lo_f32(y.y) * cb.y) * a.scale,
+                         fmaf(hi_f32(x.y), cb.z, sg * hi_f32(y.y) * cb.w) * a.scale, o.y, o.w);
+            return o;
+        });
+        __syncthreads();
+    } else {
+        first();
+        const int32_t* crd = a.coords + int64_t(b) * a.coord_seq_stride + 3 * int64_t(m_beg);
+        for (int i = tid; i < 3 * nt; i += NT) crd_s[i] = crd[i];
+        // the raw query at k-steps 2j and 2j + 1 (exact tf32 operands), whose
+        // pairs are neighbours: one word of each half
+        each_fragment([&](int hq, int j, int t) {
+            const uint32_t* q0 = q_src + hq * P + 16 * (j / 4) + 4 * t + j % 4;
+            const uint32_t w0 = __ldg(q0), w1 = __ldg(q0 + P / 2);
+            return make_uint4(w0 << 16, w1 << 16, w0 & 0xffff0000u, w1 & 0xffff0000u);
+        });
+        __syncthreads();
+    }
+
+    constexpr int STEP = CACHED ? 1 << 28 : TP;  // tiles per pass
+    for (int t0 = 0, it = warp; t0 < n_tiles; t0 += STEP) {
+        const int t1 = min(n_tiles, t0 + STEP);
+        if constexpr (!CACHED) {
+            // cos/sin of (token, pair) at each k-step, in the lanes' order
+            if (t0) __syncthreads();  // the previous pass has been read
+            for (int e = tid; e < (t1 - t0) * (D / 8) * 32; e += NT) {
+                const int s = (e / 32) % (D / 8), tile = t0 + e / (32 * (D / 8));
+                const int i = 32 * (s / 8) + 8 * tq + s % 8, ax = ax_s[i];
+                const int ta = min(16 * tile + gid, nt - 1), tb = min(16 * tile + gid + 8, nt - 1);
+                float4 v;
+                sincos_coord(int64_t(crd_s[3 * ta + ax]) - p, tf_s[i], &v.z, &v.x);
+                sincos_coord(int64_t(crd_s[3 * tb + ax]) - p, tf_s[i], &v.w, &v.y);
+                tr_s[e] = v;
+            }
+            __syncthreads();
+        }
+        for (; it < t1 * H; it += NW) {
+            const int tile = it / H, kh = it - tile * H;
+            const bool more = it + NW < n_items;
+            if (more) rows((it + NW) / H, (it + NW) % H, r_n);
+            constexpr int NC = CACHED ? 4 : 2;  // accumulator chains per head
+            float acc[NC][4];
+#pragma unroll
+            for (int u = 0; u < NC; ++u) acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.0f;
+            const uint4* qf = qf_s + kh * KQ * 32 + lane;
+            if constexpr (CACHED) {
+#pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const uint4 w0 = k[u][0], w1 = k[u][1];
+                    const uint4 qa = qf[(2 * u) * 32], qb = qf[(2 * u + 1) * 32];
+                    mma_16816(acc[0], w0.x, w1.x, w0.y, w1.y, qa.x, qa.y);
+                    mma_16816(acc[1], w0.x, w1.x, w0.y, w1.y, qa.z, qa.w);
+                    mma_16816(acc[NC - 2], w0.z, w1.z, w0.w, w1.w, qb.x, qb.y);
+                    mma_16816(acc[NC - 1], w0.z, w1.z, w0.w, w1.w, qb.z, qb.w);
+                    if (more) fetch(k[u], r_n[0], r_n[1], u);
+                }
+            } else {
+                const float4* tr = tr_s + (tile - t0) * (D / 8) * 32 + lane;
+#pragma unroll
+                for (int u = 0; u < NR; ++u) {
+#pragma unroll
+                    for (int s8 = 0; s8 < 8; ++s8) {
+                        const int w = s8 / 2;
+                        const bool up = s8 & 1;  // upper bf16 of the word
+                        const float4 t = tr[(8 * u + s8) * 32];
+                        const float2 Cs = make_float2(t.x, t.y), Sn = make_float2(t.z, t.w);
+                        const uint32_t xa = word_of(k[u][0], w), ya = word_of(k[u][1], w);
+                        const uint32_t xb = word_of(k[u][2], w), yb = word_of(k[u][3], w);
+                        const float2 X = up ? make_float2(hi_f32(xa), hi_f32(xb)) : make_float2(lo_f32(xa), lo_f32(xb));
+                        const float2 Y = up ? make_float2(hi_f32(ya), hi_f32(yb)) : make_float2(lo_f32(ya), lo_f32(yb));
+                        const float2 ys = __fmul2_rn(Y, Sn), xs = __fmul2_rn(X, Sn);
+                        const float2 Xr = __ffma2_rn(X, Cs, make_float2(-ys.x, -ys.y));
+                        const float2 Yr = __ffma2_rn(Y, Cs, xs);
+                        // tf32 heads by truncation, float32 remainders
+                        const uint32_t hxa = __float_as_uint(Xr.x) & 0xffffe000u, hxb = __float_as_uint(Xr.y) & 0xffffe000u;
+                        const uint32_t hya = __float_as_uint(Yr.x) & 0xffffe000u, hyb = __float_as_uint(Yr.y) & 0xffffe000u;
+                        const float2 lx = __ffma2_rn(make_float2(__uint_as_float(hxa), __uint_as_float(hxb)),
+                                                     make_float2(-1.0f, -1.0f), Xr);
+                        const float2 ly = __ffma2_rn(make_float2(__uint_as_float(hya), __uint_as_float(hyb)),
+                                                     make_float2(-1.0f, -1.0f), Yr);
+                        const uint4 q2 = qf[(4 * u + w) * 32];
+                        const uint32_t b0 = up ? q2.z : q2.x, b1 = up ? q2.w : q2.y;
+                        mma_1688_tf32(acc[0], hxa, hxb, hya, hyb, b0, b1);
+                        mma_1688_tf32(acc[1], __float_as_uint(lx.x), __float_as_uint(lx.y), __float_as_uint(ly.x),
+                                      __float_as_uint(ly.y), b0, b1);
+                    }
+                    if (more) fetch(k[u], r_n[0], r_n[1], u);
+                }
+            }
+            // rows gid and gid + 8 (tokens), columns 2 tq and 2 tq + 1 (heads of the group)
+            const int ta = 16 * tile + gid, tb = ta + 8;
+            bool ok_a = true, ok_b = true;
+            if constexpr (CACHED) {
+                ok_a = q_ok && row_s[min(ta, nt - 1)] >= 0;
+                ok_b = q_ok && row_s[min(tb, nt - 1)] >= 0;
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (2 * tq + c >= g) continue;
+                float va, vb;
+                if constexpr (CACHED) {  // chains 1 and 3: the query's remainder
+                    va = (acc[1][c] + acc[NC - 1][c]) + (acc[0][c] + acc[NC - 2][c]);
+                    vb = (acc[1][2 + c] + acc[NC - 1][2 + c]) + (acc[0][2 + c] + acc[NC - 2][2 + c]);
+                } else {  // chain 1: the keys' remainders
+                    va = (acc[0][c] + acc[1][c]) * a.scale;
+                    vb = (acc[0][2 + c] + acc[1][2 + c]) * a.scale;
+                }
+                float* lg = lg_s + (kh * g + 2 * tq + c) * f.pitch;
+                if (ta < nt) lg[ta] = ok_a ? va : -INFINITY;
+                if (tb < nt) lg[tb] = ok_b ? vb : -INFINITY;
+            }
+        }
+    }
+    if (CACHED && err) atomicOr(a.status, err);
+    __syncthreads();
+
+    // statistics of the CTA's tokens, two heads of a warp side by side
+    for (int h0 = warp; h0 < Hq; h0 += 2 * NW) {
+        const bool two = h0 + NW < Hq;
+        const float* ra = lg_s + h0 * f.pitch;
+        const float* rb = lg_s + (two ? h0 + NW : h0) * f.pitch;
+        float ma = -INFINITY, mb = -INFINITY, za = 0.0f, zb = 0.0f;
+        for (int t = lane; t < nt; t += 32) {
+            ma = fmaxf(ma, ra[t]);
+            mb = fmaxf(mb, rb[t]);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            ma = fmaxf(ma, __shfl_xor_sync(kAll, ma, o));
+            mb = fmaxf(mb, __shfl_xor_sync(kAll, mb, o));
+        }
+        const float sa = ma == -INFINITY ? 0.0f : ma, sb = mb == -INFINITY ? 0.0f : mb;
+        for (int t = lane; t < nt; t += 32) {
+            za += __expf(ra[t] - sa);
+            zb += __expf(rb[t] - sb);
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            za += __shfl_xor_sync(kAll, za, o);
+            zb += __shfl_xor_sync(kAll, zb, o);
+        }
+        if (lane == 0) {
+            sh.stat[h0] = make_float2(ma, za);
+            if (two) sh.stat[h0 + NW] = make_float2(mb, zb);
+        }
+    }
+    merge_stats<NT>(a, C, sh);
+
+    // relevances: `per` lanes share a token (its heads in turn) where the CTA
+    // has few tokens
+    float* rel = reinterpret_cast<float*>(keys + m_beg);
+    const int per = nt * 8 <= NT ? 8 : (nt * 4 <= NT ? 4 : (nt * 2 <= NT ? 2 : 1));
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    for (int i0 = 0; i0 < nt * per; i0 += NT) {
+        const int t = (i0 + tid) / per, j = (i0 + tid) & (per - 1);
+        float r = 0.0f;
+        if (t < nt)
+            for (int h = j; h < Hq; h += per) r = fmaf(__expf(lg_s[h * f.pitch + t] - sh.norm[h].x), sh.norm[h].y, r);
+        for (int o = per / 2; o; o >>= 1) r += __shfl_xor_sync(kAll, r, o);
+        if (t < nt && j == 0) {
+            rel[t] = r;
+            lo = min(lo, __float_as_uint(r));
+            hi = max(hi, __float_as_uint(r));
+            if (a.score_out) a.score_out[int64_t(b) * M + m_beg + t] = r;
+        }
+    }
+    select_topk<NT>(a, b, C, m_beg, nt, keys, lo, hi, sh);
+}
+
 cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaStream_t stream,
                                   cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg = {};
@@ -416,6 +754,8 @@ cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaS
     return cfg;
 }
 
+constexpr int kFusedMinTokens = 32;  // per CTA
+constexpr int kFusedRows = 640;
 constexpr size_t kMaxDynSmem = 208 * 1024;  // beside the static shared memory, within 227 KB
 
 // Clusters of 1..16 CTAs of a kernel that the current device holds at once, one
@@ -475,5 +815,43 @@ cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t str
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kTailThreads, t.cluster,
                                                   size_t(t.cluster) * t.tok_per_cta * 4, stream, attr);
     return cudaLaunchKernelEx(&cfg, select_tail_kernel, t);
+}
+
+// The one-kernel selection, or *done = false where it does not fit or is the
+// slower path. It leaves SMs idle (a cluster per sequence, and clusters do not
+// fill every GPC), so its time grows with the rows (token, KV head) of a CTA,
+// that of a logits kernel and select_tail_kernel with all rows over all SMs,
+// on top of ~6 us more for the second kernel. Measured (us, fused | two
+// kernels), raw keys, 8 heads of 128: 1 sequence of 1024 tokens (512 rows per
+// CTA) 13.0 | 15.2, of 2048 17.7 | 16.3, of 4096 27.8 | 18.1; 7 of 2048 (1024
+// rows) 19.1 | 27.1, of 4096 29.4 | 32.8, of 8192 61.9 | 43.8; 16 of 1024 21.0
+// | 28.9, of 2048 34.3 | 34.7. Cached keys: 1 of 1024 13.4 | 16.4, of 2048
+// 17.6 | 17.1; 7 of 4096 26.3 | 28.1, of 8192 44.9 | 40.1; 16 of 2048 29.1 |
+// 26.6. The line below lies between them.
+template <int D, bool CACHED>
+cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream, bool* done) {
+    auto kern = select_fused_kernel<D, CACHED>;
+    const void* k = reinterpret_cast<const void*>(kern);
+    SelectArgs t = a;
+    cudaError_t e = pick_cluster(k, kFusedThreads, n_seqs, a.n_tokens, kFusedMinTokens, &t.cluster);
+    if (e != cudaSuccess) return e;
+    t.tok_per_cta = tokens_per_cta(a.n_tokens, t.cluster);
+    const FusedLayout f = fused_layout(D, CACHED, a.n_kv_heads, a.n_q_heads, t.tok_per_cta, t.cluster);
+    const int64_t rows = int64_t(t.tok_per_cta) * a.n_kv_heads * D / 128;
+    const int64_t spread = int64_t(n_seqs) * a.n_tokens * a.n_kv_heads * D / 128 / sms;
+    // (the other path's logits kernel for raw keys of head_dim 256 takes ~3 times as long)
+    if (f.total > kMaxDynSmem || rows > kFusedRows + spread * (D == 256 && !CACHED ? 3 : 1)) return cudaSuccess;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kFusedThreads, t.cluster, f.total, stream, attr);
+    *done = true;
+    return cudaLaunchKernelEx(&cfg, kern, t);
+}
+
+cudaError_t launch_select_fused(const SelectArgs& a, bool cached, int n_seqs, int sms, cudaStream_t stream, bool* done) {
+    *done = false;
+    if (a.head_dim == 64) return cached ? try_fused<64, true>(a, n_seqs, sms, stream, done) : try_fused<64, false>(a, n_seqs, sms, stream, done);
+    if (a.head_dim == 128) return cached ? try_fused<128, true>(a, n_seqs, sms, stream, done) : try_fused<128, false>(a, n_seqs, sms, stream, done);
+    if (a.head_dim == 256) return cached ? try_fused<256, true>(a, n_seqs, sms, stream, done) : try_fused<256, false>(a, n_seqs, sms, stream, done);
+    return cudaSuccess;
 }
 }  // namespace prcr

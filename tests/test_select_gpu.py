@@ -277,3 +277,41 @@ def test_select_leftover_halves(name):
         ref = O.ads_relevance(qv[b], int(batch.p_txt[b]), k_raw, coords[b], D, wl.sections, wl.theta)
         assert (np.abs(score[b] - ref) / ref).max() <= 1e-4, b
         assert np.array_equal(idx[b], _topk_by(score[b].astype(np.float64), k))
+
+
+# raw keys through the one-kernel path (a cluster per sequence) and past it:
+# a pass of cos/sin holds 16 tiles of 16 tokens at head_dim 64, 8 at 128 and 4
+# at 256; an odd KV-head count; the last rank of a cluster short or empty
+RAW_SIZES = [  # (B, M, k, H, Hq, D)
+    (1, 33, 5, 1, 8, 128), (2, 769, 32, 3, 3, 128), (1, 2065, 700, 5, 20, 64), (9, 1030, 50, 2, 14, 256), (1, 5000, 64, 2, 8, 256),
+    (150, 200, 9, 1, 2, 64), (30, 2500, 100, 4, 16, 128),
+]
+
+
+@pytest.mark.parametrize("B,M,k,H,Hq,D", RAW_SIZES, ids=[f"B{c[0]}M{c[1]}k{c[2]}H{c[3]}Hq{c[4]}D{c[5]}" for c in RAW_SIZES])
+def test_select_raw_sizes(B, M, k, H, Hq, D):
+    """Relevances within the file's bar, and exactly the top-k of them."""
+    import paper_2606_26631_gb300 as prcr
+    sec = (D // 8, D // 4 - D // 16, D // 2 - D // 8 - (D // 4 - D // 16))
+    g = torch.Generator(device=DEV).manual_seed(200 + M)
+    store_k = torch.randn((B, 1, M, H, D), device=DEV, generator=g).to(torch.bfloat16)
+    coords = torch.randint(0, 60, (B, M, 3), device=DEV, generator=g, dtype=torch.int32)
+    coords[..., 2] = torch.arange(M, device=DEV, dtype=torch.int32) % 40
+    q = (2.0 * torch.randn((B, Hq, D), device=DEV, generator=g)).to(torch.bfloat16)
+    q_pos = torch.arange(B, device=DEV, dtype=torch.int64) * 41 + 700
+    idx = torch.full((B * k,), -7, dtype=torch.int32, device=DEV)
+    sro = torch.full((B + 1,), -7, dtype=torch.int32, device=DEV)
+    rto = torch.full((B + 1,), -7, dtype=torch.int32, device=DEV)
+    score = torch.full((B, M), -1.0, dtype=torch.float32, device=DEV)
+    ws = torch.empty(prcr.select_workspace_size(B, Hq, M), dtype=torch.uint8, device=DEV)
+    cfg = prcr.rope_cfg(1, H, D, sec, 1e6)
+    prcr.select_topk(cfg, prcr.store_desc(store_k, torch.zeros_like(store_k), coords), 0, q, q_pos, k, idx, sro, rto, ws, score)
+    torch.cuda.synchronize()
+    got, sel = score.cpu().numpy(), idx.view(B, k).cpu().numpy()
+    assert np.array_equal(sro.cpu().numpy(), np.arange(B + 1)) and np.array_equal(rto.cpu().numpy(), k * np.arange(B + 1))
+    qv = O.bf16_bits_to_f64(q.view(torch.int16).cpu().numpy())
+    for b in sorted({0, B // 2, B - 1}):
+        ref = O.ads_relevance(qv[b], int(q_pos[b]), store_k[b, 0].view(torch.int16).cpu().numpy(), coords[b].cpu().numpy(), D, sec, 1e6)
+        assert (np.abs(got[b] - ref) / ref).max() <= 1e-4
+    for b in range(B):
+        assert np.array_equal(sel[b], _topk_by(got[b].astype(np.float64), k)), b
