@@ -215,6 +215,32 @@ def test_store_raw_copies_bit_exact():
     assert torch.equal(coords, batch.coords)
 
 
+# a CTA copies 1024 16-byte vectors of a layer; token gaps on either side take
+# the path that finds each row
+@pytest.mark.parametrize("m_count", [1, 127, 128, 129, 400])
+@pytest.mark.parametrize("src_gap,dst_gap", [(0, 0), (8, 0), (0, 24), (8, 24)])
+def test_store_raw_strides(m_count, src_gap, dst_gap):
+    import paper_2606_26631_gb300 as prcr
+    H, D, nL, M = 1, 64, 3, 450
+    g = torch.Generator(device=DEV).manual_seed(m_count)
+    src = [torch.randn((nL, M, H * D + src_gap), generator=g, device=DEV).to(torch.bfloat16) for _ in range(2)]
+    dst = [torch.zeros((1, nL, M, H * D + dst_gap), dtype=torch.bfloat16, device=DEV) for _ in range(2)]
+    rows = lambda t: t[..., :H * D].unflatten(-1, (H, D))  # noqa: E731
+    crd = torch.randint(0, 99, (m_count, 3), generator=g, device=DEV, dtype=torch.int32)
+    coords = torch.zeros((1, M, 3), dtype=torch.int32, device=DEV)
+    cfg = prcr.rope_cfg(nL, H, D, (8, 12, 12))
+    desc = prcr.store_desc(rows(dst[0]), rows(dst[1]), coords)
+    prcr.store_raw(cfg, desc, 0, 0, 20, rows(src[0])[:, 3:3 + m_count], rows(src[1])[:, 3:3 + m_count], crd)
+    torch.cuda.synchronize()
+    for d, s in zip(dst, src):
+        want = torch.zeros_like(d)
+        want[0, :, 20:20 + m_count, :H * D] = s[:, 3:3 + m_count, :H * D]
+        assert torch.equal(d, want)
+    want = torch.zeros_like(coords)
+    want[0, 20:20 + m_count] = crd
+    assert torch.equal(coords, want)
+
+
 # ----------------------------------------------------------------------------
 # device-side error paths: status bits, no out-of-bounds writes, no trap
 # ----------------------------------------------------------------------------
