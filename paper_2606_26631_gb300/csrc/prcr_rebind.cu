@@ -12,26 +12,30 @@
 // formed exactly in fixed-point integers (sincos_turns) and only then handed
 // to float32 sincosf, so a position near 3e4 keeps a ~2e-7 rad angle error
 // instead of the ~2e-3 of a float32 product.
-// Then each thread owns one (token, head, 16-byte vector v) slot of the row:
-// it loads the 8 bf16 of the first half at v and the 8 bf16 of the second
-// half at v + D/2 (the rotate-half partners), for K and V, and walks the G
-// layers. Consecutive threads cover consecutive 16-byte vectors of a row, so
-// every warp-wide load and store is a set of whole 128-byte lines.
+// Each thread owns one (token, head, 16-byte vector v) slot of the row: it
+// loads the 8 bf16 of the first half at v and the 8 bf16 of the second half
+// at v + D/2 (the rotate-half partners), for K and V, and walks the G layers
+// two at a time. Consecutive threads cover consecutive 16-byte vectors of a
+// row, so every warp-wide load and store is a set of whole 128-byte lines.
+//
+// HBM-bound. The first two layers' loads go out before the cos/sin, whose
+// latency they hide: measured 16 sequences x 4 x 640 tokens x 36 layers x 8
+// heads of 128 (11.5 GB) 1689 -> 1684 us (6.83 TB/s), 8 x ~512 x 28 x 4 (0.47
+// GB) 84.0 -> 82.1 us, the smaller ones mostly from their layer groups. One
+// layer ahead of the one stored instead (72 registers): 97 us for the second.
 //
 // The kernel is launched with programmatic dependent launch behind the plan
 // kernel and waits on it (griddepcontrol.wait) before touching the plan.
-#include <cmath>
-
-#include <cuda_bf16.h>
-
 #include "prcr_device.cuh"
+#include "prcr_pdl.cuh"
 
 namespace prcr {
 namespace {
 
 __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ RebindArgs a) {
-    extern __shared__ float smem[];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    extern __shared__ __align__(16) float smem[];
+    pdl_allow();
+    pdl_wait();
     if (*reinterpret_cast<const volatile uint32_t*>(a.status) & PRCR_ST_CSR) return;
 
     const int D = a.head_dim;
@@ -40,6 +44,38 @@ __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ Reb
     float* cos_s = smem;
     float* sin_s = smem + T * P;
     const int64_t tok0 = int64_t(blockIdx.x) * T;
+
+    const int lanes = a.lanes;
+    const int my_t = threadIdx.x / lanes;
+    const int lane = threadIdx.x - my_t * lanes;
+    const int64_t my_tok = tok0 + my_t;
+    const int64_t dst = my_t < T && my_tok < a.total_k ? a.plan_dst[my_tok] : -1;
+    const int vph = D >> 4;  // 16-byte vectors per half row of one head
+    const int h = lane / vph;
+    const int v = lane - h * vph;
+    const int64_t off = int64_t(h) * D + v * 8;
+    const int l0 = blockIdx.y * a.layers_per_cta;
+    const int l1 = min(l0 + a.layers_per_cta, a.n_layers);
+    const int64_t sls = a.store_layer_stride;
+    const int64_t cls = a.cache_layer_stride;
+    const int64_t s_off = (dst < 0 ? 0 : a.plan_src[my_tok]) + int64_t(l0) * sls + off;
+    const uint16_t* sk = a.store_k + s_off;
+    const uint16_t* sv = a.store_v + s_off;
+    // two layers' vectors (K and its rotate-half partner, V likewise), the
+    // first two requested before the cos/sin
+    uint4 x[2][4];
+    auto load = [&](int n) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u < n) {
+                x[u][0] = ld_stream(sk + u * sls);
+                x[u][1] = ld_stream(sk + u * sls + P);
+                x[u][2] = ld_stream(sv + u * sls);
+                x[u][3] = ld_stream(sv + u * sls + P);
+            }
+        }
+    };
+    if (dst >= 0) load(l1 - l0);
 
     for (int q = threadIdx.x; q < T * P; q += blockDim.x) {
         const int t = q / P;
@@ -54,43 +90,35 @@ __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ Reb
         sin_s[q] = s;
     }
     __syncthreads();
-
-    const int lanes = a.lanes;
-    const int t = threadIdx.x / lanes;
-    const int lane = threadIdx.x - t * lanes;
-    const int64_t tok = tok0 + t;
-    if (t >= T || tok >= a.total_k) return;
-    const int64_t dst = a.plan_dst[tok];
     if (dst < 0) return;
-    const int64_t src = a.plan_src[tok];
-
-    const int vph = D >> 4;  // 16-byte vectors per half row of one head
-    const int h = lane / vph;
-    const int v = lane - h * vph;
-    const int half = P;      // elements between rotate-half partners
-    const int64_t off = int64_t(h) * D + v * 8;
 
     float c[8], s[8];
     {
-        const float4* cp = reinterpret_cast<const float4*>(cos_s + t * P + v * 8);
-        const float4* sp = reinterpret_cast<const float4*>(sin_s + t * P + v * 8);
+        const float4* cp = reinterpret_cast<const float4*>(cos_s + my_t * P + v * 8);
+        const float4* sp = reinterpret_cast<const float4*>(sin_s + my_t * P + v * 8);
         const float4 c0 = cp[0], c1 = cp[1], s0 = sp[0], s1 = sp[1];
         c[0] = c0.x; c[1] = c0.y; c[2] = c0.z; c[3] = c0.w;
         c[4] = c1.x; c[5] = c1.y; c[6] = c1.z; c[7] = c1.w;
         s[0] = s0.x; s[1] = s0.y; s[2] = s0.z; s[3] = s0.w;
         s[4] = s1.x; s[5] = s1.y; s[6] = s1.z; s[7] = s1.w;
     }
-
-    const int l0 = blockIdx.y * a.layers_per_cta;
-    const int l1 = min(l0 + a.layers_per_cta, a.n_layers);
-    const int64_t sls = a.store_layer_stride;
-    const int64_t cls = a.cache_layer_stride;
-    const uint16_t* sk = a.store_k + src + int64_t(l0) * sls + off;
-    const uint16_t* sv = a.store_v + src + int64_t(l0) * sls + off;
     uint16_t* ck = a.cache_k + dst + int64_t(l0) * cls + off;
     uint16_t* cv = a.cache_v + dst + int64_t(l0) * cls + off;
-
-    stream_layers(sk, sv, ck, cv, sls, cls, half, l1 - l0, c, s);
+    for (int l = l0; l < l1; l += 2) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (l + u < l1) {
+                uint4 o0, o1;
+                rotate_vec(x[u][0], x[u][1], c, s, o0, o1);
+                st_row(ck + u * cls, o0);
+                st_row(ck + u * cls + P, o1);
+                st_row(cv + u * cls, x[u][2]);
+                st_row(cv + u * cls + P, x[u][3]);
+            }
+        }
+        sk += 2 * sls; sv += 2 * sls; ck += 2 * cls; cv += 2 * cls;
+        load(l1 - l - 2);
+    }
 }
 
 }  // namespace
@@ -101,17 +129,7 @@ cudaError_t rebind_blocks_per_sm(int block, size_t smem, int* out) {
 
 cudaError_t launch_rebind(const RebindArgs& a, dim3 grid, int block, size_t smem,
                           cudaStream_t stream) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rebind_kernel, a);
+    return launch_pdl(rebind_kernel, grid, dim3(unsigned(block)), smem, stream, a);
 }
 
 }  // namespace prcr

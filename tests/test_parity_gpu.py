@@ -241,6 +241,22 @@ def test_store_raw_strides(m_count, src_gap, dst_gap):
     assert torch.equal(coords, want)
 
 
+# layer groups of the two-kernel path: an uneven split of few layers, and the
+# longer groups that a grid of over 32 waves takes
+@pytest.mark.parametrize("n_layers", [5, 83])
+def test_layer_groups(n_layers):
+    import parity_util as pu
+    wl = Workload(name="groups", n_layers=n_layers, n_kv_heads=8, head_dim=128, sections=(24, 20, 20), n_seqs=2,
+                  grids=((1, 40, 50),), selection="random", cache="paged", cur_pos=("uniform", 100, 900), extra=(2, 2, 750, 760))
+    batch = make_batch(wl, device=DEV)
+    rv = _run(batch)
+    assert rv.status_value() == 0
+    pl = pu.oracle_plan(batch)
+    pu.check_plan(rv, pl)
+    pu.check_rows(batch, rv, pl, range(0, batch.total_k, 101), range(n_layers))
+    pu.check_untouched(batch, pl)
+
+
 # ----------------------------------------------------------------------------
 # device-side error paths: status bits, no out-of-bounds writes, no trap
 # ----------------------------------------------------------------------------
