@@ -330,33 +330,19 @@ __device__ __forceinline__ void token_plan(const PlanArgs& a, const RevisitCtx& 
     dst = dest_row(a, r, slot, blk, err);
 }
 
-// Context of revisit r: its token range, sequence (the last b with
-// seq_rev_off[b] <= r), the sequence's first token, text position, cache
-// length and capacity. False (uniform over the CTA) when the offsets around
-// r are inconsistent.
-__device__ __forceinline__ bool revisit_ctx(const PlanArgs& a, int r, RevisitCtx& x) {
-    x.beg = a.rev_tok_off[r];
-    x.end = a.rev_tok_off[r + 1];
-    int lo = 0, hi = a.n_seqs;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a.seq_rev_off[mid] <= r) lo = mid; else hi = mid;
+// The last b in [0, n) with off[b] <= r (off non-decreasing, off[0] <= r), by
+// the whole warp: 32 probes a round, one round up to 32 sequences.
+__device__ __forceinline__ int sequence_of(const int32_t* off, int n, int r) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 1) {
+        const int step = (n + 31) / 32;
+        const bool le = lane * step < n && off[lo + lane * step] <= r;
+        const int k = 31 - __clz(int(__ballot_sync(0xffffffffu, le) | 1u));
+        lo += k * step;
+        n = min(step, n - k * step);
     }
-    x.b = lo;
-    const int r_first = a.seq_rev_off[x.b];
-    bool ok = x.beg >= 0 && x.beg <= x.end && int64_t(x.end) <= a.total_k &&
-              r_first <= r && r < a.seq_rev_off[x.b + 1] && r_first >= 0;
-    x.t0 = ok ? a.rev_tok_off[r_first] : 0;
-    ok = ok && x.t0 >= 0 && x.t0 <= x.beg;
-    if (!ok) return false;
-    x.K = x.end - x.beg;
-    x.p = a.p_txt[x.b];
-    x.clen = a.cache_len_in[x.b];
-    x.center = (a.flags & PRCR_FLAG_DEGENERATE_CENTER) != 0;
-    x.capacity = a.cache_kind == PRCR_CACHE_CONTIGUOUS ? int64_t(a.max_slots)
-                                                       : int64_t(a.bt_stride) * a.block_size;
-    x.inexact = false;
-    return true;
+    return lo;
 }
 
 }  // namespace prcr
