@@ -1,5 +1,6 @@
 // extern "C" entry points of libprcr.so: argument checks, launch planning
 // and the two-kernel revisit path (plan, then rebind + inject).
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <cstdint>
@@ -382,18 +383,24 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     return launch_capture(a, grid, block, smem, stream) == cudaSuccess ? PRCR_OK : PRCR_ECUDA;
 }
 
-// Which decode kernel runs, and the chunks that the sequence axis is split into.
+// The chunks that the sequence axis is split into.
 //
-// head_dim 64 and 128, large batches: sequence lengths differ, so CTAs differ
-// in work: aim at ~8 waves of resident CTAs (3 per SM) so that the last wave
-// is short, with chunks of at least 768 slots (below that a chunk's prologue
-// and its share of the merge outweigh the better balance; measured: 512 -> 768
-// slots took the qwen25vl-7b shape from 5032 to 5394 GB/s; 1184 -> 768 changed
-// qwen3vl-8b by < 1 %), a multiple of 32, at most kDecodeMaxChunk.
-// Small batches (work for fewer than ~6 waves at 768 slots per chunk) take the
-// ring kernel: the KV heads are split over CTAs of kDecodeRingWarps warps and
-// the chunk is sized so that the grid is about one wave of
-// kDecodeRingCtasPerSm CTAs per SM.
+// head_dim 64 and 128, one warp per (chunk, KV head): as many as make one wave
+// of resident warps (a step of few layers and sequences is then over in one go);
+// where those chunks would be longer than 1.25 kChunk slots, chunks of kChunk,
+// many waves of which even out lengths that differ. Measured (us; 1 wave | 2): 1
+// sequence x 36 layers x 8 heads of 933 slots 30.6 | 32.9, 4 x 28 x 4 of up to
+// 2000 (500-slot chunks) 62.8 | 70.2. Large ones at chunks of 384, 512, 768,
+// 1024 and 1536 slots: 8 x 28 x 4 of up to 4096 218, 208, 209, 232, 219; 16 x
+// 36 x 8 912, 895, 896, 886, 900; head_dim 64, 8 x 28 x 3 102, 96, 122, 95, 127.
+template <int D>
+int64_t decode_chunk(int64_t units, int64_t max_len, int sms) {
+    using Sh = DecodeShape<D>;
+    const int64_t want = std::max<int64_t>(1, int64_t(sms) * Sh::kCtas * Sh::kWarps / units);
+    const int64_t c = ((max_len + want - 1) / want + 15) / 16 * 16;
+    return c <= Sh::kChunk * 5 / 4 ? c : Sh::kChunk;
+}
+
 // head_dim 256: one KV head per CTA, about 8 waves of kDecodeWideCtasPerSm
 // CTAs per SM with chunks of at least kWideMinChunk slots; where that is less
 // than two waves, one wave. Chunks are whole rounds of the CTA's warps.
@@ -401,38 +408,22 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
 // waves, 852 us at 16; 4 sequences of up to 2000 slots 162 us at 576 slots,
 // 178 us at 384.
 constexpr int64_t kWideMinChunk = 576;
+int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms) {
+    const int64_t resident = int64_t(sms) * kDecodeWideCtasPerSm, round = 16 * kDecodeWideWarps;
+    const bool few = units * ((max_len + kWideMinChunk - 1) / kWideMinChunk) < 2 * resident;
+    const int64_t want = std::max<int64_t>(1, few ? resident / units : (8 * resident + units - 1) / units);
+    int64_t c = (max_len + want - 1) / want;
+    if (!few && c < kWideMinChunk) c = kWideMinChunk;
+    c = (c + round - 1) / round * round;
+    return std::min<int64_t>(c, kDecodeMaxChunk / round * round);
+}
 
 void decode_split(int64_t base_ctas, int64_t max_len, int sms, int n_kv_heads, int head_dim,
-                  int* splits, int* chunk, int* path) {
-    int64_t c;
-    if (head_dim == 256) {
-        *path = kDecodeWide;
-        const int64_t units = base_ctas * n_kv_heads, resident = int64_t(sms) * kDecodeWideCtasPerSm;
-        const int64_t round = 16 * kDecodeWideWarps;
-        const bool few = units * ((max_len + kWideMinChunk - 1) / kWideMinChunk) < 2 * resident;
-        int64_t want = few ? resident / units : (8 * resident + units - 1) / units;
-        if (want < 1) want = 1;
-        c = (max_len + want - 1) / want;
-        if (!few && c < kWideMinChunk) c = kWideMinChunk;
-        c = (c + round - 1) / round * round;
-        if (c > kDecodeMaxChunk) c = kDecodeMaxChunk / round * round;
-    } else if (base_ctas * ((max_len + 767) / 768) < int64_t(sms) * 6) {
-        *path = kDecodeRing;
-        const int64_t units = base_ctas * ((n_kv_heads + kDecodeRingWarps - 1) / kDecodeRingWarps);
-        int64_t want = int64_t(sms) * kDecodeRingCtasPerSm / units;
-        if (want < 1) want = 1;
-        c = (max_len + want - 1) / want;
-        c = (c + 15) / 16 * 16;
-        if (c > kDecodeMaxChunk) c = kDecodeMaxChunk;
-    } else {
-        *path = kDecodeMma;
-        int64_t want = (int64_t(sms) * 24 + base_ctas - 1) / base_ctas;
-        if (want < 1) want = 1;
-        c = (max_len + want - 1) / want;
-        c = (c + 31) / 32 * 32;
-        if (c < 768) c = 768;
-        if (c > kDecodeMaxChunk) c = kDecodeMaxChunk;
-    }
+                  int* splits, int* chunk) {
+    const int64_t units = base_ctas * n_kv_heads;
+    const int64_t c = head_dim == 64    ? decode_chunk<64>(units, max_len, sms)
+                      : head_dim == 128 ? decode_chunk<128>(units, max_len, sms)
+                                        : decode_wide_chunk(units, max_len, sms);
     *chunk = int(c);
     *splits = int((max_len + c - 1) / c);
     if (*splits < 1) *splits = 1;
@@ -625,9 +616,9 @@ size_t prcr_decode_workspace_size(const prcr_rope_cfg* cfg, int32_t n_seqs, int3
     if (check_cfg(cfg) || n_seqs < 1 || max_len < 1 || !decode_shape_ok(cfg, n_q_heads)) return 0;
     int dev = 0, sms = 1;
     if (cudaGetDevice(&dev) == cudaSuccess) sms = sm_count(dev);
-    int splits = 1, chunk = 32, path = 0;
+    int splits = 1, chunk = 32;
     decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sms, cfg->n_kv_heads, cfg->head_dim,
-                 &splits, &chunk, &path);
+                 &splits, &chunk);
     if (splits == 1) return 0;
     return size_t(n_seqs) * cfg->n_layers * n_q_heads * splits * (cfg->head_dim + 2) * sizeof(float);
 }
@@ -654,7 +645,7 @@ int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache
     if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
     DecodeArgs a = {};
     decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sm_count(dev), cfg->n_kv_heads,
-                 cfg->head_dim, &a.splits, &a.chunk, &a.path);
+                 cfg->head_dim, &a.splits, &a.chunk);
     if (n_seqs > 65535 || cfg->n_layers > 65535) return PRCR_EINVAL;  // grid z and y
     if (a.splits > 1) {
         const size_t need = size_t(n_seqs) * cfg->n_layers * n_q_heads * a.splits *

@@ -256,18 +256,20 @@ struct DecodeArgs {
     int32_t group;
     int32_t splits;
     int32_t chunk;
-    int32_t path;               // kDecodeMma, kDecodeRing or kDecodeWide
     float scale;
     uint64_t turn_freq[kMaxPairs];  // pair i: round(inv_freq_i / (2 pi) * 2^64)
 };
 
+// Shape of the decode kernel at head_dim 64 and 128: warps per CTA, stages of a
+// warp's ring and CTAs per SM (shared memory and registers bound them; copies in
+// flight per SM: 12 warps x 3 tiles x 4.3 KB, 12 x 8.4 KB), and slots of a
+// chunk of a large batch.
+template <int D> struct DecodeShape;
+template <> struct DecodeShape<64> { static constexpr int kWarps = 4, kStages = 4, kCtas = 3, kChunk = 512; };
+template <> struct DecodeShape<128> { static constexpr int kWarps = 4, kStages = 2, kCtas = 3, kChunk = 512; };
 constexpr int kDecodeMaxChunk = 4096;
-// the decode kernels: head_dim 64 and 128 for large and small batches, and 256
-constexpr int kDecodeMma = 0, kDecodeRing = 1, kDecodeWide = 2;
-constexpr int kDecodeWideWarps = 3;   // warps (taking a chunk's tiles in turn) per CTA of the wide kernel
+constexpr int kDecodeWideWarps = 3;   // head_dim 256: warps (taking a chunk's tiles in turn) per CTA
 constexpr int kDecodeWideCtasPerSm = 2;
-constexpr int kDecodeRingWarps = 4;   // KV heads (one per warp) per CTA of the ring kernel
-constexpr int kDecodeRingCtasPerSm = 3;
 
 constexpr int kSelectMaxQHeads = 128;
 

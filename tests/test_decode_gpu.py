@@ -221,17 +221,20 @@ def test_decode_unaligned_query():
     assert torch.equal(ref, got)
 
 
-# slots at the edges of a 16-slot tile, of a round of the CTA's three warps (48)
-# and of a chunk (576), one per sequence of the batch; the group's ends
-@pytest.mark.parametrize("H,Hq,paged,bs", [(1, 8, True, 7), (3, 3, False, 16), (4, 28, True, 16)])
+# slots at the edges of a 16-slot tile, of a round of the head_dim 256 CTA's
+# three warps (48) and of a chunk (512, 576), one per sequence of the batch;
+# head counts that leave a CTA's last warps without a unit; the group's ends
+@pytest.mark.parametrize("H,Hq,D,paged,bs", [(1, 8, 256, True, 7), (3, 3, 256, False, 16), (4, 28, 256, True, 16),
+                                             (1, 8, 128, True, 7), (5, 5, 128, False, 16), (3, 21, 64, True, 16)])
 @pytest.mark.parametrize("n_layers", [1, 40])
-def test_decode_head_dim_256_edges(H, Hq, paged, bs, n_layers):
+def test_decode_edges(H, Hq, D, paged, bs, n_layers):
     """head_dim 256: every product has 24 significant bits and is summed in
     float32, so a logit (sum of ~10 in magnitude over 48 MMAs) is off by about
-    sqrt(48) 2^-24 10 = 4e-6 and the output by no more than twice that."""
+    sqrt(48) 2^-24 10 = 4e-6 and the output by no more than twice that. Below,
+    the file's bar: 16 significant bits per operand, 10 * 2^-17 = 8e-5."""
     import paper_2606_26631_gb300 as prcr
-    D, sec = 256, (40, 44, 44)
-    lens = [1, 15, 16, 17, 47, 48, 49, 575, 576, 577, 593, 0, 1153]
+    sec = (D // 8, D // 4, D // 8)
+    lens = [1, 15, 16, 17, 47, 48, 49, 511, 512, 513, 575, 576, 577, 593, 0, 1153]
     B, max_len = len(lens), 1153
     inp = make_decode_inputs(B, n_layers, H, Hq, D, max_len, paged, device=DEV, seed=31, block_size=bs)
     if paged:  # every sequence's table maps all of its slots
@@ -257,7 +260,7 @@ def test_decode_head_dim_256_edges(H, Hq, paged, bs, n_layers):
         else:
             K, V = (_f64(inp[x][b, l, :n]) for x in ("cache_k", "cache_v"))
         ref = O.decode_attention(qv[b, l], int(inp["q_pos"][b]), K, V, D, sec, 1e6)
-        assert np.abs(got[b, l] - ref).max() / np.abs(V).max() <= 8e-6, (b, n)
+        assert np.abs(got[b, l] - ref).max() / np.abs(V).max() <= (8e-6 if D == 256 else 1e-4), (b, n)
 
 
 def test_inject_then_decode():
