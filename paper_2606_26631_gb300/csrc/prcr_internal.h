@@ -344,6 +344,8 @@ cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaS
 // the whole selection in one kernel, where that is the faster path (else
 // *done = false and nothing is launched)
 cudaError_t launch_select_fused(const SelectArgs& a, bool cached, int n_seqs, int sms, cudaStream_t stream, bool* done);
+// the logits of the cached-key selection
+cudaError_t launch_select_cached_logits(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
 // the steps after the logits: normalisers, relevances, top-k
 cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream);
 

@@ -15,10 +15,10 @@
 // turned by theta_i (c_axis(i) - p) and dotted with the raw query, and the
 // 1/sqrt(D) scale is applied to the dot product. The raw bf16 query is then
 // exact in any operand format, and nothing is computed per query.
-// A logits kernel here (from the raw keys, rotated on the fly, or from the
-// position-bound cache) writes every (token, query head) logit to the
-// workspace; prcr_select_cluster.cu does the rest: softmax normalisers,
-// relevances, top-k.
+// The logits kernels here (from the raw keys, rotated on the fly) write every
+// (token, query head) logit to the workspace; prcr_select_cluster.cu does the
+// rest: softmax normalisers, relevances, top-k; and all of it for small calls
+// and for the keys of the position-bound cache.
 #include <cmath>
 
 #include "prcr_pdl.cuh"
@@ -475,264 +475,6 @@ __global__ void __launch_bounds__(NW * 32, 2) ads_logits_mma_kernel(const __grid
     }
 }
 
-// Logits of the selection over the position-bound cache (head_dim 64 or
-// 128). The cache already holds each visual token's key rotated at its own
-// coordinates, so only the query is turned, once, at (p, p, p); the step is
-// then a plain product with the cached rows and runs at memory speed. A
-// warp's work item is (sequence b, KV head kh, tile of 16 tokens); items run
-// (b, kh) major with tiles fastest and a warp takes a contiguous run of them,
-// so it rotates its group's queries once per (b, kh). S^T (16 rows = the
-// item's tokens; 8 columns = the group's query heads, columns >= g zero) =
-// K Q^T over D/16 k-steps of mma.sync m16n8k16: the bf16 keys are exact
-// operands and the float32 query (pre-scaled by 1/sqrt(D)) enters as a bf16
-// head and a bf16 remainder (two MMAs per k-step). The key dimensions are
-// permuted per lane group so that a lane loads its two tokens' 64 contiguous
-// bytes each straight into A fragments. The next item's rows are loaded
-// during this item's MMAs (each 16-byte run as soon as the register it goes
-// into is used), the rows of the one after that requested into L2. An item
-// writes its 16 logits per head; a token without a readable row gets logit -inf.
-template <int D>
-__global__ void __launch_bounds__(256, D > 128 ? 1 : 2)
-    ads_logits_cache_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    constexpr int KS = D / 16, LV = D / 32, P = D / 2;
-    extern __shared__ __align__(16) float sm[];
-    const int Hq = a.n_q_heads, H = a.n_kv_heads, g = Hq / H, M = a.n_tokens, NT = a.n_tiles;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gid = lane >> 2, t = lane & 3;
-    float* qw = sm + warp * g * D;  // this warp's rotated query rows
-    const int64_t n_items = int64_t(a.n_seqs) * H * NT;
-    const int64_t n_warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    const int64_t gw = int64_t(blockIdx.x) * (blockDim.x >> 5) + warp;
-    const int64_t i_beg = n_items * gw / n_warps, i_end = n_items * (gw + 1) / n_warps;
-    uint32_t err = 0;
-    pdl_wait();
-
-    // a work item as (sequence, KV head, tile); a warp's items are consecutive,
-    // so they are advanced in place rather than divided out of the index
-    struct Item {
-        int b, kh, j;
-    };
-    auto advance = [&](Item& x) {
-        if (++x.j == NT) {
-            x.j = 0;
-            if (++x.kh == H) {
-                x.kh = 0;
-                ++x.b;
-            }
-        }
-    };
-    // element offset, without the KV head's D elements, of the key row of
-    // token 16 j + (lane & 15) of sequence b, or -1 (past the end, or no
-    // readable row). Computed once per item, when its rows are requested.
-    const int64_t layer_off = int64_t(a.layer) * a.cache_layer_stride;
-    // The row lookup in two halves, one item apart: start() forms the slot of
-    // this lane's token and issues its block-table load (paged caches), whose
-    // value finish() uses an item later, when the lookup's dependent loads
-    // have long returned. The sequence's first image slot is kept per
-    // sequence (items run sequence-major).
-    struct RowReq {
-        int64_t slot;  // -1: no row
-        int32_t blk;
-    };
-    int s0_b = -1;
-    int32_t s0_v = 0;
-    auto row_start = [&](const Item& x, RowReq& q) {
-        q.slot = -1;
-        q.blk = 0;
-        const int m = 16 * x.j + (lane & 15);
-        if (m >= M) return;
-        if (x.b != s0_b) {
-            s0_b = x.b;
-            s0_v = a.img_slot0[x.b];
-        }
-        const int64_t slot = int64_t(s0_v) + m;
-        if (slot < 0 || slot >= a.cache_capacity) {
-            err |= PRCR_ST_CAPACITY;
-            return;
-        }
-        q.slot = slot;
-        if (a.cache_kind != PRCR_CACHE_CONTIGUOUS) {
-            // block index by a 32-bit division when the slot fits in 31 bits
-            // (a 64-bit division costs several times as many instructions as
-            // the rest of a row lookup)
-            const int64_t lb = slot <= INT32_MAX ? int64_t(uint32_t(slot) / uint32_t(a.block_size))
-                                                 : slot / a.block_size;
-            q.blk = a.block_table[int64_t(x.b) * a.bt_stride + lb];
-        }
-    };
-    auto row_finish = [&](const Item& x, const RowReq& q) -> int64_t {
-        if (q.slot < 0) return -1;
-        int64_t row;
-        if (a.cache_kind == PRCR_CACHE_CONTIGUOUS) {
-            row = int64_t(x.b) * a.cache_seq_stride + q.slot * a.cache_slot_stride;
-        } else {
-            if (q.blk < 0 || q.blk >= a.n_blocks) {
-                err |= PRCR_ST_NO_BLOCK;
-                return -1;
-            }
-            const int64_t off = q.slot <= INT32_MAX ? int64_t(uint32_t(q.slot) % uint32_t(a.block_size))
-                                                    : q.slot % a.block_size;
-            row = int64_t(q.blk) * a.cache_block_stride + off * a.cache_slot_stride;
-        }
-        return row + layer_off;
-    };
-    auto row_of = [&](const Item& x) -> int64_t {
-        RowReq q;
-        row_start(x, q);
-        return row_finish(x, q);
-    };
-    uint4 kn[2][LV];
-    uint32_t mask_n = 0u;
-    // loads an item's 16 key rows (row: this lane's token, from row_of). A
-    // token without a row reads the cache's first row instead: its logit is
-    // set to -inf whatever the row holds (tokens are separate MMA rows).
-    // this lane's two token rows (tokens gid and gid + 8) of an item, and the
-    // item's row mask
-    auto rows_of = [&](int64_t row, int kh, const uint16_t* (&kp)[2]) -> uint32_t {
-        const uint32_t m = __ballot_sync(0xffffffffu, row >= 0) & 0xffffu;
-        const int64_t r0 = (row >= 0 ? row : 0) + int64_t(kh) * D;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-            kp[nt] = a.cache_k + __shfl_sync(0xffffffffu, r0, nt * 8 + gid) + t * (D / 4);
-        return m;
-    };
-    auto fetch = [&](int64_t row, int kh) {
-        const uint16_t* kp[2];
-        mask_n = rows_of(row, kh, kp);
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-#pragma unroll
-            for (int u = 0; u < LV; ++u) kn[nt][u] = ld_stream(kp[nt] + 8 * u);
-        }
-    };
-    // the rows of the item after next are requested into L2 (lanes 0..15,
-    // one token row each), so that its fetch finds them there
-    auto request = [&](int64_t row, int kh) {
-        if (lane < 16 && row >= 0) {
-            const char* p = reinterpret_cast<const char*>(a.cache_k + row + int64_t(kh) * D);
-#pragma unroll
-            for (int o = 0; o < D * 2; o += 128) prefetch_l2(p + o);
-        }
-    };
-
-    uint32_t qh[KS][2], ql[KS][2];
-    float* lg_base[2] = {nullptr, nullptr};
-    int cur_b = -1, cur_kh = -1;
-    bool q_ok = true;  // the sequence's query position is within the angle range
-    Item cur, nxt, pf;
-    {
-        const int64_t bk = i_beg / NT;
-        cur.j = int(i_beg - bk * NT);
-        cur.b = int(bk / H);
-        cur.kh = int(bk - int64_t(cur.b) * H);
-    }
-    nxt = cur;
-    advance(nxt);
-    pf = nxt;
-    advance(pf);
-    int64_t row_nxt = -1, row_pf = -1;
-    RowReq req_pf = {-1, 0};  // the started lookup of pf
-    if (i_beg < i_end) fetch(row_of(cur), cur.kh);
-    if (i_beg + 1 < i_end) {
-        row_nxt = row_of(nxt);
-        request(row_nxt, nxt.kh);
-    }
-    if (i_beg + 2 < i_end) row_start(pf, req_pf);
-    for (int64_t left = i_end - i_beg; left > 0; --left) {
-        const int b = cur.b, kh = cur.kh, j = cur.j;
-        if (b != cur_b || kh != cur_kh) {
-            // the group's queries turned at (p, p, p), pre-scaled, as A fragments
-            // a query position beyond the fixed-point angle reduction is
-            // reported and the sequence's logits are all -inf (relevance 0)
-            const int64_t p = a.q_pos[b];
-            q_ok = p > -2147483648LL && p < 2147483648LL;
-            if (!q_ok) err |= PRCR_ST_POS_RANGE;
-            const uint16_t* qg = a.q + (int64_t(b) * Hq + kh * g) * D;
-            for (int i = lane; i < P; i += 32) {
-                float sn, cs;
-                sincos_turns(double(p), a.turn_freq[i], &sn, &cs);
-                for (int h = 0; h < g; ++h) {
-                    const float x = __uint_as_float(uint32_t(qg[h * D + i]) << 16);
-                    const float y = __uint_as_float(uint32_t(qg[h * D + i + P]) << 16);
-                    qw[h * D + i] = fmaf(x, cs, -y * sn) * a.scale;
-                    qw[h * D + i + P] = fmaf(y, cs, x * sn) * a.scale;
-                }
-            }
-            __syncwarp();
-            const bool hv = gid < g;
-            const float* qr = qw + (hv ? gid : 0) * D + t * (D / 4);
-#pragma unroll
-            for (int k = 0; k < KS; ++k) {
-                const float x0 = hv ? qr[4 * k] : 0.0f, x1 = hv ? qr[4 * k + 1] : 0.0f;
-                const float x2 = hv ? qr[4 * k + 2] : 0.0f, x3 = hv ? qr[4 * k + 3] : 0.0f;
-                split_bf16x2(x0, x1, qh[k][0], ql[k][0]);
-                split_bf16x2(x2, x3, qh[k][1], ql[k][1]);
-            }
-            __syncwarp();  // qw is rewritten for the next (b, kh)
-            cur_b = b;
-            cur_kh = kh;
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {  // rows of this lane's heads 2t, 2t + 1
-                const int64_t r = int64_t(b) * Hq + kh * g + min(2 * t + hh, g - 1);
-                lg_base[hh] = a.logits + r * M;
-            }
-        }
-        // S^T (16 tokens x 8 columns = the group's query heads, columns >= g
-        // zero) = K Q^T: rows gid (kn[0]) and gid + 8 (kn[1]) are this lane's
-        // tokens, and the query fragments serve as the B operand unchanged
-        const uint32_t mask = q_ok ? mask_n : 0u;
-        // the next item's rows, each 16-byte run requested as soon as this
-        // item's MMAs have used the registers it goes into
-        const uint16_t* kp[2] = {a.cache_k, a.cache_k};
-        if (left > 1) mask_n = rows_of(row_nxt, nxt.kh, kp);
-        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            const uint4& w0 = kn[0][k >> 1];
-            const uint4& w1 = kn[1][k >> 1];
-            const uint32_t a0 = (k & 1) ? w0.z : w0.x, a2 = (k & 1) ? w0.w : w0.y;
-            const uint32_t a1 = (k & 1) ? w1.z : w1.x, a3 = (k & 1) ? w1.w : w1.y;
-            mma_16816(c, a0, a1, a2, a3, qh[k][0], qh[k][1]);
-            mma_16816(c, a0, a1, a2, a3, ql[k][0], ql[k][1]);
-            if ((k & 1) && left > 1) {
-                kn[0][k >> 1] = ld_stream(kp[0] + 8 * (k >> 1));
-                kn[1][k >> 1] = ld_stream(kp[1] + 8 * (k >> 1));
-            }
-        }
-        Item pf2 = pf;  // the item after pf: its lookup starts now
-        advance(pf2);
-        if (left > 2) {
-            row_pf = row_finish(pf, req_pf);
-            request(row_pf, pf.kh);
-        }
-        if (left > 3) row_start(pf2, req_pf);
-
-        // token gid: heads 2t, 2t + 1 in c[0], c[1]; token gid + 8 in c[2], c[3]
-        const bool ok0 = (mask >> gid) & 1u, ok1 = (mask >> (gid + 8)) & 1u;
-        float v[4] = {ok0 ? c[0] : -INFINITY, ok0 ? c[1] : -INFINITY, ok1 ? c[2] : -INFINITY,
-                      ok1 ? c[3] : -INFINITY};
-        const int m0 = 16 * j;
-        const bool full = m0 + 16 <= M;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            if (2 * t + hh >= g) continue;
-            float* lg = lg_base[hh] + m0;
-            if (full) {
-                lg[gid] = v[hh];
-                lg[gid + 8] = v[2 + hh];
-            } else {
-                if (m0 + gid < M) lg[gid] = v[hh];
-                if (m0 + gid + 8 < M) lg[gid + 8] = v[2 + hh];
-            }
-        }
-        cur = nxt;
-        nxt = pf;
-        row_nxt = row_pf;
-        pf = pf2;
-    }
-    if (err) atomicOr(a.status, err);
-}
-
 }  // namespace
 
 size_t select_logits_smem(const SelectArgs& a) {
@@ -821,19 +563,7 @@ cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaS
     bool done = false;
     cudaError_t e = launch_select_fused(a, true, n_seqs, sms, stream, &done);
     if (e != cudaSuccess || done) return e;
-    const int g = a.n_q_heads / a.n_kv_heads;
-    const size_t smem = size_t(8) * g * a.head_dim * sizeof(float);  // 8 warps
-    auto k = a.head_dim == 64 ? ads_logits_cache_kernel<64>
-             : a.head_dim == 128 ? ads_logits_cache_kernel<128>
-                                 : ads_logits_cache_kernel<256>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t items = int64_t(n_seqs) * a.n_kv_heads * a.n_tiles;
-    const int64_t ctas = (items + 7) / 8;
-    const int64_t resident = int64_t(sms) * (per_sm > 0 ? per_sm : 1);
-    e = launch_pdl(k, dim3(unsigned(ctas < resident ? ctas : resident)), dim3(256), smem, stream, a);
+    e = launch_select_cached_logits(a, n_seqs, sms, stream);
     if (e != cudaSuccess) return e;
     return launch_select_tail(a, n_seqs, stream);
 }

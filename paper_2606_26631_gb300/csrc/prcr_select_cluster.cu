@@ -1,7 +1,7 @@
 // The selection on clusters of CTAs, one cluster per sequence: in one kernel
 // from the keys to the indices where the logits fit in the cluster's shared
 // memory (select_fused_kernel), else everything after a logits kernel
-// (select_tail_kernel).
+// (select_tail_kernel), which for cached keys is select_logits_kernel here.
 //
 // Rank r of a cluster of C CTAs takes the tokens r * T .. r * T + T - 1 of its
 // sequence (T = tok_per_cta). Two exchanges through distributed shared memory
@@ -20,6 +20,7 @@
 // the smallest to the largest relevance, counted by shared-memory atomics
 // (about M / 2048 keys meet in a bucket), then the few keys of its bucket
 // ranked by one warp; or again over that bucket while it holds many.
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <map>
@@ -78,8 +79,8 @@ struct SelectShared {
     uint32_t list[32], n_list;
 };
 
-// Exchange 1: the heads' normalisers from every CTA's statistics. Also
-// sets up the search's shared state.
+// Exchange 1: the heads' normalisers from every CTA's statistics. Also sets up
+// the search's shared state.
 template <int NT>
 __device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, SelectShared& sh) {
     cluster_arrive();
@@ -287,32 +288,11 @@ __device__ __forceinline__ void stats16(const float (&x)[16], float& mx, float& 
     mx = cm;
 }
 
-// Everything after a logits kernel: logits in global memory (mostly L2), read
-// once for the statistics and once for the relevances. L2 bounds the large
-// ones: 32 sequences x 16,384 tokens x 32 heads (67 MB) on 128 CTAs take ~20
-// us: statistics 13k cycles, relevances 11k, the two exchanges 7k, search 6k,
-// output 3k. Measured against the three kernels it replaced (normaliser,
-// relevance, a top-k of one CTA per sequence counting two bits a round), whole
-// selections: that shape 262 -> 244 us, 16 x 8192 cached 72.8 -> 66.9 us, one
-// sequence of 16,384 43.9 -> 35.4 us; one of 64 tokens, where the chain of
-// exchanges shows, 10.5 -> 14 us of GPU time but 21 -> 16 us with its launches.
-constexpr int kTailThreads = 1024;
-constexpr int kTailMinTokens = 64;  // per CTA
-
-__global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
-    constexpr int NT = kTailThreads, NW = NT / 32;
-    __shared__ SelectShared sh;
-    extern __shared__ __align__(16) uint32_t keys[];  // [cluster * tok_per_cta] relevances
-    const int C = a.cluster, b = int(blockIdx.x) / C, rank = int(cluster_rank());
-    const int M = a.n_tokens, Hq = a.n_q_heads;
-    const int m_beg = rank * a.tok_per_cta, nt = max(0, min(a.tok_per_cta, M - m_beg));
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float* rel = reinterpret_cast<float*>(keys + m_beg);
-    const float* lg = a.logits + int64_t(b) * Hq * M + m_beg;
-    const bool vec = (M & 3) == 0;  // rows of logits 16-byte aligned (m_beg is a multiple of 16)
-    pdl_wait();
-
+// The statistics of a CTA's nt tokens, a warp per query head, from logits in
+// global memory.
+template <int NW>
+__device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int nt, bool vec, SelectShared& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int hq = warp; hq < Hq; hq += NW) {
         const float* row = lg + int64_t(hq) * M;
         float mx = -INFINITY, z = 0.0f;
@@ -345,8 +325,36 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
         }
         if (lane == 0) sh.stat[hq] = make_float2(mx, z);
     }
-    merge_stats<NT>(a, C, sh);
+}
 
+// Everything after a logits kernel: logits in global memory (mostly L2), read
+// once for the statistics and once for the relevances. L2 bounds the large
+// ones: 32 sequences x 16,384 tokens x 32 heads (67 MB) on 128 CTAs take ~20
+// us: statistics 13k cycles, relevances 11k, the two exchanges 7k, search 6k,
+// output 3k. Measured against the three kernels it replaced (normaliser,
+// relevance, a top-k of one CTA per sequence counting two bits a round), whole
+// selections: that shape 262 -> 244 us, 16 x 8192 cached 72.8 -> 66.9 us, one
+// sequence of 16,384 43.9 -> 35.4 us; one of 64 tokens, where the chain of
+// exchanges shows, 10.5 -> 14 us of GPU time but 21 -> 16 us with its launches.
+constexpr int kTailThreads = 1024;
+constexpr int kTailMinTokens = 64;  // per CTA
+
+__global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __grid_constant__ SelectArgs a) {
+    pdl_allow();
+    constexpr int NT = kTailThreads, NW = NT / 32;
+    __shared__ SelectShared sh;
+    extern __shared__ __align__(16) uint32_t keys[];  // [cluster * tok_per_cta] relevances
+    const int C = a.cluster, b = int(blockIdx.x) / C, rank = int(cluster_rank());
+    const int M = a.n_tokens, Hq = a.n_q_heads;
+    const int m_beg = rank * a.tok_per_cta, nt = max(0, min(a.tok_per_cta, M - m_beg));
+    const int tid = threadIdx.x;
+    float* rel = reinterpret_cast<float*>(keys + m_beg);
+    const float* lg = a.logits + int64_t(b) * Hq * M + m_beg;
+    const bool vec = (M & 3) == 0;  // rows of logits 16-byte aligned (m_beg is a multiple of 16)
+    pdl_wait();
+
+    tail_stats<NW>(lg, M, Hq, nt, vec, sh);
+    merge_stats<NT>(a, C, sh);
     uint32_t lo = 0xffffffffu, hi = 0u;
     auto seen = [&](float r) {
         lo = min(lo, __float_as_uint(r));
@@ -400,28 +408,13 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
     select_topk<NT>(a, b, C, m_beg, nt, keys, lo, hi, sh);
 }
 
-// The whole selection in one kernel. The CTA's logits stay in shared memory;
-// their computation is that of ads_logits_mma_kernel (raw keys turned by the
-// offsets of their coordinates, CACHED = false) or of ads_logits_cache_kernel
-// (position-bound rows against the turned query, CACHED = true), as work items
-// of (16 tokens, KV head) that the CTA's warps take in turn. The queries'
-// fragments, and the raw keys' cos/sin (a pass of 1024 / D tiles at a time),
-// are computed once per CTA; an item's rows are loaded during the item before.
-// Small calls are a chain of latencies, which one kernel shortens by three
-// launches: 768 tokens x 8 KV heads in a cluster of 16, ~20k cycles: queries
-// and first rows 2.7k, cos/sin and MMAs 5.5k, statistics and their exchange
-// 4.8k, relevances and theirs 5k, search and output 2.7k. Measured with its
-// launches 20.9 -> 12.5 us (four kernels before), 8 sequences 20.6 -> 13.6 us,
-// 4 of 1000 tokens at head_dim 256 29.6 -> 13.9 us (CUDA cores before).
-constexpr int kFusedThreads = 512;
-
-// Shared memory of the fused kernel, in the order of its sections.
+// Shared memory of cta_logits and the fused kernel, in the order of its sections.
 struct FusedLayout {
     int pitch;  // floats per head's row of logits: 4 mod 32, free of bank conflicts for the MMA's accumulators
     size_t trig, tok, query, logits, keys, total;
 };
 
-__host__ __device__ inline FusedLayout fused_layout(int D, bool cached, int H, int Hq, int T, int C) {
+__host__ __device__ inline FusedLayout fused_layout(int D, bool cached, int H, int Hq, int T, int C, bool logits = true) {
     FusedLayout f;
     f.pitch = (T + 31) / 32 * 32 + 4;
     f.trig = size_t(H) * D * 32;  // after the queries' fragments [H][D / 16][32] uint4
@@ -429,51 +422,60 @@ __host__ __device__ inline FusedLayout fused_layout(int D, bool cached, int H, i
     f.tok = f.trig + (cached ? 0 : size_t(tiles) * D * 64);          // [tiles][D / 8][32] float4
     f.query = f.tok + (size_t(T) * (cached ? 8 : 12) + 15) / 16 * 16;  // rows (int64) or coordinates (3 int32)
     f.logits = f.query + (cached ? size_t(Hq) * (D + 8) * 2 : 0);      // the raw queries
-    f.keys = f.logits + size_t(Hq) * f.pitch * 4;
+    f.keys = f.logits + (logits ? size_t(Hq) * f.pitch * 4 : 0);
     f.total = f.keys + size_t(C) * T * 4;
     return f;
 }
 
-template <int D, bool CACHED>
-__global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __grid_constant__ SelectArgs a) {
-    constexpr int NT = kFusedThreads, NW = NT / 32, P = D / 2;
+// What depends on the rotary configuration alone, in static shared memory.
+template <int D, bool CACHED, int NT>
+struct PairTables {
+    uint64_t tf[D / 2];                                     // turn rates
+    alignas(16) float2 cs[CACHED ? D / 2 : 1];              // (cos, sin) of the query's turn
+    uint8_t ax[D / 2];                                      // axes
+    __device__ void set(const SelectArgs& a) {
+        for (int i = threadIdx.x; i < D / 2; i += NT) {
+            tf[i] = a.turn_freq[i];
+            ax[i] = uint8_t(pair_axis(i, a.layout, a.sec_t, a.sec_h, a.sec_w));
+        }
+    }
+};
+
+// Logits of tokens m_beg .. m_beg + nt - 1 of sequence b for the query heads of
+// KV heads kh0 .. kh0 + H - 1: query head kh0 g + h, token m_beg + t at
+// lg[h * lg_pitch + t]. Raw keys are turned by the offsets of their
+// coordinates as in ads_logits_mma_kernel (CACHED = false); position-bound rows
+// meet the query turned at (p, p, p), a bf16 head and remainder (CACHED = true;
+// the bf16 keys are exact operands, S^T = K Q^T by m16n8k16). A work item is
+// (16 tokens, KV head), and the CTA's warps take them in turn, heads fastest;
+// an item's rows are loaded during the item before. The queries' fragments,
+// the cache rows of the tokens, and the raw keys' cos/sin (a pass of 1024 / D
+// tiles at a time) are found once per CTA.
+template <int D, bool CACHED, int NT>
+__device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayout& f, int b, int kh0, int H, int m_beg,
+                                           int nt, unsigned char* smem_raw, PairTables<D, CACHED, NT>& pt, float* lg,
+                                           int lg_pitch, uint32_t& err) {
+    constexpr int NW = NT / 32, P = D / 2;
     constexpr int KQ = D / 16;                  // 16-byte fragment entries per lane of a KV head's queries
     constexpr int NR = CACHED ? D / 32 : D / 64;  // groups of 16-byte loads of an item, refilled as they are used
     constexpr int RL = CACHED ? 2 : 4;            // loads per group
     constexpr int TP = 1024 / D;                // tiles of a pass (raw keys)
     constexpr int QP = D + 8;                   // bf16 per staged query row
-    __shared__ SelectShared sh;
-    __shared__ uint64_t tf_s[P];
-    __shared__ __align__(16) float2 cs_s[CACHED ? P : 1];  // (cos, sin) of the query's turn
-    __shared__ uint8_t ax_s[P];
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_allow();
-    const int C = a.cluster, b = int(blockIdx.x) / C, rank = int(cluster_rank()), T = a.tok_per_cta;
-    const int M = a.n_tokens, Hq = a.n_q_heads, H = a.n_kv_heads, g = Hq / H;
-    const int m_beg = rank * T, nt = max(0, min(T, M - m_beg)), n_tiles = (nt + 15) / 16;
+    const int Hq = a.n_q_heads, g = Hq / a.n_kv_heads, n_tiles = (nt + 15) / 16;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tq = lane & 3;
-    const FusedLayout f = fused_layout(D, CACHED, H, Hq, T, C);
     uint4* qf_s = reinterpret_cast<uint4*>(smem_raw);
     float4* tr_s = reinterpret_cast<float4*>(smem_raw + f.trig);
     int* crd_s = reinterpret_cast<int*>(smem_raw + f.tok);
     int64_t* row_s = reinterpret_cast<int64_t*>(smem_raw + f.tok);
     uint32_t* q_s = reinterpret_cast<uint32_t*>(smem_raw + f.query);
-    float* lg_s = reinterpret_cast<float*>(smem_raw + f.logits);
-    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + f.keys);
-    for (int i = tid; i < P; i += NT) {
-        tf_s[i] = a.turn_freq[i];
-        ax_s[i] = uint8_t(pair_axis(i, a.layout, a.sec_t, a.sec_h, a.sec_w));
-    }
-    uint32_t err = 0;
-    pdl_wait();
     const int64_t p = a.q_pos[b];
-    const uint16_t* qs = a.q + int64_t(b) * Hq * D;
+    const uint16_t* qs = a.q + (int64_t(b) * Hq + kh0 * g) * D;
 
     // the items of this warp: warp, warp + NW, ... of (tile, KV head), heads fastest
     uint4 k[NR][RL];
-    const uint16_t* kb = CACHED ? a.cache_k + int64_t(a.layer) * a.cache_layer_stride + tq * (D / 4)
+    const uint16_t* kb = CACHED ? a.cache_k + int64_t(a.layer) * a.cache_layer_stride + kh0 * D + 8 * tq
                                 : a.store_k + int64_t(b) * a.store_seq_stride + int64_t(m_beg) * a.store_token_stride +
-                                      int64_t(a.layer) * a.store_layer_stride + 8 * tq;
+                                      int64_t(a.layer) * a.store_layer_stride + kh0 * D + 8 * tq;
     // this lane's two token rows (gid and gid + 8 of the tile) at KV head kh; a
     // token past the end reads the last one, one without a row the cache's
     // first row (their logits are not stored, or are -inf)
@@ -490,8 +492,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     };
     auto fetch = [&](uint4 (&x)[RL], const uint16_t* ra, const uint16_t* rb, int u) {
         if constexpr (CACHED) {
-            x[0] = ld_stream(ra + 8 * u);
-            x[1] = ld_stream(rb + 8 * u);
+            x[0] = ld_stream(ra + 32 * u);
+            x[1] = ld_stream(rb + 32 * u);
         } else {
             x[0] = ld_stream(ra + 32 * u);
             x[1] = ld_stream(ra + 32 * u + P);
@@ -527,7 +529,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
         // the query rows into shared memory, the cache rows of the CTA's tokens
         // (-1: none), and the query's turn
 #pragma unroll 4
-        for (int i = tid; i < Hq * P; i += NT) q_s[(i / P) * (QP / 2) + i % P] = __ldg(q_src + i);
+        for (int i = tid; i < H * g * P; i += NT) q_s[(i / P) * (QP / 2) + i % P] = __ldg(q_src + i);
         const int64_t s0 = a.img_slot0[b];
         for (int t = tid; t < nt; t += NT) {
             const int64_t slot = s0 + m_beg + t;
@@ -551,18 +553,20 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
         if (!q_ok) err |= PRCR_ST_POS_RANGE;
         for (int i = tid; i < P; i += NT) {
             float sn, cs;
-            sincos_fixed(q_ok ? static_cast<long long>(p) * (1ll << 32) : 0ll, tf_s[i], &sn, &cs);
-            cs_s[i] = make_float2(cs, sn);
+            sincos_fixed(q_ok ? static_cast<long long>(p) * (1ll << 32) : 0ll, pt.tf[i], &sn, &cs);
+            pt.cs[i] = make_float2(cs, sn);
         }
         __syncthreads();
         first();
-        // dimensions t D/4 + 4j .. + 3 (those that the lane's key loads hold),
-        // turned at (p, p, p) and scaled, a bf16 head and remainder each
+        // four dimensions of 16-byte chunk t + 4 (j / 2) (the chunks that the
+        // lane loads of its keys: the four lanes of a token cover 64 contiguous
+        // bytes per load), turned at (p, p, p) and scaled, a bf16 head and
+        // remainder each
         each_fragment([&](int hq, int j, int t) {
             const uint32_t* q0 = q_s + hq * (QP / 2);
-            const int d = t * (D / 4) + 4 * j, dp = d < P ? d + P : d - P, i = d < P ? d : dp;
+            const int d = 8 * (t + 4 * (j >> 1)) + 4 * (j & 1), dp = d < P ? d + P : d - P, i = d < P ? d : dp;
             const uint2 x = *reinterpret_cast<const uint2*>(q0 + d / 2), y = *reinterpret_cast<const uint2*>(q0 + dp / 2);
-            const float4 ca = *reinterpret_cast<const float4*>(cs_s + i), cb = *reinterpret_cast<const float4*>(cs_s + i + 2);
+            const float4 ca = *reinterpret_cast<const float4*>(pt.cs + i), cb = *reinterpret_cast<const float4*>(pt.cs + i + 2);
             const float sg = d < P ? -1.0f : 1.0f;
             uint4 o;
             split_bf16x2(fmaf(lo_f32(x.x), ca.x, sg * lo_f32(y.x) * ca.y) * a.scale,
@@ -594,11 +598,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
             if (t0) __syncthreads();  // the previous pass has been read
             for (int e = tid; e < (t1 - t0) * (D / 8) * 32; e += NT) {
                 const int s = (e / 32) % (D / 8), tile = t0 + e / (32 * (D / 8));
-                const int i = 32 * (s / 8) + 8 * tq + s % 8, ax = ax_s[i];
+                const int i = 32 * (s / 8) + 8 * tq + s % 8, ax = pt.ax[i];
                 const int ta = min(16 * tile + gid, nt - 1), tb = min(16 * tile + gid + 8, nt - 1);
                 float4 v;
-                sincos_coord(int64_t(crd_s[3 * ta + ax]) - p, tf_s[i], &v.z, &v.x);
-                sincos_coord(int64_t(crd_s[3 * tb + ax]) - p, tf_s[i], &v.w, &v.y);
+                sincos_coord(int64_t(crd_s[3 * ta + ax]) - p, pt.tf[i], &v.z, &v.x);
+                sincos_coord(int64_t(crd_s[3 * tb + ax]) - p, pt.tf[i], &v.w, &v.y);
                 tr_s[e] = v;
             }
             __syncthreads();
@@ -674,20 +678,24 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
                     va = (acc[0][c] + acc[1][c]) * a.scale;
                     vb = (acc[0][2 + c] + acc[1][2 + c]) * a.scale;
                 }
-                float* lg = lg_s + (kh * g + 2 * tq + c) * f.pitch;
-                if (ta < nt) lg[ta] = ok_a ? va : -INFINITY;
-                if (tb < nt) lg[tb] = ok_b ? vb : -INFINITY;
+                float* dst = lg + (kh * g + 2 * tq + c) * lg_pitch;
+                if (ta < nt) dst[ta] = ok_a ? va : -INFINITY;
+                if (tb < nt) dst[tb] = ok_b ? vb : -INFINITY;
             }
         }
     }
-    if (CACHED && err) atomicOr(a.status, err);
-    __syncthreads();
+}
 
-    // statistics of the CTA's tokens, two heads of a warp side by side
+// (max, sum of exp) per query head of nt tokens' logits in shared memory, two
+// heads of a warp side by side.
+template <int NT>
+__device__ __forceinline__ void cta_stats(const float* lg_s, int pitch, int Hq, int nt, float2* stat) {
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int h0 = warp; h0 < Hq; h0 += 2 * NW) {
         const bool two = h0 + NW < Hq;
-        const float* ra = lg_s + h0 * f.pitch;
-        const float* rb = lg_s + (two ? h0 + NW : h0) * f.pitch;
+        const float* ra = lg_s + h0 * pitch;
+        const float* rb = lg_s + (two ? h0 + NW : h0) * pitch;
         float ma = -INFINITY, mb = -INFINITY, za = 0.0f, zb = 0.0f;
         for (int t = lane; t < nt; t += 32) {
             ma = fmaxf(ma, ra[t]);
@@ -709,10 +717,42 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
             zb += __shfl_xor_sync(kAll, zb, o);
         }
         if (lane == 0) {
-            sh.stat[h0] = make_float2(ma, za);
-            if (two) sh.stat[h0 + NW] = make_float2(mb, zb);
+            stat[h0] = make_float2(ma, za);
+            if (two) stat[h0 + NW] = make_float2(mb, zb);
         }
     }
+}
+
+// The whole selection in one kernel; the CTA's logits stay in shared memory.
+// Small calls are a chain of latencies, which one kernel shortens by three
+// launches: 768 tokens x 8 KV heads in a cluster of 16, ~20k cycles: queries
+// and first rows 2.7k, cos/sin and MMAs 5.5k, statistics and their exchange
+// 4.8k, relevances and theirs 5k, search and output 2.7k. Measured with its
+// launches 20.9 -> 12.5 us (four kernels before), 8 sequences 20.6 -> 13.6 us,
+// 4 of 1000 tokens at head_dim 256 29.6 -> 13.9 us (CUDA cores before).
+constexpr int kFusedThreads = 512;
+
+template <int D, bool CACHED>
+__global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __grid_constant__ SelectArgs a) {
+    constexpr int NT = kFusedThreads;
+    __shared__ SelectShared sh;
+    __shared__ PairTables<D, CACHED, NT> pt;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_allow();
+    const int C = a.cluster, b = int(blockIdx.x) / C, rank = int(cluster_rank()), T = a.tok_per_cta;
+    const int M = a.n_tokens, Hq = a.n_q_heads;
+    const int m_beg = rank * T, nt = max(0, min(T, M - m_beg));
+    const int tid = threadIdx.x;
+    const FusedLayout f = fused_layout(D, CACHED, a.n_kv_heads, Hq, T, C);
+    float* lg_s = reinterpret_cast<float*>(smem_raw + f.logits);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + f.keys);
+    pt.set(a);
+    uint32_t err = 0;
+    pdl_wait();
+    cta_logits<D, CACHED, NT>(a, f, b, 0, a.n_kv_heads, m_beg, nt, smem_raw, pt, lg_s, f.pitch, err);
+    if (CACHED && err) atomicOr(a.status, err);
+    __syncthreads();
+    cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
     merge_stats<NT>(a, C, sh);
 
     // relevances: `per` lanes share a token (its heads in turn) where the CTA
@@ -736,6 +776,37 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     select_topk<NT>(a, b, C, m_beg, nt, keys, lo, hi, sh);
 }
 
+// Logits of the cached-key selection to global memory, where it is too large for
+// one cluster per sequence: a CTA takes one (sequence, chunk of tok_per_cta
+// tokens, group of kh_per_item KV heads), two CTAs per SM, so that one's set-up
+// runs beside the other's streaming. DRAM bounds it, with 64 KB of keys in flight
+// per SM; these need lines of L1, so shared memory is kept small (logits staged
+// there for whole-line stores and statistics, 200 KB per SM, made it 2 to 3
+// times slower). Measured against a kernel whose warps each looked up their rows
+// per item and loaded 64 bytes per lane (half a sector per load), whole selections:
+// 16 sequences of 8192 tokens x 8 heads of 128 66.8 -> 63.1 us, 32 of 16,384 212.6
+// -> 206.0 us, 16 of 4096 40.1 -> 36.6 us, 7 of 8192 40.3 -> 36.0 us.
+constexpr int kSplitThreads = 256;
+
+template <int D>
+__global__ void __launch_bounds__(kSplitThreads, 2) select_logits_kernel(const __grid_constant__ SelectArgs a) {
+    constexpr int NT = kSplitThreads;
+    __shared__ PairTables<D, true, NT> pt;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Hq = a.n_q_heads, H = a.n_kv_heads, g = Hq / H, M = a.n_tokens, T = a.tok_per_cta;
+    const int n_hg = (H + a.kh_per_item - 1) / a.kh_per_item, n_chunks = (M + T - 1) / T;
+    const int unit = int(blockIdx.x) / n_hg, kh0 = (int(blockIdx.x) - unit * n_hg) * a.kh_per_item;
+    const int b = unit / n_chunks, m_beg = (unit - b * n_chunks) * T;
+    const FusedLayout f = fused_layout(D, true, a.kh_per_item, a.kh_per_item * g, T, 0, false);
+    pdl_allow();
+    pt.set(a);
+    uint32_t err = 0;
+    pdl_wait();
+    cta_logits<D, true, NT>(a, f, b, kh0, min(a.kh_per_item, H - kh0), m_beg, min(T, M - m_beg), smem_raw, pt,
+                            a.logits + (int64_t(b) * Hq + kh0 * g) * M + m_beg, M, err);
+    if (err) atomicOr(a.status, err);
+}
+
 cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaStream_t stream,
                                   cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg = {};
@@ -756,6 +827,7 @@ cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaS
 
 constexpr int kFusedMinTokens = 32;  // per CTA
 constexpr int kFusedRows = 640;
+constexpr int kSplitMinTokens = 64, kSplitMaxTokens = 2048;  // per CTA of the logits kernel
 constexpr size_t kMaxDynSmem = 208 * 1024;  // beside the static shared memory, within 227 KB
 
 // Clusters of 1..16 CTAs of a kernel that the current device holds at once, one
@@ -845,6 +917,31 @@ cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t str
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kFusedThreads, t.cluster, f.total, stream, attr);
     *done = true;
     return cudaLaunchKernelEx(&cfg, kern, t);
+}
+
+// Chunks of the cached-key logits: as many per sequence as make one wave of two
+// CTAs per SM, of at least kSplitMinTokens tokens and at most kSplitMaxTokens.
+template <int D>
+cudaError_t launch_logits_split(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
+    SelectArgs t = a;
+    const int H = a.n_kv_heads, g = a.n_q_heads / H;
+    t.kh_per_item = H < 1024 / D ? H : 1024 / D;  // 32 KB of query fragments at most
+    const int64_t per = int64_t(n_seqs) * ((H + t.kh_per_item - 1) / t.kh_per_item);
+    const int64_t n = std::max<int64_t>(1, 2 * int64_t(sms) / per);
+    const int64_t T = std::min<int64_t>(kSplitMaxTokens, std::max<int64_t>(kSplitMinTokens, (a.n_tokens + n - 1) / n));
+    t.tok_per_cta = int((T + 15) / 16 * 16);
+    const size_t smem = fused_layout(D, true, t.kh_per_item, t.kh_per_item * g, t.tok_per_cta, 0, false).total;
+    const int64_t grid = per * ((a.n_tokens + t.tok_per_cta - 1) / t.tok_per_cta);
+    if (grid > INT32_MAX) return cudaErrorInvalidValue;
+    const cudaError_t e = cudaFuncSetAttribute(select_logits_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(select_logits_kernel<D>, dim3(unsigned(grid)), dim3(kSplitThreads), smem, stream, t);
+}
+
+cudaError_t launch_select_cached_logits(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
+    return a.head_dim == 64    ? launch_logits_split<64>(a, n_seqs, sms, stream)
+           : a.head_dim == 128 ? launch_logits_split<128>(a, n_seqs, sms, stream)
+                               : launch_logits_split<256>(a, n_seqs, sms, stream);
 }
 
 cudaError_t launch_select_fused(const SelectArgs& a, bool cached, int n_seqs, int sms, cudaStream_t stream, bool* done) {
