@@ -826,7 +826,7 @@ cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaS
 }
 
 constexpr int kFusedMinTokens = 32;  // per CTA
-constexpr int kFusedRows = 640;
+constexpr int kFusedRowsRaw = 640, kFusedRowsCached = 1152;
 constexpr int kSplitMinTokens = 64, kSplitMaxTokens = 2048;  // per CTA of the logits kernel
 constexpr size_t kMaxDynSmem = 208 * 1024;  // beside the static shared memory, within 227 KB
 
@@ -897,9 +897,9 @@ cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t str
 // kernels), raw keys, 8 heads of 128: 1 sequence of 1024 tokens (512 rows per
 // CTA) 13.0 | 15.2, of 2048 17.7 | 16.3, of 4096 27.8 | 18.1; 7 of 2048 (1024
 // rows) 19.1 | 27.1, of 4096 29.4 | 32.8, of 8192 61.9 | 43.8; 16 of 1024 21.0
-// | 28.9, of 2048 34.3 | 34.7. Cached keys: 1 of 1024 13.4 | 16.4, of 2048
-// 17.6 | 17.1; 7 of 4096 26.3 | 28.1, of 8192 44.9 | 40.1; 16 of 2048 29.1 |
-// 26.6. The line below lies between them.
+// | 28.9, of 2048 34.3 | 34.7. Cached keys: 1 of 1024 12.4 | 16.2, of 2048
+// 15.3 | 17.5, of 4096 20.0 | 19.0; 7 of 4096 22.5 | 25.5, of 8192 35.9 | 36.6; 16
+// of 2048 23.7 | 24.7, of 4096 40.3 | 36.6. The line below lies between them.
 template <int D, bool CACHED>
 cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream, bool* done) {
     auto kern = select_fused_kernel<D, CACHED>;
@@ -912,7 +912,7 @@ cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t str
     const int64_t rows = int64_t(t.tok_per_cta) * a.n_kv_heads * D / 128;
     const int64_t spread = int64_t(n_seqs) * a.n_tokens * a.n_kv_heads * D / 128 / sms;
     // (the other path's logits kernel for raw keys of head_dim 256 takes ~3 times as long)
-    if (f.total > kMaxDynSmem || rows > kFusedRows + spread * (D == 256 && !CACHED ? 3 : 1)) return cudaSuccess;
+    if (f.total > kMaxDynSmem || rows > (CACHED ? kFusedRowsCached : kFusedRowsRaw) + spread * (D == 256 && !CACHED ? 3 : 1)) return cudaSuccess;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kFusedThreads, t.cluster, f.total, stream, attr);
     *done = true;
