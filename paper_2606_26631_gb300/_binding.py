@@ -139,8 +139,16 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# torch's current stream as the raw handle alone: a torch.cuda.Stream object
+# made for every call costs more host time (3.7 us) than the rest of the binding
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         if torch.cuda.is_available():
             return torch.cuda.current_stream().cuda_stream
         return None
@@ -164,7 +172,8 @@ def rope_cfg(n_layers: int, n_kv_heads: int, head_dim: int, sections, theta: flo
 def _bf16(t: torch.Tensor, name: str):
     if t.dtype != torch.bfloat16:
         raise TypeError(f"{name} must be bfloat16")
-    if t.stride(-1) != 1 or t.stride(-2) != t.shape[-1]:
+    stride = t.stride()
+    if stride[-1] != 1 or stride[-2] != t.shape[-1]:
         raise ValueError(f"{name}: a [heads, head_dim] row must be contiguous")
 
 
@@ -289,14 +298,15 @@ def store_raw(cfg, store, seq: int, layer_begin: int, m_begin: int, k_src: torch
               v_src: torch.Tensor, coords_src: Optional[torch.Tensor] = None, stream=None):
     """prcr_store_raw: k_src / v_src are [n_layers, m_count, H, D] bf16 (row-contiguous)."""
     _bf16(k_src, "k_src"); _bf16(v_src, "v_src")
-    if k_src.stride() != v_src.stride() or k_src.shape != v_src.shape:
+    stride, shape = k_src.stride(), k_src.shape
+    if stride != v_src.stride() or shape != v_src.shape:
         raise ValueError("k_src and v_src must have the same shape and strides")
     if coords_src is not None and (coords_src.dtype != torch.int32 or not coords_src.is_contiguous()):
         raise TypeError("coords_src must be a contiguous int32 [m_count, 3] tensor")
     rc = lib().prcr_store_raw(C.byref(cfg), C.byref(store), int(seq), int(layer_begin),
-                              int(k_src.shape[0]), int(m_begin), int(k_src.shape[1]),
-                              k_src.data_ptr(), v_src.data_ptr(), k_src.stride(0), k_src.stride(1),
-                              _ptr(coords_src), _stream(stream))
+                              shape[0], int(m_begin), shape[1], k_src.data_ptr(),
+                              v_src.data_ptr(), stride[0], stride[1], _ptr(coords_src),
+                              _stream(stream))
     return _check(rc, "prcr_store_raw")
 
 
@@ -306,15 +316,15 @@ def prefill_capture(cfg, store, cache, seq: int, layer_begin: int, m_begin: int,
     """prcr_prefill_capture: k_src / v_src are the prefill's pre-rotation rows
     [n_layers, m_count, H, D] bf16 (row-contiguous); coords_src [m_count, 3] int32."""
     _bf16(k_src, "k_src"); _bf16(v_src, "v_src")
-    if k_src.stride() != v_src.stride() or k_src.shape != v_src.shape:
+    stride, shape = k_src.stride(), k_src.shape
+    if stride != v_src.stride() or shape != v_src.shape:
         raise ValueError("k_src and v_src must have the same shape and strides")
     if coords_src.dtype != torch.int32 or not coords_src.is_contiguous():
         raise TypeError("coords_src must be a contiguous int32 [m_count, 3] tensor")
     rc = lib().prcr_prefill_capture(C.byref(cfg), C.byref(store), C.byref(cache), int(seq),
-                                    int(layer_begin), int(k_src.shape[0]), int(m_begin),
-                                    int(k_src.shape[1]), int(slot_begin), k_src.data_ptr(),
-                                    v_src.data_ptr(), k_src.stride(0), k_src.stride(1),
-                                    coords_src.data_ptr(), status.data_ptr(), _stream(stream))
+                                    int(layer_begin), shape[0], int(m_begin), shape[1],
+                                    int(slot_begin), k_src.data_ptr(), v_src.data_ptr(),
+                                    stride[0], stride[1], coords_src.data_ptr(), status.data_ptr(), _stream(stream))
     return _check(rc, "prcr_prefill_capture")
 
 
