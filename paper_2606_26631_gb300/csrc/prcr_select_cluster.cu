@@ -7,11 +7,12 @@
 // sequence (T = tok_per_cta). Two exchanges through distributed shared memory
 // stand where kernel boundaries would:
 //   1. softmax statistics: every CTA reduces its tokens' logits to a (max, sum
-//      of exp) per query head; after a cluster barrier each CTA merges all C
-//      of them into the heads' normalisers;
+//      of exp) per query head and writes them into all C CTAs; after a cluster
+//      barrier each CTA merges them into the heads' normalisers;
 //   2. relevance of the CTA's own tokens (mean over the heads of the softmax
-//      weight, heads in ascending order), left in shared memory; after a
-//      second barrier each CTA copies the whole sequence's relevances.
+//      weight), written into all of them as well; after a second barrier each
+//      CTA holds the whole sequence's relevances.
+// (Remote writes before a barrier cost less than remote reads after it.)
 // Every CTA then finds the K-th largest relevance by itself (the same answer
 // in each) and writes its own tokens' share of the selection in index order,
 // knowing from the copy how many lie before its first token. The search
@@ -46,7 +47,7 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // Address of this CTA's shared variable at `p` in the shared memory of CTA
-// `rank` of the cluster, and loads from there.
+// `rank` of the cluster, and stores to there.
 __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
@@ -54,47 +55,47 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
                  : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
     return r;
 }
-__device__ __forceinline__ float2 peer_f32x2(uint32_t addr) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-    return v;
+__device__ __forceinline__ void peer_store(uint32_t addr, uint32_t x, uint32_t y) {
+    asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
 }
-__device__ __forceinline__ uint4 peer_u32x4(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(addr));
-    return v;
+__device__ __forceinline__ void peer_store(uint32_t addr, const uint4& v) {
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
 }
 
 // What the phases share, in static shared memory.
 struct SelectShared {
-    float2 stat[kSelectMaxQHeads];  // this CTA's (max, sum) per query head; read by the peers
+    float2 stat[kSelectMaxQHeads];  // this CTA's (max, sum) per query head
+    float2 all[kMaxCluster][kSelectMaxQHeads];  // every CTA's; written by the peers
     float2 norm[kSelectMaxQHeads];  // (max, 1 / (sum * n_q_heads)) over the whole sequence
     uint32_t hist[kBuckets];
-    uint2 range;                    // smallest and largest key of this CTA's tokens; read by the peers
+    uint2 range[kMaxCluster][32];   // smallest and largest key of every CTA's warps; written by the peers
     uint32_t wsum[32];              // per warp: keys in its buckets; later equal | above << 16 in its tokens
     uint32_t before[2][32];         // per warp: keys equal to X and above it before this CTA's first token
     uint32_t pick[3];               // bucket of the K-th largest, keys in it, keys above it
     uint32_t list[32], n_list;
 };
 
-// Exchange 1: the heads' normalisers from every CTA's statistics. Also sets up
-// the search's shared state.
+// Exchange 1: the heads' normalisers from every CTA's statistics (stat, visible
+// to the CTA), which each CTA writes into all of them. Also sets up the search's
+// shared state. The caller has arrived at the cluster barrier once at its start:
+// its completion here means that every peer is running.
 template <int NT>
-__device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, SelectShared& sh) {
+__device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, int rank, SelectShared& sh) {
+    const int c = threadIdx.x & (kMaxCluster - 1);
+    cluster_wait();
+    for (int hq = threadIdx.x / kMaxCluster; hq < a.n_q_heads; hq += NT / kMaxCluster) {
+        const float2 v = sh.stat[hq];
+        if (c < C) peer_store(peer_addr(&sh.all[rank][hq], uint32_t(c)), __float_as_uint(v.x), __float_as_uint(v.y));
+    }
     cluster_arrive();
     for (int i = threadIdx.x; i < kBuckets; i += NT) sh.hist[i] = 0u;
-    if (threadIdx.x == 0) {
-        sh.range = make_uint2(0xffffffffu, 0u);
-        sh.n_list = 0u;
-    }
+    if (threadIdx.x == 0) sh.n_list = 0u;
     cluster_wait();
-    const int c = threadIdx.x & (kMaxCluster - 1);
     for (int h0 = 0; h0 < a.n_q_heads; h0 += NT / kMaxCluster) {
         const int hq = h0 + threadIdx.x / kMaxCluster;
         float2 v = make_float2(-INFINITY, 0.0f);
-        if (hq < a.n_q_heads && c < C) v = peer_f32x2(peer_addr(&sh.stat[hq], uint32_t(c)));
+        if (hq < a.n_q_heads && c < C) v = sh.all[c][hq];
         float m = v.x;
 #pragma unroll
         for (int o = kMaxCluster / 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
@@ -111,8 +112,8 @@ __device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, SelectSh
 }
 
 // Exchange 2, the search and the output. keys [C * T] holds this CTA's own
-// tokens' relevances at m_beg; the peers' are copied in. lo, hi: smallest and
-// largest of the relevances that this thread wrote.
+// tokens' relevances at m_beg, which are copied to the peers as theirs are
+// here. lo, hi: smallest and largest of the relevances that this thread wrote.
 template <int NT>
 __device__ __forceinline__ void select_topk(const SelectArgs& a, int b, int C, int m_beg, int nt, uint32_t* keys,
                                             uint32_t lo, uint32_t hi, SelectShared& sh) {
@@ -121,27 +122,27 @@ __device__ __forceinline__ void select_topk(const SelectArgs& a, int b, int C, i
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     lo = __reduce_min_sync(kAll, lo);
     hi = __reduce_max_sync(kAll, hi);
-    if (lane == 0 && lo <= hi) {
-        atomicMin(&sh.range.x, lo);
-        atomicMax(&sh.range.y, hi);
+    if (lane < C) peer_store(peer_addr(&sh.range[m_beg / T][warp], uint32_t(lane)), lo, hi);
+    __syncthreads();  // the CTA's relevances
+    {
+        const int n4 = (nt + 3) / 4;  // T is a multiple of 16: whole groups of four
+        for (int i = tid; i < n4 * C; i += NT) {
+            const int c = i / n4, j = m_beg + 4 * (i - c * n4);
+            if (c * T != m_beg) peer_store(peer_addr(keys + j, uint32_t(c)), *reinterpret_cast<const uint4*>(keys + j));
+        }
     }
     cluster_arrive();
     cluster_wait();
-    uint2 range = make_uint2(0xffffffffu, 0u);
-    if (lane < C) {
-        const float2 v = peer_f32x2(peer_addr(&sh.range, uint32_t(lane)));
-        range = make_uint2(__float_as_uint(v.x), __float_as_uint(v.y));
+    {
+        uint2 v = make_uint2(0xffffffffu, 0u);
+        for (int i = lane; i < C * NW; i += 32) {
+            const uint2 w = sh.range[i / NW][i % NW];
+            v.x = min(v.x, w.x);
+            v.y = max(v.y, w.y);
+        }
+        lo = __reduce_min_sync(kAll, v.x);
+        hi = __reduce_max_sync(kAll, v.y);
     }
-#pragma unroll 4
-    for (int i = 4 * tid; i < M; i += 4 * NT) {  // T is a multiple of 16: four tokens share a rank
-        const int r = i / T;
-        const uint4 v = peer_u32x4(peer_addr(keys + i, uint32_t(r)));
-        if (r * T != m_beg) *reinterpret_cast<uint4*>(keys + i) = v;
-    }
-    cluster_arrive();  // this CTA has read its peers; it waits for their reads before it ends
-    lo = __reduce_min_sync(kAll, range.x);
-    hi = __reduce_max_sync(kAll, range.y);
-    __syncthreads();
 
     // the K-th largest key X lies in [lo, hi]; `above` keys are larger than hi
     const uint32_t K = uint32_t(a.k);
@@ -272,7 +273,6 @@ __device__ __forceinline__ void select_topk(const SelectArgs& a, int b, int C, i
             a.seq_rev_off[b + 1] = b + 1;
         }
     }
-    cluster_wait();
 }
 
 // (max, sum of exp) of 16 logits (-inf where there is none) into a running one.
@@ -351,10 +351,12 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
     float* rel = reinterpret_cast<float*>(keys + m_beg);
     const float* lg = a.logits + int64_t(b) * Hq * M + m_beg;
     const bool vec = (M & 3) == 0;  // rows of logits 16-byte aligned (m_beg is a multiple of 16)
+    cluster_arrive();
     pdl_wait();
 
     tail_stats<NW>(lg, M, Hq, nt, vec, sh);
-    merge_stats<NT>(a, C, sh);
+    __syncthreads();
+    merge_stats<NT>(a, C, rank, sh);
     uint32_t lo = 0xffffffffu, hi = 0u;
     auto seen = [&](float r) {
         lo = min(lo, __float_as_uint(r));
@@ -747,13 +749,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     float* lg_s = reinterpret_cast<float*>(smem_raw + f.logits);
     uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + f.keys);
     pt.set(a);
+    cluster_arrive();
     uint32_t err = 0;
     pdl_wait();
     cta_logits<D, CACHED, NT>(a, f, b, 0, a.n_kv_heads, m_beg, nt, smem_raw, pt, lg_s, f.pitch, err);
     if (CACHED && err) atomicOr(a.status, err);
     __syncthreads();
     cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
-    merge_stats<NT>(a, C, sh);
+    __syncthreads();
+    merge_stats<NT>(a, C, rank, sh);
 
     // relevances: `per` lanes share a token (its heads in turn) where the CTA
     // has few tokens
@@ -828,7 +832,7 @@ cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaS
 constexpr int kFusedMinTokens = 32;  // per CTA
 constexpr int kFusedRowsRaw = 640, kFusedRowsCached = 1152;
 constexpr int kSplitMinTokens = 64, kSplitMaxTokens = 2048;  // per CTA of the logits kernel
-constexpr size_t kMaxDynSmem = 208 * 1024;  // beside the static shared memory, within 227 KB
+constexpr size_t kMaxDynSmem = 192 * 1024;  // beside the static shared memory, within 227 KB
 
 // Clusters of 1..16 CTAs of a kernel that the current device holds at once, one
 // CTA per SM; found, and the kernel's attributes set, once per device.
