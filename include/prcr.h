@@ -310,7 +310,8 @@ PRCR_API int prcr_prefill_capture(const prcr_rope_cfg* cfg, const prcr_store_des
  * query heads per KV head and n_q_heads * D <= PRCR_DECODE_MAX_Q_ELEMS;
  * n_seqs and n_layers at most 65535 (launch grid limits).
  * workspace: device, >= prcr_decode_workspace_size(...) bytes (0 when the
- * sequence axis is not split), 16-byte aligned. A seq_len beyond the
+ * sequence axis is not split for any length up to max_len), 16-byte aligned.
+ * A seq_len beyond the
  * capacity, or above max_len, sets PRCR_ST_CAPACITY (the slots past the
  * capacity, or past the split made for max_len, are left out); an unmapped
  * block in range sets

@@ -383,22 +383,72 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     return launch_capture(a, grid, block, smem, stream) == cudaSuccess ? PRCR_OK : PRCR_ECUDA;
 }
 
-// The chunks that the sequence axis is split into.
+// The chunks that the sequence axis is split into, and *most, the most that any
+// max_len up to this one is split into (a workspace sized for it then holds the
+// shorter calls too).
 //
-// head_dim 64 and 128, one warp per (chunk, KV head): as many as make one wave
-// of resident warps (a step of few layers and sequences is then over in one go);
-// where those chunks would be longer than 1.25 kChunk slots, chunks of kChunk,
-// many waves of which even out lengths that differ. Measured (us; 1 wave | 2): 1
-// sequence x 36 layers x 8 heads of 933 slots 30.6 | 32.9, 4 x 28 x 4 of up to
-// 2000 (500-slot chunks) 62.8 | 70.2. Large ones at chunks of 384, 512, 768,
-// 1024 and 1536 slots: 8 x 28 x 4 of up to 4096 218, 208, 209, 232, 219; 16 x
-// 36 x 8 912, 895, 896, 886, 900; head_dim 64, 8 x 28 x 3 102, 96, 122, 95, 127.
+// head_dim 64 and 128, a small batch: teams of 2..12 warps in one wave of the
+// GPU's resident warps (12 per SM, whatever their CTAs).
+// - The largest team of which every (sequence, layer, KV head) has one at once
+//   takes it unsplit, and no merge follows, if that keeps two thirds of the warps
+//   busy (three quarters above 1024 slots, where a merge weighs less). Measured
+//   (us, calls in a row; chunks for one warp each | unsplit | split teams): 1
+//   sequence x 36 layers x 8 heads of 933 slots 29.2 | 25.2 | 27.5, 1 x 28 x 4 of
+//   933 (74 % busy) 20.0 | 15.5 | 16.7, of 4096 48.7 | 42.6 | 44.0; head_dim 64,
+//   1 x 28 x 4 of 4096 27.0 | 27.9 | 25.3, 2 x 28 x 4 of up to 800 13.9 | 13.5 | 14.5.
+// - Else the team and chunks that keep the most warps busy, two tiles or more
+//   each; a smaller team, whose chunks are more to merge, only for an eighth more
+//   (14 x 2 x 1 of up to 7132: 24.4 with chunks for one warp each, 19.9; 1 x 4 x 8
+//   of 6000 28.7 -> 21.3; 2 x 10 x 8 of up to 1500 29.0 -> 26.9).
+// - Several sequences' lengths differ, so where a team's warps would have more
+//   than 2 kChunk slots (a warp by itself 1.25 kChunk) the batch is a large one:
+//   8 x 28 x 4 of up to 4096 would take 222 us with teams of two, not 207; of up
+//   to 2000 it takes 110, not 123. One sequence has no such limit: 1 x 36 x 8 of
+//   4096 slots 113 -> 94, of 16384 383 -> 366.
+// Large batches: one warp per chunk of kChunk slots, many waves of which even
+// out lengths that differ. Measured at chunks of 384, 512, 768, 1024 and 1536
+// slots: 8 sequences x 28 layers x 4 heads of up to 4096 slots 218, 208, 209,
+// 232, 219 us; 16 x 36 x 8 912, 895, 896, 886, 900; head_dim 64, 8 x 28 x 3 102,
+// 96, 122, 95, 127.
 template <int D>
-int64_t decode_chunk(int64_t units, int64_t max_len, int sms) {
+int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, int* team,
+                     int64_t* most) {
     using Sh = DecodeShape<D>;
-    const int64_t want = std::max<int64_t>(1, int64_t(sms) * Sh::kCtas * Sh::kWarps / units);
-    const int64_t c = ((max_len + want - 1) / want + 15) / 16 * 16;
-    return c <= Sh::kChunk * 5 / 4 ? c : Sh::kChunk;
+    constexpr int kPerSm = Sh::kCtas * Sh::kWarps;
+    static_assert(kPerSm == kDecodeMaxTeam, "the largest team fills an SM");
+    const int64_t warps = int64_t(sms) * kPerSm, tiles = (max_len + 15) / 16;
+    const bool lng = max_len > 1024;
+    int64_t busy = 0, splits = 1;
+    *team = 0;
+    *most = 1;
+    for (int w : {12, 6, 4, 3, 2, 1}) {
+        const int64_t slots = int64_t(sms) * (kPerSm / w);
+        if (units > slots) continue;
+        if (busy == 0 && w > 1 && units * w * 12 > warps * (lng ? 9 : 8)) {
+            *team = w;  // unsplit
+            break;
+        }
+        const int64_t s = std::max<int64_t>(1, std::min(slots / units, tiles / (2 * w)));
+        *most = std::max(*most, s);
+        if (units * w * s * 8 > busy * 9) {
+            busy = units * w * s;
+            *team = w;
+            splits = s;
+        }
+    }
+    const int64_t share = splits * std::max(1, *team);
+    if ((*team <= 1 || n_seqs > 1) &&
+        (max_len + share - 1) / share > Sh::kChunk * (*team > 1 ? 2 : 1.25)) {
+        *team = 0;
+        *most = std::max(*most, (max_len + Sh::kChunk - 1) / Sh::kChunk);
+        return Sh::kChunk;
+    }
+    // the fewest warps that take as many rounds of tiles
+    const int64_t per = (tiles + splits - 1) / splits;
+    for (int w : {6, 4, 3, 2})
+        if (w < *team && (per + w - 1) / w == (per + *team - 1) / *team) *team = w;
+    if (*team == 1) *team = 0;
+    return per * 16;
 }
 
 // head_dim 256: one KV head per CTA, about 8 waves of kDecodeWideCtasPerSm
@@ -418,15 +468,17 @@ int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms) {
     return std::min<int64_t>(c, kDecodeMaxChunk / round * round);
 }
 
-void decode_split(int64_t base_ctas, int64_t max_len, int sms, int n_kv_heads, int head_dim,
-                  int* splits, int* chunk) {
-    const int64_t units = base_ctas * n_kv_heads;
-    const int64_t c = head_dim == 64    ? decode_chunk<64>(units, max_len, sms)
-                      : head_dim == 128 ? decode_chunk<128>(units, max_len, sms)
+void decode_split(int64_t n_seqs, int n_layers, int64_t max_len, int sms, int n_kv_heads,
+                  int head_dim, int* splits, int* chunk, int* team, int64_t* most) {
+    const int64_t units = n_seqs * n_layers * n_kv_heads;
+    *team = 0;
+    *most = 1;
+    const int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, team, most)
+                      : head_dim == 128 ? decode_chunk<128>(n_seqs, units, max_len, sms, team, most)
                                         : decode_wide_chunk(units, max_len, sms);
     *chunk = int(c);
     *splits = int((max_len + c - 1) / c);
-    if (*splits < 1) *splits = 1;
+    *most = std::max<int64_t>(*most, *splits);
 }
 
 bool decode_shape_ok(const prcr_rope_cfg* cfg, int32_t n_q_heads) {
@@ -616,11 +668,12 @@ size_t prcr_decode_workspace_size(const prcr_rope_cfg* cfg, int32_t n_seqs, int3
     if (check_cfg(cfg) || n_seqs < 1 || max_len < 1 || !decode_shape_ok(cfg, n_q_heads)) return 0;
     int dev = 0, sms = 1;
     if (cudaGetDevice(&dev) == cudaSuccess) sms = sm_count(dev);
-    int splits = 1, chunk = 32;
-    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sms, cfg->n_kv_heads, cfg->head_dim,
-                 &splits, &chunk);
-    if (splits == 1) return 0;
-    return size_t(n_seqs) * cfg->n_layers * n_q_heads * splits * (cfg->head_dim + 2) * sizeof(float);
+    int splits = 1, chunk = 32, team = 0;
+    int64_t most = 1;
+    decode_split(n_seqs, cfg->n_layers, max_len, sms, cfg->n_kv_heads, cfg->head_dim,
+                 &splits, &chunk, &team, &most);
+    if (most == 1) return 0;
+    return size_t(n_seqs) * cfg->n_layers * n_q_heads * most * (cfg->head_dim + 2) * sizeof(float);
 }
 
 int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache, int32_t n_seqs,
@@ -644,8 +697,9 @@ int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
     DecodeArgs a = {};
-    decode_split(int64_t(n_seqs) * cfg->n_layers, max_len, sm_count(dev), cfg->n_kv_heads,
-                 cfg->head_dim, &a.splits, &a.chunk);
+    int64_t most;
+    decode_split(n_seqs, cfg->n_layers, max_len, sm_count(dev), cfg->n_kv_heads,
+                 cfg->head_dim, &a.splits, &a.chunk, &a.team, &most);
     if (n_seqs > 65535 || cfg->n_layers > 65535) return PRCR_EINVAL;  // grid z and y
     if (a.splits > 1) {
         const size_t need = size_t(n_seqs) * cfg->n_layers * n_q_heads * a.splits *

@@ -65,19 +65,23 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
 // each): products stay exact and the result keeps ~16 bits per operand; K and V
 // are bf16 already and enter exactly. A tile's P V is summed from zero and
 // added to the running accumulator by the FMA that rescales it.
+// TEAM: a CTA of up to kDecodeMaxTeam warps takes one unit, its warps the chunk's
+// tiles in turn, and merges their (max, sum, accumulator) in shared memory, so
+// that a small batch needs no chunks and no merge kernel (29.2 -> 25.2 us for one
+// sequence of 933 slots x 36 layers x 8 heads; the rule is decode_chunk's).
 // DRAM bounds it: an SM's 12 warps keep ~100 KB in flight (~2.2 us at its share
 // of the copy rate). Measured, before | now (before: a CTA looping over the KV
 // heads with K in registers for large batches, CTAs of four heads each for
 // small ones): 16 sequences x 36 layers x 8 heads of up to 4096 slots 925 | 893
 // us (6.5 TB/s), 8 x 28 x 4 214 | 207, 11 x 24 x 5 of up to 6900 573 | 453, 5 x
-// 36 x 8 of up to 3500 346 | 308, 14 x 2 x 1 head of up to 7132 37.6 | 24.3; head_dim
-// 64: 12 x 28 x 8 275 | 223, 1 x 28 x 4 31.7 | 27.2. 8 x 28 x 4 of up to 3000
+// 36 x 8 of up to 3500 346 | 308, 14 x 2 x 1 head of up to 7132 37.6 | 19.9; head_dim
+// 64: 12 x 28 x 8 275 | 223, 1 x 28 x 4 31.7 | 25.3. 8 x 28 x 4 of up to 3000
 // slots went 166 -> 171: its 512-slot chunks end in a short last wave. Equal
 // static runs of tiles per warp instead of chunks: 229 us for the second.
-template <int D>
-__global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::kCtas)
+template <int D, bool TEAM>
+__global__ void __launch_bounds__(TEAM ? kDecodeMaxTeam * 32 : DecodeShape<D>::kWarps * 32, TEAM ? 1 : DecodeShape<D>::kCtas)
     decode_kernel(const __grid_constant__ DecodeArgs a) {
-    constexpr int kRingWarps = DecodeShape<D>::kWarps;
+    const int kRingWarps = TEAM ? int(blockDim.x >> 5) : DecodeShape<D>::kWarps;
     // rounds of eight query pairs per lane: a GQA group is at most 8 heads
     constexpr int kRingQRounds = (D / 2 + 31) / 32;
     constexpr int KS = D / 16;      // k-steps of QK, m-tiles of PV
@@ -90,7 +94,8 @@ __global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::k
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) float s_cos[kMaxPairs];
     __shared__ __align__(16) float s_sin[kMaxPairs];
-    __shared__ uint32_t s_mask[kRingWarps][NS];
+    __shared__ uint32_t s_mask[TEAM ? kDecodeMaxTeam : DecodeShape<D>::kWarps][NS];
+    __shared__ float s_m[TEAM ? kDecodeMaxTeam : 1][8], s_l[TEAM ? kDecodeMaxTeam : 1][8];
     const int P = D / 2;
     const int g = a.group;
     const int H = a.n_kv_heads;
@@ -106,16 +111,16 @@ __global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::k
     const int gid = lane >> 2;
     const int t = lane & 3;
     float* q_s = reinterpret_cast<float*>(ring + size_t((NS - 1) * kRingWarps + warp) * (KT + VT));
-    // this warp's chunk and KV head: units of (chunk, head), heads fastest
-    const int unit = int(blockIdx.x) * kRingWarps + warp;
+    // this warp's (or the team's) chunk and KV head: units of (chunk, head), heads
+    // fastest
+    const int unit = TEAM ? int(blockIdx.x) : int(blockIdx.x) * kRingWarps + warp;
     const int split = unit / H, kh = unit - split * H;
     const bool wact = split < a.splits;
     const uint16_t* wk = ring + size_t(warp) * (KT + VT);  // this warp's stage 0
     const uint32_t wk_s = uint32_t(__cvta_generic_to_shared(wk));
     const uint32_t wv_s = wk_s + uint32_t(KT * 2);
-    constexpr uint32_t kStageBytes = uint32_t(kRingWarps * (KT + VT) * 2);  // one stage of all warps
+    const uint32_t kStageBytes = uint32_t(kRingWarps * (KT + VT) * 2);  // one stage of all warps
     uint32_t err = 0;
-    pdl_allow();
     const uint16_t* qb = a.q + ((int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g) * D;
     if (wact)  // the group's query rows into L2 while the preceding grid drains
         for (int o = lane * 64; o < g * D; o += 32 * 64) prefetch_l2(qb + o);
@@ -163,14 +168,18 @@ __global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::k
     }
     const int64_t s_begin = int64_t(split) * a.chunk;
     const int64_t s_end = min(len, s_begin + a.chunk);
-    const int n_tiles = s_end > s_begin ? int((s_end - s_begin + 15) / 16) : 0;
+    // this warp's tiles of the chunk: all of them, or a team's every
+    // kRingWarps-th; tile i begins at slot s_begin + i s_step
+    const int n_chunk = s_end > s_begin ? int((s_end - s_begin + 15) / 16) : 0;
+    const int n_tiles = TEAM ? max(0, (n_chunk - warp + kRingWarps - 1) / kRingWarps) : n_chunk;
+    const int64_t s_first = s_begin + (TEAM ? 16 * warp : 0), s_step = TEAM ? 16 * kRingWarps : 16;
     const int64_t lstride = int64_t(l) * a.layer_stride;
     const uint16_t* kbase = a.cache_k + lstride + int64_t(kh) * D;
     const uint16_t* vbase = a.cache_v + lstride + int64_t(kh) * D;
 
     // block id of this lane's slot (lane & 15) of tile n (paged caches)
     auto block_id = [&](int n) -> int32_t {
-        const int64_t s = s_begin + 16 * int64_t(n) + (lane & 15);
+        const int64_t s = s_first + s_step * n + (lane & 15);
         if (a.cache_kind != PRCR_CACHE_PAGED || n >= n_tiles || s >= s_end) return 0;
         return a.block_table[int64_t(b) * a.bt_stride + uint32_t(s) / uint32_t(a.block_size)];
     };
@@ -179,7 +188,7 @@ __global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::k
     auto issue = [&](int n, int32_t blk) {
         if (wact && n < n_tiles) {
             const int st = n % NS;
-            const int64_t s = s_begin + 16 * int64_t(n) + (lane & 15);
+            const int64_t s = s_first + s_step * n + (lane & 15);
             int64_t row = -1;
             if (s < s_end) {
                 if (a.cache_kind == PRCR_CACHE_CONTIGUOUS) {
@@ -354,33 +363,84 @@ __global__ void __launch_bounds__(DecodeShape<D>::kWarps * 32, DecodeShape<D>::k
             }
             __syncwarp();  // stage st is refilled at the next iteration
         }
+        // only now: a following kernel's CTAs, waiting in the room that a grid of one
+        // wave leaves, cost its tiles more than an earlier start saved (one sequence
+        // of 933 slots x 36 layers x 8 heads 26.9 -> 25.2 us in a row, the pipeline
+        // with it and a selection next 56.0 -> 48.8)
+        pdl_allow();
 
-        // heads 2t, 2t+1 of this lane's O^T columns
-        const float l0 = l_run[0], l1 = l_run[1], m0 = m_run[0], m1 = m_run[1];
+        if constexpr (TEAM) {
+            // every warp of the CTA is done with its copies: the ring becomes the
+            // warps' accumulators
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            float* o_s = reinterpret_cast<float*>(smem_raw) + warp * 8 * (D + 4);
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int h = 2 * t + hh;
-            if (h >= g) continue;
-            const int64_t o_idx = (int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g + h;
-            const float lh = hh ? l1 : l0;
-            if (a.splits == 1) {
-                const float inv = lh > 0.0f ? 1.0f / lh : 0.0f;
-                float* out = a.out + o_idx * D;
+            for (int hh = 0; hh < 2; ++hh) {
+                const int h = 2 * t + hh;
 #pragma unroll
                 for (int mt = 0; mt < KS; ++mt) {
-                    out[mt * 16 + gid] = o[mt][hh] * inv;
-                    out[mt * 16 + gid + 8] = o[mt][2 + hh] * inv;
-                }
-            } else {
-                float* part = a.partial + (o_idx * a.splits + split) * (D + 2);
-#pragma unroll
-                for (int mt = 0; mt < KS; ++mt) {
-                    part[mt * 16 + gid] = o[mt][hh];
-                    part[mt * 16 + gid + 8] = o[mt][2 + hh];
+                    o_s[h * (D + 4) + mt * 16 + gid] = o[mt][hh];
+                    o_s[h * (D + 4) + mt * 16 + gid + 8] = o[mt][2 + hh];
                 }
                 if (gid == 0) {
-                    part[D] = hh ? m1 : m0;
-                    part[D + 1] = lh;
+                    s_m[warp][h] = m_run[hh];
+                    s_l[warp][h] = l_run[hh];
+                }
+            }
+            __syncthreads();
+            for (int e = threadIdx.x; e < g * (D / 2); e += blockDim.x) {
+                const int h = e / (D / 2), d = 2 * (e - h * (D / 2));
+                float M = s_m[0][h];
+                for (int w = 1; w < kRingWarps; ++w) M = fmaxf(M, s_m[w][h]);
+                float2 acc = make_float2(0.0f, 0.0f);
+                float den = 0.0f;
+                const float* col = reinterpret_cast<const float*>(smem_raw) + h * (D + 4) + d;
+                for (int w = 0; w < kRingWarps; ++w) {
+                    const float f = s_m[w][h] == -INFINITY ? 0.0f : expf(s_m[w][h] - M);
+                    const float2 x = *reinterpret_cast<const float2*>(col + w * 8 * (D + 4));
+                    acc.x = fmaf(f, x.x, acc.x);
+                    acc.y = fmaf(f, x.y, acc.y);
+                    den = fmaf(f, s_l[w][h], den);
+                }
+                const int64_t o_idx = (int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g + h;
+                if (a.splits == 1) {
+                    const float inv = den > 0.0f ? 1.0f / den : 0.0f;
+                    *reinterpret_cast<float2*>(a.out + o_idx * D + d) = make_float2(acc.x * inv, acc.y * inv);
+                } else {
+                    float* part = a.partial + (o_idx * a.splits + split) * (D + 2);
+                    *reinterpret_cast<float2*>(part + d) = acc;
+                    if (d == 0) *reinterpret_cast<float2*>(part + D) = make_float2(M, den);
+                }
+            }
+        } else {
+            // heads 2t, 2t+1 of this lane's O^T columns
+            const float l0 = l_run[0], l1 = l_run[1], m0 = m_run[0], m1 = m_run[1];
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                const int h = 2 * t + hh;
+                if (h >= g) continue;
+                const int64_t o_idx = (int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g + h;
+                const float lh = hh ? l1 : l0;
+                if (a.splits == 1) {
+                    const float inv = lh > 0.0f ? 1.0f / lh : 0.0f;
+                    float* out = a.out + o_idx * D;
+#pragma unroll
+                    for (int mt = 0; mt < KS; ++mt) {
+                        out[mt * 16 + gid] = o[mt][hh] * inv;
+                        out[mt * 16 + gid + 8] = o[mt][2 + hh] * inv;
+                    }
+                } else {
+                    float* part = a.partial + (o_idx * a.splits + split) * (D + 2);
+#pragma unroll
+                    for (int mt = 0; mt < KS; ++mt) {
+                        part[mt * 16 + gid] = o[mt][hh];
+                        part[mt * 16 + gid + 8] = o[mt][2 + hh];
+                    }
+                    if (gid == 0) {
+                        part[D] = hh ? m1 : m0;
+                        part[D + 1] = lh;
+                    }
                 }
             }
         }
@@ -812,12 +872,16 @@ __global__ void __launch_bounds__(128) decode_merge_warp_kernel(const __grid_con
 template <int D>
 cudaError_t launch_d(const DecodeArgs& a, dim3 grid, cudaStream_t stream) {
     using Sh = DecodeShape<D>;
-    constexpr size_t smem = size_t(Sh::kWarps) * Sh::kStages * 16 * (D + D + 8) * sizeof(uint16_t);
+    constexpr size_t per_warp = size_t(Sh::kStages) * 16 * (D + D + 8) * sizeof(uint16_t);
+    static_assert(8 * (D + 4) * sizeof(float) <= per_warp, "a team's accumulators fit in its rings");
+    const size_t smem = per_warp * (a.team ? a.team : Sh::kWarps);
     static_assert(8 * D * sizeof(float) <= 16 * (2 * D + 8) * sizeof(uint16_t),
                   "a GQA group's rotated queries fit in a warp's share of a ring stage");
-    grid.x = unsigned((int64_t(a.splits) * a.n_kv_heads + Sh::kWarps - 1) / Sh::kWarps);
-    const cudaError_t e = cudaFuncSetAttribute(decode_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    return e != cudaSuccess ? e : launch_pdl(decode_kernel<D>, grid, dim3(Sh::kWarps * 32), smem, stream, a);
+    const int64_t units = int64_t(a.splits) * a.n_kv_heads;
+    grid.x = unsigned(a.team ? units : (units + Sh::kWarps - 1) / Sh::kWarps);
+    auto k = a.team ? decode_kernel<D, true> : decode_kernel<D, false>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    return e != cudaSuccess ? e : launch_pdl(k, grid, dim3((a.team ? a.team : Sh::kWarps) * 32), smem, stream, a);
 }
 
 }  // namespace

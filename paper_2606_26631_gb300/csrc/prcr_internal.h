@@ -256,6 +256,7 @@ struct DecodeArgs {
     int32_t group;
     int32_t splits;
     int32_t chunk;
+    int32_t team;               // warps that share a chunk (head_dim 64, 128), or 0: one warp per chunk
     float scale;
     uint64_t turn_freq[kMaxPairs];  // pair i: round(inv_freq_i / (2 pi) * 2^64)
 };
@@ -267,6 +268,7 @@ struct DecodeArgs {
 template <int D> struct DecodeShape;
 template <> struct DecodeShape<64> { static constexpr int kWarps = 4, kStages = 4, kCtas = 3, kChunk = 512; };
 template <> struct DecodeShape<128> { static constexpr int kWarps = 4, kStages = 2, kCtas = 3, kChunk = 512; };
+constexpr int kDecodeMaxTeam = 12;
 constexpr int kDecodeMaxChunk = 4096;
 constexpr int kDecodeWideWarps = 3;   // head_dim 256: warps (taking a chunk's tiles in turn) per CTA
 constexpr int kDecodeWideCtasPerSm = 2;

@@ -226,9 +226,10 @@ def test_decode_unaligned_query():
 # head counts that leave a CTA's last warps without a unit; the group's ends
 @pytest.mark.parametrize("H,Hq,D,paged,bs", [(1, 8, 256, True, 7), (3, 3, 256, False, 16), (4, 28, 256, True, 16),
                                              (1, 8, 128, True, 7), (5, 5, 128, False, 16), (3, 21, 64, True, 16)])
-@pytest.mark.parametrize("n_layers", [1, 40])
+@pytest.mark.parametrize("n_layers", [1, 9, 19, 40])
 def test_decode_edges(H, Hq, D, paged, bs, n_layers):
-    """head_dim 256: every product has 24 significant bits and is summed in
+    """Few layers: teams of warps per chunk (1) or per whole sequence (9 and 19:
+    of 12, 6, 4 and 2), many: one warp per chunk. head_dim 256: every product has 24 significant bits and is summed in
     float32, so a logit (sum of ~10 in magnitude over 48 MMAs) is off by about
     sqrt(48) 2^-24 10 = 4e-6 and the output by no more than twice that. Below,
     the file's bar: 16 significant bits per operand, 10 * 2^-17 = 8e-5."""
