@@ -460,17 +460,21 @@ __global__ void __launch_bounds__(TEAM ? kDecodeMaxTeam * 32 : DecodeShape<D>::k
 //   PV:  O^T (256 dims x 8 heads) += V^T P^T, 16 m-tiles, as in the kernels above.
 // The float32 query and probabilities enter as three bf16 pieces each (24
 // significant bits, three MMAs), the queries' fragments kept in registers
-// (96), and a tile's P V is summed from zero and added to the running
-// accumulator by the FMA that rescales it, so neither the split nor the tensor
-// core's accumulation costs precision against float32 FMAs.
+// (96). A tensor core truncates what it adds, so the leading pieces' sums are
+// short and start from zero: two k-steps of a logit, one tile of P V, added by
+// float32 adds, and by the FMA that rescales the running accumulator; the other
+// pieces, 2^-8 as large, are summed apart. Error against float64 over 1..16
+// sequences of 64..8192 slots: 1.4e-7 to 2.1e-7 (CUDA-core float32 FMAs 1.8e-7 to
+// 5.1e-7; one chain for a tile's P V and two for a logit's sixteen k-steps 2.0e-7
+// to 2.7e-7, and slower, each MMA waiting for the last: 813 us for the largest
+// below, now 795).
 // What bounds it: DRAM. A tile is 16 KB and ~450 warp instructions; an SM's
 // share of the copy bandwidth brings a tile in ~745 cycles, in which it can
 // issue ~2980. Two CTAs per SM (113 KB of shared memory each) keep six tiles,
 // ~100 KB, in flight per SM and hide each other's prologue. Measured against
 // the CUDA-core kernel it replaced (one warp per KV head, shuffle-reduced dot
 // products, 1.4 TB/s): 16 sequences of up to 4096 slots x 26 layers x 4 KV
-// heads (4.9 GB) 3400 -> 822 us, 6.0 TB/s; one of 933 slots 109 -> 34 us;
-// error against float64 5.2e-7 -> 2.7e-7.
+// heads (4.9 GB) 3400 -> 795 us, 6.2 TB/s; one of 933 slots 109 -> 29 us.
 constexpr int kWideWarps = kDecodeWideWarps;
 constexpr int kWideD = 256;
 constexpr int kWidePitch = kWideD + 8;           // bf16 per staged row
@@ -518,7 +522,6 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
     const uint32_t wk_s = uint32_t(__cvta_generic_to_shared(ring + size_t(warp) * 2 * kWideTile));
     constexpr uint32_t kStageBytes = uint32_t(kWideSmem / 2), kTileBytes = uint32_t(kWideTile * 2);
     uint32_t err = 0;
-    pdl_allow();
     pdl_wait();
     const int64_t p = a.q_pos[b];
     int64_t len = a.seq_len[b];
@@ -633,14 +636,21 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
         asm volatile("cp.async.commit_group;" ::: "memory");
 
         const uint32_t base = wk_s + uint32_t(st) * kStageBytes;
-        float c[4][4];
+        float c[4][4], y[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) c[u][0] = c[u][1] = c[u][2] = c[u][3] = 0.0f;
 #pragma unroll
         for (int j = 0; j < KS; ++j) {
             uint32_t r[4];
             ldmatrix_x4(base + k_ld + uint32_t(j * 32), r);
-            mma_16816(c[j & 1], r[0], r[1], r[2], r[3], qf[j][0][0], qf[j][0][1]);
+            if (j & 1) {
+                mma_16816(y, r[0], r[1], r[2], r[3], qf[j][0][0], qf[j][0][1]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[(j >> 1) & 1][u] += y[u];
+            } else {
+                y[0] = y[1] = y[2] = y[3] = 0.0f;
+                mma_16816(y, r[0], r[1], r[2], r[3], qf[j][0][0], qf[j][0][1]);
+            }
             mma_16816(c[2], r[0], r[1], r[2], r[3], qf[j][1][0], qf[j][1][1]);
             mma_16816(c[3], r[0], r[1], r[2], r[3], qf[j][2][0], qf[j][2][1]);
         }
@@ -683,10 +693,12 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
         for (int mt = 0; mt < KS; ++mt) {
             uint32_t r[4];
             ldmatrix_x4_trans(base + v_ld + uint32_t(mt * 32), r);
-            float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            mma_16816(x, r[0], r[1], r[2], r[3], pf[2][0], pf[2][1]);
-            mma_16816(x, r[0], r[1], r[2], r[3], pf[1][0], pf[1][1]);
+            float x[4] = {0.0f, 0.0f, 0.0f, 0.0f}, xl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            mma_16816(xl, r[0], r[1], r[2], r[3], pf[2][0], pf[2][1]);
+            mma_16816(xl, r[0], r[1], r[2], r[3], pf[1][0], pf[1][1]);
             mma_16816(x, r[0], r[1], r[2], r[3], pf[0][0], pf[0][1]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] += xl[u];
             o[mt][0] = fmaf(o[mt][0], alpha[0], x[0]);
             o[mt][1] = fmaf(o[mt][1], alpha[1], x[1]);
             o[mt][2] = fmaf(o[mt][2], alpha[0], x[2]);
@@ -694,6 +706,7 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
         }
     }
 
+    pdl_allow();  // late, as in decode_kernel
     // merge the warps (the ring is free: no copy is in flight past a warp's last tile)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
