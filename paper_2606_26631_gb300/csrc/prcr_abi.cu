@@ -268,6 +268,14 @@ int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     a.plan_dst = pv.dst;
     a.plan_pos = pv.pos;
     a.status = o->status;
+    a.idx = b->idx;
+    a.rev_tok_off = b->rev_tok_off;
+    a.seq_rev_off = b->seq_rev_off;
+    a.store_seq_stride = store->seq_stride;
+    a.store_token_stride = store->token_stride;
+    a.n_seqs = b->n_seqs;
+    a.n_revisits = b->n_revisits;
+    a.n_tokens = store->n_tokens;
     a.total_k = b->total_k;
     a.n_layers = cfg->n_layers;
     a.head_dim = cfg->head_dim;
@@ -296,6 +304,7 @@ int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                                    : stream_layers_per_cta(tiles, cfg->n_layers, slots, 4, 12);
     const int64_t groups = (cfg->n_layers + G - 1) / G;
     a.layers_per_cta = G;
+    a.early_ctas = int32_t(slots);
     if (tiles > INT32_MAX) return PRCR_EINVAL;
     grid = dim3(unsigned(tiles), unsigned(groups), 1);
     return PRCR_OK;

@@ -164,6 +164,16 @@ struct RebindArgs {
     const int64_t* plan_dst;
     const double* plan_pos;
     const uint32_t* status;
+    // the batch, from which the first wave's rows are prefetched during the plan
+    const int32_t* idx;
+    const int32_t* rev_tok_off;
+    const int32_t* seq_rev_off;
+    int64_t store_seq_stride;
+    int64_t store_token_stride;
+    int32_t n_seqs;
+    int32_t n_revisits;
+    int32_t n_tokens;
+    int32_t early_ctas;      // CTAs of the first wave
     int64_t total_k;
     int32_t n_layers;
     int32_t head_dim;
@@ -339,8 +349,7 @@ int check_revisit_args(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                        const prcr_outputs* o, int32_t mode, int32_t L, int32_t flags);
 
 cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
-// the logits of the cached-key selection, then the same normaliser, relevance
-// and selection kernels
+// the logits of the cached-key selection, then the same tail
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
 
 // the whole selection in one kernel, where that is the faster path (else

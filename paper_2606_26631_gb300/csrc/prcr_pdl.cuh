@@ -2,7 +2,9 @@
 //
 // Every kernel of the revisit path is launched with programmatic stream
 // serialization. It allows its dependents at entry, so the next kernel's CTAs
-// may be launched as soon as every CTA of this grid is resident. Before its
+// may be launched as soon as every CTA of this grid is resident, or, where those
+// CTAs would slow a grid of one wave by waiting beside it (the decode and fused
+// revisit kernels say by how much), late in its work. Before its
 // first global load or store it waits for the grid it depends on to complete
 // and its writes to be visible. Only L2 prefetches, which return nothing to
 // the thread, go before that wait. A kernel whose predecessor is not one of

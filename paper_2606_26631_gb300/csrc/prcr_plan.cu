@@ -167,10 +167,11 @@ __device__ void plan_revisit(const PlanArgs& a, int r, int* s_part, double (*s_t
 }
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constant__ PlanArgs a) {
-    // The rebind grid may start launching now; it waits for this grid to
-    // finish (griddepcontrol.wait) before it reads the plan.
-    pdl_allow();
+    // The rebind grid may start launching now, when the batch it prefetches rows
+    // by is there; it waits for this grid to finish (griddepcontrol.wait)
+    // before it reads the plan.
     pdl_wait();
+    pdl_allow();
     __shared__ int s_part[33 * 6];
     __shared__ double s_tab[3][kPosTable];
     uint32_t err = 0;

@@ -25,16 +25,47 @@
 // layer ahead of the one stored instead (72 registers): 97 us for the second.
 //
 // The kernel is launched with programmatic dependent launch behind the plan
-// kernel and waits on it (griddepcontrol.wait) before touching the plan.
+// kernel and waits on it (griddepcontrol.wait) before touching the plan; its
+// first rows are prefetched into L2 meanwhile (prefetch_rows).
 #include "prcr_device.cuh"
 #include "prcr_pdl.cuh"
 
 namespace prcr {
 namespace {
 
+constexpr int kEarlyLayers = 4;
+
+// The raw rows of the CTA's tokens (its first kEarlyLayers layers) into L2 while
+// the plan kernel runs. Hints only: nothing read here is used for anything else,
+// so indices or offsets that are wrong, or not written yet, cost time alone; what
+// is prefetched lies in the store whatever they hold. The plan takes ~8 us,
+// of which the lookups here leave a few. Only the first wave's CTAs are there by
+// then. Measured (calls in a row, without | 2 layers | 4 | 12): 3 x 267 tokens x 8
+// layers x 8 heads of 128 32.2 | 31.9 | 31.1 | 31.1 us, 5 x 443 x 32 x 5 41.2 | 40.6
+// | 39.9 | 39.9, 12 x 201 x 11 x 5 of 256 49.9 | 49.9 | 49.0 | 49.0, 8 x ~512 x 28
+// x 4 81.6 | 82.1 | 81.5 | 81.5.
+__device__ __forceinline__ void prefetch_rows(const RebindArgs& a) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = int(blockDim.x + 31) >> 5;
+    if ((blockDim.x & 31) && warp == nw - 1) return;  // a part of a warp
+    const int l = int(blockIdx.y) * a.layers_per_cta + (lane >> 1);
+    const int n = min(kEarlyLayers, a.layers_per_cta);
+    const uint32_t bytes = uint32_t(a.lanes) * 32;  // of a row
+    for (int t = warp; t < a.tok_per_cta; t += nw) {
+        const int64_t j = int64_t(blockIdx.x) * a.tok_per_cta + t;
+        if (j >= a.total_k) break;
+        const int m = a.idx[j];
+        const int b = sequence_of(a.seq_rev_off, a.n_seqs, sequence_of(a.rev_tok_off, a.n_revisits, int(j)));
+        if (m < 0 || m >= a.n_tokens || (lane >> 1) >= n || l >= a.n_layers) continue;
+        const uint16_t* row = (lane & 1 ? a.store_v : a.store_k) + b * a.store_seq_stride +
+                              int64_t(l) * a.store_layer_stride + int64_t(m) * a.store_token_stride;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row), "r"(bytes) : "memory");
+    }
+}
+
 __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ RebindArgs a) {
     extern __shared__ __align__(16) float smem[];
     pdl_allow();
+    if (int64_t(blockIdx.y) * gridDim.x + blockIdx.x < a.early_ctas) prefetch_rows(a);
     pdl_wait();
     if (*reinterpret_cast<const volatile uint32_t*>(a.status) & PRCR_ST_CSR) return;
 
