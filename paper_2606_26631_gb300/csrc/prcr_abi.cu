@@ -411,14 +411,19 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
 //   of 6000 28.7 -> 21.3; 2 x 10 x 8 of up to 1500 29.0 -> 26.9).
 // - Several sequences' lengths differ, so where a team's warps would have more
 //   than 2 kChunk slots (a warp by itself 1.25 kChunk) the batch is a large one:
-//   8 x 28 x 4 of up to 4096 would take 222 us with teams of two, not 207; of up
-//   to 2000 it takes 110, not 123. One sequence has no such limit: 1 x 36 x 8 of
-//   4096 slots 113 -> 94, of 16384 383 -> 366.
-// Large batches: one warp per chunk of kChunk slots, many waves of which even
-// out lengths that differ. Measured at chunks of 384, 512, 768, 1024 and 1536
-// slots: 8 sequences x 28 layers x 4 heads of up to 4096 slots 218, 208, 209,
-// 232, 219 us; 16 x 36 x 8 912, 895, 896, 886, 900; head_dim 64, 8 x 28 x 3 102,
-// 96, 122, 95, 127.
+//   8 x 28 x 4 of up to 4096 would take 222 us with teams of two, not 200; 5 x 28
+//   x 4 of up to 3000 takes 114 with teams of three, 124 as a large batch. One
+//   sequence has no such limit: 1 x 36 x 8 of 4096 slots 113 -> 94, of 16384 383
+//   -> 366.
+// Large batches: many waves, which even out lengths that differ. head_dim 128:
+// teams of four on equal chunks of at most 4 kChunk slots, a quarter of the
+// partials to merge that one warp per chunk of kChunk has. Measured (us, one warp
+// on 512 | teams of four on 768 | 1024 | 1536 | 2048 slots): 8 sequences x 28
+// layers x 4 heads of up to 4096 slots 205 | 213 | 208 | 208 | 200, of up to 8192
+// 404 | 404 | 394 | 384 | 390, 6 of up to 4096 180 | 175 | 169 | 169 | 166; 16 x 36
+// x 8 of up to 4096 851 | 856 | 833 | 828 | 826; 16 x 28 x 4 of up to 900 103 | 94;
+// teams of six and twelve 174 and 169 for the third. head_dim 64: one warp on 512
+// (8 x 28 x 4 of up to 4096 110 us, teams 114; 12 x 28 x 8 326, 333).
 template <int D>
 int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, int* team,
                      int64_t* most) {
@@ -448,9 +453,11 @@ int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, in
     const int64_t share = splits * std::max(1, *team);
     if ((*team <= 1 || n_seqs > 1) &&
         (max_len + share - 1) / share > Sh::kChunk * (*team > 1 ? 2 : 1.25)) {
-        *team = 0;
-        *most = std::max(*most, (max_len + Sh::kChunk - 1) / Sh::kChunk);
-        return Sh::kChunk;
+        *team = Sh::kLargeTeam;
+        const int64_t longest = Sh::kChunk * std::max(1, *team);
+        splits = (max_len + longest - 1) / longest;
+        *most = std::max(*most, splits);
+        return *team ? (tiles + splits - 1) / splits * 16 : longest;
     }
     // the fewest warps that take as many rounds of tiles
     const int64_t per = (tiles + splits - 1) / splits;

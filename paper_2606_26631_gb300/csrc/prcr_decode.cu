@@ -72,12 +72,11 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
 // DRAM bounds it: an SM's 12 warps keep ~100 KB in flight (~2.2 us at its share
 // of the copy rate). Measured, before | now (before: a CTA looping over the KV
 // heads with K in registers for large batches, CTAs of four heads each for
-// small ones): 16 sequences x 36 layers x 8 heads of up to 4096 slots 925 | 893
-// us (6.5 TB/s), 8 x 28 x 4 214 | 207, 11 x 24 x 5 of up to 6900 573 | 453, 5 x
-// 36 x 8 of up to 3500 346 | 308, 14 x 2 x 1 head of up to 7132 37.6 | 19.9; head_dim
-// 64: 12 x 28 x 8 275 | 223, 1 x 28 x 4 31.7 | 25.3. 8 x 28 x 4 of up to 3000
-// slots went 166 -> 171: its 512-slot chunks end in a short last wave. Equal
-// static runs of tiles per warp instead of chunks: 229 us for the second.
+// small ones): 16 sequences x 36 layers x 8 heads of up to 4096 slots 890 | 826
+// us, 8 x 28 x 4 212 | 200, 11 x 24 x 5 of up to 6900 554 | 423, 5 x 36 x 8 of up
+// to 3500 329 | 287, 14 x 2 x 1 head of up to 7132 37.6 | 19.9; head_dim 64: 12 x
+// 28 x 8 275 | 223, 1 x 28 x 4 31.7 | 25.3. Equal static runs of tiles per warp
+// instead of chunks: 229 us for the second.
 template <int D, bool TEAM>
 __global__ void __launch_bounds__(TEAM ? kDecodeMaxTeam * 32 : DecodeShape<D>::kWarps * 32, TEAM ? 1 : DecodeShape<D>::kCtas)
     decode_kernel(const __grid_constant__ DecodeArgs a) {

@@ -273,11 +273,11 @@ struct DecodeArgs {
 
 // Shape of the decode kernel at head_dim 64 and 128: warps per CTA, stages of a
 // warp's ring and CTAs per SM (shared memory and registers bound them; copies in
-// flight per SM: 12 warps x 3 tiles x 4.3 KB, 12 x 8.4 KB), and slots of a
-// chunk of a large batch.
+// flight per SM: 12 warps x 3 tiles x 4.3 KB, 12 x 8.4 KB), slots of a
+// chunk per warp of a large batch, and the warps of its teams (0: none).
 template <int D> struct DecodeShape;
-template <> struct DecodeShape<64> { static constexpr int kWarps = 4, kStages = 4, kCtas = 3, kChunk = 512; };
-template <> struct DecodeShape<128> { static constexpr int kWarps = 4, kStages = 2, kCtas = 3, kChunk = 512; };
+template <> struct DecodeShape<64> { static constexpr int kWarps = 4, kStages = 4, kCtas = 3, kChunk = 512, kLargeTeam = 0; };
+template <> struct DecodeShape<128> { static constexpr int kWarps = 4, kStages = 2, kCtas = 3, kChunk = 512, kLargeTeam = 4; };
 constexpr int kDecodeMaxTeam = 12;
 constexpr int kDecodeMaxChunk = 4096;
 constexpr int kDecodeWideWarps = 3;   // head_dim 256: warps (taking a chunk's tiles in turn) per CTA
