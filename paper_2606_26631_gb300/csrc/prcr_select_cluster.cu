@@ -614,7 +614,7 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
             const bool more = it + NW < n_items;
             if (more) rows((it + NW) / H, (it + NW) % H, r_n);
             constexpr int NC = CACHED ? 4 : 2;  // accumulator chains per head
-            float acc[NC][4];
+            float acc[NC][4], lead[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int u = 0; u < NC; ++u) acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.0f;
             const uint4* qf = qf_s + kh * KQ * 32 + lane;
@@ -655,9 +655,25 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
                                                      make_float2(-1.0f, -1.0f), Yr);
                         const uint4 q2 = qf[(4 * u + w) * 32];
                         const uint32_t b0 = up ? q2.z : q2.x, b1 = up ? q2.w : q2.y;
+                        // head_dim 256: remainders rounded (half a tf32 unit added) and, the
+                        // tensor core truncating what it adds, the leading chain cut every
+                        // two k-steps and added with its rounding error kept (Knuth's
+                        // two-sum). Error against float64 0.8e-7 to 1.5e-7, of one chain 2.7e-7
+                        // to 7e-7 (float32 FMAs on the CUDA cores 1.1e-7 to 1.7e-7); 13
+                        // sequences of 456 tokens x 8 heads 15.9 -> 17.4 us (CUDA cores 48.8).
+                        constexpr uint32_t kHalf = D == 256 ? 0x1000u : 0u;
                         mma_1688_tf32(acc[0], hxa, hxb, hya, hyb, b0, b1);
-                        mma_1688_tf32(acc[1], __float_as_uint(lx.x), __float_as_uint(lx.y), __float_as_uint(ly.x),
-                                      __float_as_uint(ly.y), b0, b1);
+                        mma_1688_tf32(acc[1], __float_as_uint(lx.x) + kHalf, __float_as_uint(lx.y) + kHalf, __float_as_uint(ly.x) + kHalf,
+                                      __float_as_uint(ly.y) + kHalf, b0, b1);
+                        if (D == 256 && s8 % 2 == 1) {
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) {
+                                const float sum = lead[v] + acc[0][v], part = sum - lead[v];
+                                acc[1][v] += (lead[v] - (sum - part)) + (acc[0][v] - part);
+                                lead[v] = sum;
+                                acc[0][v] = 0.0f;
+                            }
+                        }
                     }
                     if (more) fetch(k[u], r_n[0], r_n[1], u);
                 }
@@ -676,9 +692,9 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
                 if constexpr (CACHED) {  // chains 1 and 3: the query's remainder
                     va = (acc[1][c] + acc[NC - 1][c]) + (acc[0][c] + acc[NC - 2][c]);
                     vb = (acc[1][2 + c] + acc[NC - 1][2 + c]) + (acc[0][2 + c] + acc[NC - 2][2 + c]);
-                } else {  // chain 1: the keys' remainders
-                    va = (acc[0][c] + acc[1][c]) * a.scale;
-                    vb = (acc[0][2 + c] + acc[1][2 + c]) * a.scale;
+                } else {  // chain 1: the keys' remainders (and lead's rounding errors)
+                    va = ((D == 256 ? lead[c] : acc[0][c]) + acc[1][c]) * a.scale;
+                    vb = ((D == 256 ? lead[2 + c] : acc[0][2 + c]) + acc[1][2 + c]) * a.scale;
                 }
                 float* dst = lg + (kh * g + 2 * tq + c) * lg_pitch;
                 if (ta < nt) dst[ta] = ok_a ? va : -INFINITY;
@@ -730,8 +746,8 @@ __device__ __forceinline__ void cta_stats(const float* lg_s, int pitch, int Hq, 
 // launches: 768 tokens x 8 KV heads in a cluster of 16, ~20k cycles: queries
 // and first rows 2.7k, cos/sin and MMAs 5.5k, statistics and their exchange
 // 4.8k, relevances and theirs 5k, search and output 2.7k. Measured with its
-// launches 20.9 -> 12.5 us (four kernels before), 8 sequences 20.6 -> 13.6 us,
-// 4 of 1000 tokens at head_dim 256 29.6 -> 13.9 us (CUDA cores before).
+// launches 20.9 -> 11.5 us (four kernels before), 8 sequences 20.1 -> 13.1 us,
+// 4 of 1000 tokens at head_dim 256 29.7 -> 14.7 us (CUDA cores before).
 constexpr int kFusedThreads = 512;
 
 template <int D, bool CACHED>
