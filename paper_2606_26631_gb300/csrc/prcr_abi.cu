@@ -88,6 +88,20 @@ int check_cache(const prcr_rope_cfg* c, const prcr_cache_desc* k) {
 
 }  // namespace
 
+cudaError_t raise_smem_limit(const void* kernel, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> limits;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> g(mu);
+    size_t& have = limits[std::make_pair(dev, kernel)];
+    if (have >= smem) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e == cudaSuccess) have = smem;
+    return e;
+}
+
 // Every check of a revisit call except the workspace's.
 int check_revisit_args(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                        const prcr_cache_desc* cache, const prcr_revisit_batch* b,

@@ -892,7 +892,7 @@ cudaError_t launch_d(const DecodeArgs& a, dim3 grid, cudaStream_t stream) {
     const int64_t units = int64_t(a.splits) * a.n_kv_heads;
     grid.x = unsigned(a.team ? units : (units + Sh::kWarps - 1) / Sh::kWarps);
     auto k = a.team ? decode_kernel<D, true> : decode_kernel<D, false>;
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k), smem);
     return e != cudaSuccess ? e : launch_pdl(k, grid, dim3((a.team ? a.team : Sh::kWarps) * 32), smem, stream, a);
 }
 
@@ -908,8 +908,7 @@ cudaError_t launch_decode(const DecodeArgs& a, dim3 grid, cudaStream_t stream) {
         // head_dim 256: one KV head per CTA
         dim3 g2 = grid;
         g2.x *= unsigned(a.n_kv_heads);
-        e = cudaFuncSetAttribute(decode_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(kWideSmem));
+        e = raise_smem_limit(reinterpret_cast<const void*>(decode_wide_kernel), kWideSmem);
         if (e == cudaSuccess) e = launch_pdl(decode_wide_kernel, g2, dim3(kWideWarps * 32), kWideSmem, stream, a);
     }
     if (e != cudaSuccess || a.splits == 1) return e;

@@ -22,8 +22,6 @@
 //   E. the rows already in registers are rotated and stored, and the
 //      group's other layers streamed as in the rebind kernel.
 // Results are bit-identical to plan + rebind.
-#include <map>
-#include <mutex>
 
 #include "prcr_device.cuh"
 #include "prcr_pdl.cuh"
@@ -404,34 +402,17 @@ __global__ void __launch_bounds__(512) fused_kernel(const __grid_constant__ Fuse
     }
 }
 
-// The kernel's dynamic shared-memory limit raised to `smem` on the current
-// device (once per device and size: the attribute is set only when a larger
-// size is first needed).
-cudaError_t fused_smem_limit(size_t smem) {
-    static std::mutex mu;
-    static std::map<int, size_t> done;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> g(mu);
-    size_t& have = done[dev];
-    if (have >= smem) return cudaSuccess;
-    e = cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e == cudaSuccess) have = smem;
-    return e;
-}
-
 }  // namespace
 
 cudaError_t fused_blocks_per_sm(int block, size_t smem, int* out) {
-    const cudaError_t e = fused_smem_limit(smem);
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(fused_kernel), smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, fused_kernel, block, smem);
 }
 
 cudaError_t launch_fused(const FusedArgs& a, dim3 grid, int block, size_t smem,
                          cudaStream_t stream) {
-    const cudaError_t e = fused_smem_limit(smem);
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(fused_kernel), smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(fused_kernel, grid, dim3(block), smem, stream, a);
 }

@@ -360,6 +360,11 @@ cudaError_t launch_select_cached_logits(const SelectArgs& a, int n_seqs, int sms
 // the steps after the logits: normalisers, relevances, top-k
 cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream);
 
+// The dynamic shared-memory limit of a kernel on the current device, raised to
+// `smem` where it is lower. It belongs to the kernel, not to a launch, so it is
+// never lowered: another thread may be about to launch with the larger one.
+cudaError_t raise_smem_limit(const void* kernel, size_t smem);
+
 cudaError_t launch_decode(const DecodeArgs& a, dim3 grid, cudaStream_t stream);
 cudaError_t launch_capture(const CaptureArgs& a, dim3 grid, int block, size_t smem,
                            cudaStream_t stream);

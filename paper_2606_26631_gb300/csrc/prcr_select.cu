@@ -486,8 +486,7 @@ size_t select_logits_smem(const SelectArgs& a) {
 template <int L, int G>
 cudaError_t launch_logits_g(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
     const size_t smem = select_logits_smem(a);
-    cudaError_t e = cudaFuncSetAttribute(ads_logits_kernel<L, G>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(ads_logits_kernel<L, G>), smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ads_logits_kernel<L, G>, 256, smem);
@@ -522,7 +521,7 @@ cudaError_t launch_logits_mma(const SelectArgs& a, int n_seqs, int sms, cudaStre
     SelectArgs b = a;
     b.kh_per_item = H < 8 ? H : 8;  // KV heads per work item (sizes the query fragments)
     const size_t smem_max = logits_mma_smem<D>(b.kh_per_item);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem_max));
+    cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(kern), smem_max);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMmaWarps * 32, smem_max);

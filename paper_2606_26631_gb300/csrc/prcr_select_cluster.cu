@@ -953,7 +953,7 @@ cudaError_t launch_logits_split(const SelectArgs& a, int n_seqs, int sms, cudaSt
     const size_t smem = fused_layout(D, true, t.kh_per_item, t.kh_per_item * g, t.tok_per_cta, 0, false).total;
     const int64_t grid = per * ((a.n_tokens + t.tok_per_cta - 1) / t.tok_per_cta);
     if (grid > INT32_MAX) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(select_logits_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(select_logits_kernel<D>), smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(select_logits_kernel<D>, dim3(unsigned(grid)), dim3(kSplitThreads), smem, stream, t);
 }

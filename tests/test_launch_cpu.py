@@ -1,0 +1,42 @@
+"""CPU checks of what the host side launches, against a CUDA runtime that only
+keeps the launches (fake_gpu)."""
+import ctypes as C
+import threading
+
+import pytest
+
+import fake_gpu as F
+
+
+def test_shared_memory_limits_only_rise():
+    """The limit belongs to the kernel, not to the call: a call that lowers it
+    fails another thread's launch. Calls of one kernel with different needs
+    (decode teams of 12, 6, 4, 3 and 2 warps, one warp per chunk and head_dim
+    256; cached and raw selections past one cluster), from several threads."""
+    b8, b256, small = F.cfg(36, 8, 128), F.cfg(26, 4, 256), F.cfg(2, 4, 128)
+    calls = [(lambda c=c, n=n, m=m: F.decode(c, n, 4, m, 1 << 40)) for c in (small, b8, b256) for n, m in ((1, 200), (1, 933), (3, 933), (16, 300), (16, 8192))]
+    calls += [(lambda H=H, D=D, n=n, m=m: F.select_cached(F.cfg(1, H, D), n, 4, m))
+              for H, D in ((8, 128), (2, 128)) for n, m in ((1, 32768), (4, 16384), (32, 8192))]
+    calls += [(lambda H=H, D=D, n=n: F.select_raw(F.cfg(1, H, D), n, 4, 16384))
+              for H, D in ((8, 128), (2, 128), (2, 96), (8, 96), (4, 256)) for n in (1, 32)]
+    F.lib()
+    bad, done = [], []
+
+    def work(first):
+        for i in range(3 * len(calls)):
+            which = (i + first) % len(calls)
+            rc = calls[which]()
+            if rc:
+                bad.append((which, rc))
+        done.append(first)
+
+    threads = [threading.Thread(target=work, args=(7 * t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    names = {n for n, _ in F.launches()}
+    for part in ("decode_kernelILi128ELb1E", "decode_kernelILi128ELb0E", "decode_wide", "select_logits", "ads_logits_mma", "ads_logits_kernel"):
+        assert any(part in n for n in names), part
+    assert not bad and len(done) == len(threads), bad[:5]
+    assert F.lib().fake_lowered() == 0
