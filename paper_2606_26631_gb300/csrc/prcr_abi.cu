@@ -483,29 +483,35 @@ int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, in
 
 // head_dim 256: one KV head per CTA, about 8 waves of kDecodeWideCtasPerSm
 // CTAs per SM with chunks of at least kWideMinChunk slots; where that is less
-// than two waves, one wave. Chunks are whole rounds of the CTA's warps.
+// than two waves, one wave. Chunks are whole rounds of the CTA's warps, so a
+// longer max_len may be split into fewer; *most bounds what any up to it is.
 // Measured: 16 sequences x 26 layers x 4 heads of up to 4096 slots 822 us at 8
 // waves, 852 us at 16; 4 sequences of up to 2000 slots 162 us at 576 slots,
 // 178 us at 384.
 constexpr int64_t kWideMinChunk = 576;
-int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms) {
-    const int64_t resident = int64_t(sms) * kDecodeWideCtasPerSm, round = 16 * kDecodeWideWarps;
-    const bool few = units * ((max_len + kWideMinChunk - 1) / kWideMinChunk) < 2 * resident;
-    const int64_t want = std::max<int64_t>(1, few ? resident / units : (8 * resident + units - 1) / units);
-    int64_t c = (max_len + want - 1) / want;
+int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms, int64_t* most) {
+    constexpr int64_t round = 16 * kDecodeWideWarps, longest = kDecodeMaxChunk / round * round;
+    static_assert(kWideMinChunk % round == 0, "whole rounds");
+    auto ceil_div = [](int64_t x, int64_t y) { return (x + y - 1) / y; };
+    const int64_t resident = int64_t(sms) * kDecodeWideCtasPerSm;
+    const int64_t one_wave = std::max<int64_t>(1, resident / units), waves = ceil_div(8 * resident, units);
+    // the lengths up to this one are split for one wave
+    const int64_t few_len = (2 * resident - 1) / units * kWideMinChunk;
+    const bool few = max_len <= few_len;
+    *most = std::max(std::min(one_wave, ceil_div(std::min(max_len, few_len), round)), ceil_div(max_len, longest));
+    if (!few) *most = std::max(*most, std::min(waves, ceil_div(max_len, kWideMinChunk)));
+    int64_t c = ceil_div(max_len, few ? one_wave : waves);
     if (!few && c < kWideMinChunk) c = kWideMinChunk;
-    c = (c + round - 1) / round * round;
-    return std::min<int64_t>(c, kDecodeMaxChunk / round * round);
+    return std::min(ceil_div(c, round) * round, longest);
 }
 
 void decode_split(int64_t n_seqs, int n_layers, int64_t max_len, int sms, int n_kv_heads,
                   int head_dim, int* splits, int* chunk, int* team, int64_t* most) {
     const int64_t units = n_seqs * n_layers * n_kv_heads;
     *team = 0;
-    *most = 1;
     const int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, team, most)
                       : head_dim == 128 ? decode_chunk<128>(n_seqs, units, max_len, sms, team, most)
-                                        : decode_wide_chunk(units, max_len, sms);
+                                        : decode_wide_chunk(units, max_len, sms, most);
     *chunk = int(c);
     *splits = int((max_len + c - 1) / c);
     *most = std::max<int64_t>(*most, *splits);

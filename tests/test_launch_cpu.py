@@ -40,3 +40,29 @@ def test_shared_memory_limits_only_rise():
         assert any(part in n for n in names), part
     assert not bad and len(done) == len(threads), bad[:5]
     assert F.lib().fake_lowered() == 0
+
+
+@pytest.mark.parametrize("D", [64, 128, 256])
+def test_decode_workspace_holds_shorter_calls(D):
+    """A workspace sized once, for the longest length, is enough for every
+    shorter one: no length needs more chunks than the size for it holds, and
+    sizes fall nowhere as max_len grows. Lengths around the rules' lines."""
+    for layers, H in ((1, 1), (1, 4), (2, 4), (4, 1), (26, 4), (36, 8), (3, 3)):
+        c = F.cfg(layers, H, D)
+        for seqs in (1, 2, 5, 16):
+            unit = seqs * layers * H * (D + 2) * 4  # one head per KV head
+            lengths = sorted({*range(1, 700, 7), *range(1, 40000, 391), *(m * e + d for m in (16, 48, 512, 576, 640, 2048, 4080, 4096)
+                                                                       for e in (1, 2, 3, 9, 38, 76) for d in (-1, 0, 1)), 30000, 200000})
+            before = 0
+            for n in lengths:
+                size = F.workspace(c, seqs, 1, n)
+                assert size >= before, (layers, H, seqs, n)
+                before = size
+                F.launches()
+                assert F.decode(c, seqs, 1, n, 1 << 40) == 0
+                splits = F.launches()[0][1][5]
+                assert size >= (unit * splits if splits > 1 else 0), (layers, H, seqs, n, splits)
+    # the calls that were refused: (layers, KV heads, sequences, longest, shorter)
+    for layers, H, seqs, longest, shorter in ((1, 4, 1, 3649, 3601), (2, 4, 1, 1825, 1777), (1, 4, 5, 721, 673), (1, 1, 2, 7297, 7249)):
+        c = F.cfg(layers, H, D)
+        assert F.decode(c, seqs, 2, shorter, F.workspace(c, seqs, 2, longest)) == 0
