@@ -18,8 +18,9 @@
  *    (a cudaStream_t; NULL = the legacy default stream) and runs
  *    asynchronously. Kernels are launched with programmatic stream
  *    serialization: one may become resident while the preceding kernel on
- *    the stream drains, but it reads and writes no memory before that
- *    kernel has completed, so stream order is exactly that of plain launches.
+ *    the stream drains, but a call reads and writes no memory before the
+ *    kernels that precede the call have completed, so stream order is exactly
+ *    that of plain launches.
  *  - K/V elements are bf16 (IEEE binary16-brain bit patterns). A token row is
  *    [n_kv_heads][head_dim] contiguous elements; strides between rows,
  *    layers, sequences and blocks are given in elements. Every row start must

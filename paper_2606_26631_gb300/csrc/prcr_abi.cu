@@ -266,10 +266,13 @@ int stream_layers_per_cta(int64_t tiles, int n_layers, int64_t slots, int few, i
 }
 
 // Arguments and launch shape of the row-moving kernel (rebind or fused).
+// after_plan: this call's own plan kernel precedes it, which releases it only
+// when everything before the call is done; only then may it look at the batch
+// before its wait.
 int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                  const prcr_cache_desc* cache, const prcr_revisit_batch* b, const prcr_outputs* o,
                  void* ws, RebindArgs& a, dim3& grid, int& block, size_t& smem,
-                 KernelId kernel = kRebind) {
+                 KernelId kernel, bool after_plan) {
     a = RebindArgs{};
     a.store_k = static_cast<const uint16_t*>(store->k);
     a.store_v = static_cast<const uint16_t*>(store->v);
@@ -318,7 +321,7 @@ int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                                    : stream_layers_per_cta(tiles, cfg->n_layers, slots, 4, 12);
     const int64_t groups = (cfg->n_layers + G - 1) / G;
     a.layers_per_cta = G;
-    a.early_ctas = int32_t(slots);
+    a.early_ctas = after_plan ? int32_t(slots) : 0;
     if (tiles > INT32_MAX) return PRCR_EINVAL;
     grid = dim3(unsigned(tiles), unsigned(groups), 1);
     return PRCR_OK;
@@ -326,13 +329,13 @@ int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
 
 int do_rebind(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
               const prcr_cache_desc* cache, const prcr_revisit_batch* b, const prcr_outputs* o,
-              void* ws, cudaStream_t stream) {
+              void* ws, bool after_plan, cudaStream_t stream) {
     if (b->total_k == 0) return PRCR_OK;
     RebindArgs a;
     dim3 grid;
     int block = 0;
     size_t smem = 0;
-    const int rc = rebind_setup(cfg, store, cache, b, o, ws, a, grid, block, smem);
+    const int rc = rebind_setup(cfg, store, cache, b, o, ws, a, grid, block, smem, kRebind, after_plan);
     if (rc) return rc;
     return launch_rebind(a, grid, block, smem, stream) == cudaSuccess ? PRCR_OK : PRCR_ECUDA;
 }
@@ -596,7 +599,7 @@ int prcr_rebind_apply(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
                       void* workspace, size_t workspace_bytes, void* stream) {
     int rc = check_call(cfg, store, cache, batch, out, mode, L, flags, workspace, workspace_bytes);
     if (rc || batch->n_seqs == 0) return rc;
-    return do_rebind(cfg, store, cache, batch, out, workspace, static_cast<cudaStream_t>(stream));
+    return do_rebind(cfg, store, cache, batch, out, workspace, false, static_cast<cudaStream_t>(stream));
 }
 
 int prcr_rebind_inject(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
@@ -616,7 +619,7 @@ int prcr_rebind_inject(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
         int block = 0;
         size_t smem = 0;
         rc = rebind_setup(cfg, store, cache, batch, out, workspace, fa.rebind, grid, block, smem,
-                          kFused);
+                          kFused, false);
         if (rc) return rc;
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
@@ -630,7 +633,7 @@ int prcr_rebind_inject(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     }
     rc = do_plan(store, cache, batch, out, mode, L, flags, workspace, s);
     if (rc) return rc;
-    return do_rebind(cfg, store, cache, batch, out, workspace, s);
+    return do_rebind(cfg, store, cache, batch, out, workspace, true, s);
 }
 
 int prcr_store_raw(const prcr_rope_cfg* cfg, const prcr_store_desc* store, int32_t seq,

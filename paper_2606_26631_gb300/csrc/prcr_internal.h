@@ -173,7 +173,7 @@ struct RebindArgs {
     int32_t n_seqs;
     int32_t n_revisits;
     int32_t n_tokens;
-    int32_t early_ctas;      // CTAs of the first wave
+    int32_t early_ctas;      // CTAs that prefetch: the first wave behind this call's plan, else none
     int64_t total_k;
     int32_t n_layers;
     int32_t head_dim;

@@ -7,7 +7,11 @@
 // revisit kernels say by how much), late in its work. Before its
 // first global load or store it waits for the grid it depends on to complete
 // and its writes to be visible. Only L2 prefetches, which return nothing to
-// the thread, go before that wait. A kernel whose predecessor is not one of
+// the thread, go before that wait; and, behind the plan kernel of the same
+// call, the rebind kernel's lookups of the rows that it prefetches: the plan
+// releases it only after its own wait, so that whatever wrote the batch is
+// done. Those values are checked against their ranges and used for nothing
+// else. A kernel whose predecessor is not one of
 // these (it never allows dependents) is launched when the predecessor
 // completes, as with a plain launch, and its wait returns at once.
 #pragma once

@@ -74,3 +74,14 @@ def select_raw(c, seqs, group, n_tokens):
     Hq = c.n_kv_heads * group
     return lib().prcr_select_topk(C.byref(c), C.byref(s), seqs, 0, Hq, FAKE, FAKE, 1, FAKE, FAKE, FAKE, None, FAKE,
                                   lib().prcr_select_workspace_size(seqs, Hq, n_tokens), None)
+
+
+def revisit(c, seqs, tokens, entry="inject"):
+    """A batch of one revisit of `tokens` per sequence: prcr_rebind_inject, prcr_plan or prcr_rebind_apply."""
+    total = seqs * tokens
+    st, ca = store(c, seqs, tokens), contiguous(c, seqs, 2 * tokens)
+    b = B.RevisitBatch(seq_rev_off=FAKE, rev_tok_off=FAKE, idx=FAKE, p_txt=FAKE, cache_len_in=FAKE, n_seqs=seqs, n_revisits=seqs,
+                       total_k=total)
+    o = B.Outputs(cache_len_out=FAKE + 4096, next_pos_out=FAKE, pos_out=None, slot_out=None, status=FAKE)
+    f = {"inject": lib().prcr_rebind_inject, "plan": lib().prcr_plan, "apply": lib().prcr_rebind_apply}[entry]
+    return f(C.byref(c), C.byref(st), C.byref(ca), C.byref(b), C.byref(o), 0, 2, 0, FAKE, lib().prcr_workspace_size(total), None)

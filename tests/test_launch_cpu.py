@@ -66,3 +66,18 @@ def test_decode_workspace_holds_shorter_calls(D):
     for layers, H, seqs, longest, shorter in ((1, 4, 1, 3649, 3601), (2, 4, 1, 1825, 1777), (1, 4, 5, 721, 673), (1, 1, 2, 7297, 7249)):
         c = F.cfg(layers, H, D)
         assert F.decode(c, seqs, 2, shorter, F.workspace(c, seqs, 2, longest)) == 0
+
+
+def test_rebind_looks_ahead_only_behind_its_own_plan():
+    """The rebind kernel reads the batch before its wait only where this call's
+    plan kernel, which waits first, stands before it. prcr_rebind_apply may
+    follow any kernel, one that still writes the batch among them."""
+    c = F.cfg(28, 4, 128)
+    F.launches()
+    assert F.revisit(c, 8, 512) == 0
+    plan, rebind = F.launches()
+    assert "plan_kernel" in plan[0] and "rebind_kernel" in rebind[0] and rebind[1][5] > 0
+    assert F.revisit(c, 8, 512, "plan") == 0 and F.revisit(c, 8, 512, "apply") == 0
+    plan, alone = F.launches()
+    assert "plan_kernel" in plan[0] and "rebind_kernel" in alone[0]
+    assert alone[1][:5] == rebind[1][:5] and alone[1][5] == 0
