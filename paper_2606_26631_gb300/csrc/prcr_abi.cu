@@ -511,10 +511,12 @@ int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms, int64_t* most
 void decode_split(int64_t n_seqs, int n_layers, int64_t max_len, int sms, int n_kv_heads,
                   int head_dim, int* splits, int* chunk, int* team, int64_t* most) {
     const int64_t units = n_seqs * n_layers * n_kv_heads;
+    max_len = std::min<int64_t>(max_len, INT32_MAX);  // a sequence's length is an int32
     *team = 0;
-    const int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, team, most)
+    int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, team, most)
                       : head_dim == 128 ? decode_chunk<128>(n_seqs, units, max_len, sms, team, most)
                                         : decode_wide_chunk(units, max_len, sms, most);
+    c = std::min<int64_t>(c, 1 << 30);
     *chunk = int(c);
     *splits = int((max_len + c - 1) / c);
     *most = std::max<int64_t>(*most, *splits);

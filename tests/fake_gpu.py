@@ -85,3 +85,9 @@ def revisit(c, seqs, tokens, entry="inject"):
     o = B.Outputs(cache_len_out=FAKE + 4096, next_pos_out=FAKE, pos_out=None, slot_out=None, status=FAKE)
     f = {"inject": lib().prcr_rebind_inject, "plan": lib().prcr_plan, "apply": lib().prcr_rebind_apply}[entry]
     return f(C.byref(c), C.byref(st), C.byref(ca), C.byref(b), C.byref(o), 0, 2, 0, FAKE, lib().prcr_workspace_size(total), None)
+
+
+def paged(c, seqs, blocks_per_seq, block):
+    row = c.n_kv_heads * c.head_dim
+    return B.CacheDesc(kind=1, block_size=block, k=FAKE, v=FAKE, seq_stride=0, layer_stride=1024 * block * row, block_stride=block * row,
+                       slot_stride=row, block_table=FAKE, bt_stride=blocks_per_seq, n_blocks=1024, max_slots=0, n_seqs=seqs)

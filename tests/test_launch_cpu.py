@@ -81,3 +81,16 @@ def test_rebind_looks_ahead_only_behind_its_own_plan():
     plan, alone = F.launches()
     assert "plan_kernel" in plan[0] and "rebind_kernel" in alone[0]
     assert alone[1][:5] == rebind[1][:5] and alone[1][5] == 0
+
+
+@pytest.mark.parametrize("D", [64, 128, 256])
+@pytest.mark.parametrize("max_len", [2 ** 31 - 17, 2 ** 31 - 1, 2 ** 31, 2 ** 32, 2 ** 40])
+def test_decode_any_max_len(D, max_len):
+    """A paged cache's capacity, and max_len with it, may exceed an int32 (a
+    sequence's length cannot): the split still covers every length."""
+    for layers, H, seqs in ((1, 1, 1), (36, 8, 1), (36, 8, 16)):
+        c = F.cfg(layers, H, D)
+        F.launches()
+        assert F.decode(c, seqs, 2, max_len, 1 << 60, F.paged(c, seqs, 2 ** 30, 2 ** 10)) == 0
+        splits, chunk = F.launches()[0][1][5:7]
+        assert 0 < chunk <= 2 ** 30 and splits * chunk >= 2 ** 31 - 17, (splits, chunk)
