@@ -10,6 +10,7 @@ from paper_2606_26631_gb300 import _binding as B
 from paper_2606_26631_gb300 import _build
 
 FAKE = 1 << 40  # a device address, never dereferenced
+WORK = FAKE + (1 << 30)  # a selection's workspace
 
 
 @functools.lru_cache(None)
@@ -56,11 +57,11 @@ def decode(c, seqs, group, max_len, ws_bytes, cache=None):
                                        ws_bytes, None)
 
 
-def select_cached(c, seqs, group, n_tokens):
-    cache = contiguous(c, seqs, n_tokens)
+def select_cached(c, seqs, group, n_tokens, cache=None):
+    cache = cache or contiguous(c, seqs, n_tokens)
     Hq = c.n_kv_heads * group
     return lib().prcr_select_topk_cached(C.byref(c), C.byref(cache), seqs, 0, Hq, n_tokens, FAKE, FAKE, FAKE, 1, FAKE, FAKE, FAKE, None, FAKE,
-                                         FAKE, lib().prcr_select_workspace_size(seqs, Hq, n_tokens), None)
+                                         WORK, lib().prcr_select_workspace_size(seqs, Hq, n_tokens), None)
 
 
 def store(c, seqs, n_tokens):
@@ -87,7 +88,7 @@ def revisit(c, seqs, tokens, entry="inject"):
     return f(C.byref(c), C.byref(st), C.byref(ca), C.byref(b), C.byref(o), 0, 2, 0, FAKE, lib().prcr_workspace_size(total), None)
 
 
-def paged(c, seqs, blocks_per_seq, block):
+def paged(c, seqs, blocks_per_seq, block, n_blocks=1024):
     row = c.n_kv_heads * c.head_dim
     return B.CacheDesc(kind=1, block_size=block, k=FAKE, v=FAKE, seq_stride=0, layer_stride=1024 * block * row, block_stride=block * row,
-                       slot_stride=row, block_table=FAKE, bt_stride=blocks_per_seq, n_blocks=1024, max_slots=0, n_seqs=seqs)
+                       slot_stride=row, block_table=FAKE, bt_stride=blocks_per_seq, n_blocks=n_blocks, max_slots=0, n_seqs=seqs)

@@ -94,3 +94,15 @@ def test_decode_any_max_len(D, max_len):
         assert F.decode(c, seqs, 2, max_len, 1 << 60, F.paged(c, seqs, 2 ** 30, 2 ** 10)) == 0
         splits, chunk = F.launches()[0][1][5:7]
         assert 0 < chunk <= 2 ** 30 and splits * chunk >= 2 ** 31 - 17, (splits, chunk)
+
+
+@pytest.mark.parametrize("n_tokens", [64, 16384])  # one kernel, and two
+def test_cached_selection_of_a_cache_without_rows(n_tokens):
+    """A token without a cache row reads the cache's first row (and drops it);
+    a cache that has none is no readable memory, so the workspace stands in."""
+    c = F.cfg(1, 8, 128)
+    for cache, first_row in ((F.paged(c, 4, 2048, 16), 1), (F.contiguous(c, 4, n_tokens), 1), (F.paged(c, 4, 2048, 16, n_blocks=0), 0),
+                             (F.paged(c, 4, 0, 16), 0), (F.contiguous(c, 4, 0), 0)):
+        F.launches()
+        assert F.select_cached(c, 4, 4, n_tokens, cache) == 0
+        assert F.launches()[0][1][5] == first_row

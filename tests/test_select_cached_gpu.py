@@ -354,3 +354,18 @@ def test_select_cached_sizes(B, M, k, dup):
         assert (np.abs(score[b] - ref) / ref).max() <= 1e-4
     for b in range(B):
         assert np.array_equal(idx[b], _topk_by(score[b].astype(np.float64), k)), b
+
+
+@pytest.mark.parametrize("M", [70, 9000])  # one kernel, and two
+def test_select_cached_no_rows(M):
+    """A cache of no blocks: PRCR_ST_NO_BLOCK, relevance 0, the first k tokens."""
+    import paper_2606_26631_gb300 as prcr
+    B, H, Hq, D, k = 2, 4, 8, 128, 9
+    cache_k, bt, img0 = _make_cache(B, 1, H, D, M, True, 16, 3)
+    cd = prcr.cache_paged(cache_k, cache_k, bt)
+    cd.n_blocks = 0
+    q = torch.randn((B, Hq, D), device=DEV).to(torch.bfloat16)
+    q_pos = torch.full((B,), M + 50, dtype=torch.int64, device=DEV)
+    sel, _, _, score, st = _run(prcr.rope_cfg(1, H, D, (24, 20, 20), 1e6), cd, 0, q, q_pos, img0, M, k)
+    assert st == prcr.ST_NO_BLOCK and np.all(score == 0.0)
+    assert np.array_equal(sel, np.tile(np.arange(k), (B, 1)))
