@@ -503,13 +503,79 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4
                  : "r"(addr));
 }
 
+// What the phases of decode_wide_kernel share, in static shared memory.
+struct WideShared {
+    float cos[kWideD / 2], sin[kWideD / 2];            // of the query's turn
+    float m[kWideWarps][8], l[kWideWarps][8];          // every warp's maximum and sum per head
+};
+
+// A warp's share of a chunk again, by float32 FMAs, into its accumulators in
+// shared memory: for the rare chunk with an infinite or NaN key, value or query. An
+// infinity times a zero or negative piece of a split operand is a NaN, where the
+// product with the whole operand is an infinity (and a logit of -inf a weight of 0).
+// A call, and over the accumulators stored as usual: inlined 801 us for the largest
+// shape below, stored in its place 805, this 797, without it 795.
+__device__ __noinline__ void wide_exact(const DecodeArgs& a, WideShared& sh, uint32_t s_begin, uint32_t s_end) {
+    constexpr int D = kWideD, P = D / 2, V = P / 32;  // a lane has V pairs
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = a.group;
+    const int b = blockIdx.z, l = blockIdx.y, kh = int(blockIdx.x) % a.n_kv_heads;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* o_s = reinterpret_cast<float*>(smem_raw) + warp * 8 * kWideOPitch;
+    const float *cs = sh.cos, *sn = sh.sin;
+    float *m_s = sh.m[warp], *l_s = sh.l[warp];
+    const uint16_t* qb = a.q + ((int64_t(b) * a.n_layers + l) * a.n_q_heads + kh * g) * D + lane * V;
+    const int64_t head_off = int64_t(l) * a.layer_stride + int64_t(kh) * D + lane * V;
+    auto value = [](uint16_t w) { return __uint_as_float(uint32_t(w) << 16); };
+    __syncwarp();  // the warp's stores that are overwritten here
+    for (int h = 0; h < g; ++h) {
+        float qx[V], qy[V], ox[V], oy[V], m = -INFINITY, sum = 0.0f;
+        for (int i = 0; i < V; ++i) {
+            const float x = value(qb[h * D + i]), y = value(qb[h * D + i + P]), c = cs[lane * V + i], s = sn[lane * V + i];
+            qx[i] = fmaf(x, c, -y * s) * a.scale;
+            qy[i] = fmaf(y, c, x * s) * a.scale;
+            ox[i] = oy[i] = 0.0f;
+        }
+        for (uint32_t t = s_begin + 16 * warp; t < s_end; t += 16 * kWideWarps) {
+            for (uint32_t s = t; s < min(t + 16, s_end); ++s) {
+                int64_t row = int64_t(b) * a.seq_stride + int64_t(s) * a.slot_stride;
+                if (a.cache_kind == PRCR_CACHE_PAGED) {
+                    const int32_t blk = a.block_table[int64_t(b) * a.bt_stride + s / uint32_t(a.block_size)];
+                    if (blk < 0 || blk >= a.n_blocks) continue;
+                    row = int64_t(blk) * a.block_stride + int64_t(s % uint32_t(a.block_size)) * a.slot_stride;
+                }
+                const uint16_t* k = a.cache_k + head_off + row;
+                const uint16_t* v = a.cache_v + head_off + row;
+                float logit = 0.0f;
+                for (int i = 0; i < V; ++i) logit = fmaf(qy[i], value(k[i + P]), fmaf(qx[i], value(k[i]), logit));
+                for (int o = 16; o; o >>= 1) logit += __shfl_xor_sync(kFull, logit, o);
+                const float m_new = fmaxf(m, logit), alpha = m_new == -INFINITY ? 1.0f : expf(m - m_new);
+                const float p = logit == -INFINITY ? 0.0f : expf(logit - m_new);
+                m = m_new;
+                sum = sum * alpha + p;
+                for (int i = 0; i < V; ++i) {
+                    ox[i] = fmaf(p, value(v[i]), ox[i] * alpha);
+                    oy[i] = fmaf(p, value(v[i + P]), oy[i] * alpha);
+                }
+            }
+        }
+        for (int i = 0; i < V; ++i) {
+            o_s[h * kWideOPitch + lane * V + i] = ox[i];
+            o_s[h * kWideOPitch + lane * V + i + P] = oy[i];
+        }
+        if (lane == 0) {
+            m_s[h] = m;
+            l_s[h] = sum;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kWideWarps * 32, 2)
     decode_wide_kernel(const __grid_constant__ DecodeArgs a) {
     constexpr int D = kWideD, P = D / 2, KS = D / 16;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) float s_cos[P];
-    __shared__ __align__(16) float s_sin[P];
-    __shared__ float s_m[kWideWarps][8], s_l[kWideWarps][8];
+    __shared__ WideShared sh;
+    auto &s_cos = sh.cos, &s_sin = sh.sin;
+    auto &s_m = sh.m, &s_l = sh.l;
     const int b = blockIdx.z, l = blockIdx.y, H = a.n_kv_heads, g = a.group;
     const int split = int(blockIdx.x) / H, kh = int(blockIdx.x) - split * H;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
@@ -710,6 +776,9 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     float* o_s = reinterpret_cast<float*>(smem_raw) + warp * 8 * kWideOPitch;
+    float any = 0.0f;  // not finite where an accumulator is not
+#pragma unroll
+    for (int mt = 0; mt < KS; ++mt) any += (o[mt][0] + o[mt][1]) + (o[mt][2] + o[mt][3]);
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
         const int h = 2 * t + hh;
@@ -723,6 +792,7 @@ __global__ void __launch_bounds__(kWideWarps * 32, 2)
             s_l[warp][h] = l_run[hh];
         }
     }
+    if (__any_sync(kFull, !(fabsf(any) <= 3.0e38f))) wide_exact(a, sh, s_begin, s_end);
     __syncthreads();
     const float* o_all = reinterpret_cast<const float*>(smem_raw);
     for (int e = threadIdx.x; e < g * (D / 2); e += blockDim.x) {

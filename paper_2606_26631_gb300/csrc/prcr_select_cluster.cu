@@ -443,6 +443,28 @@ struct PairTables {
     }
 };
 
+// One logit of a raw key by float32 FMAs, for the rare key or query with an
+// infinity or NaN: an infinity's remainder is a NaN, where the product with the whole
+// operand is an infinity (and a logit of -inf a weight of 0).
+template <int D>
+__device__ __noinline__ float raw_logit(const SelectArgs& a, int b, int hq, int m, int64_t p, const uint64_t* tf, const uint8_t* ax) {
+    constexpr int P = D / 2;
+    const uint16_t* q = a.q + (int64_t(b) * a.n_q_heads + hq) * D;
+    const uint16_t* k = a.store_k + int64_t(b) * a.store_seq_stride + int64_t(a.layer) * a.store_layer_stride +
+                        int64_t(m) * a.store_token_stride + int64_t(hq / (a.n_q_heads / a.n_kv_heads)) * D;
+    const int32_t* crd = a.coords + int64_t(b) * a.coord_seq_stride + 3 * int64_t(m);
+    auto value = [](uint16_t w) { return __uint_as_float(uint32_t(w) << 16); };
+    float sum = 0.0f;
+    for (int i = 0; i < P; ++i) {
+        float sn, cs;
+        sincos_coord(int64_t(crd[ax[i]]) - p, tf[i], &sn, &cs);
+        const float x = value(k[i]), y = value(k[i + P]);
+        sum = fmaf(value(q[i]), fmaf(x, cs, -y * sn), sum);
+        sum = fmaf(value(q[i + P]), fmaf(y, cs, x * sn), sum);
+    }
+    return sum * a.scale;
+}
+
 // Logits of tokens m_beg .. m_beg + nt - 1 of sequence b for the query heads of
 // KV heads kh0 .. kh0 + H - 1: query head kh0 g + h, token m_beg + t at
 // lg[h * lg_pitch + t]. Raw keys are turned by the offsets of their
@@ -695,6 +717,10 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
                 } else {  // chain 1: the keys' remainders (and lead's rounding errors)
                     va = ((D == 256 ? lead[c] : acc[0][c]) + acc[1][c]) * a.scale;
                     vb = ((D == 256 ? lead[2 + c] : acc[0][2 + c]) + acc[1][2 + c]) * a.scale;
+                }
+                if constexpr (D == 256 && !CACHED) {
+                    if (va != va && ta < nt) va = raw_logit<D>(a, b, kh0 * g + kh * g + 2 * tq + c, m_beg + ta, p, pt.tf, pt.ax);
+                    if (vb != vb && tb < nt) vb = raw_logit<D>(a, b, kh0 * g + kh * g + 2 * tq + c, m_beg + tb, p, pt.tf, pt.ax);
                 }
                 float* dst = lg + (kh * g + 2 * tq + c) * lg_pitch;
                 if (ta < nt) dst[ta] = ok_a ? va : -INFINITY;

@@ -370,3 +370,54 @@ def test_decode_full_size_sampled():
             assert err <= 1e-4, (b, l, n, err)
     del inp
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("max_len,paged,nL", [(100, False, 1), (1200, True, 2), (5000, False, 30)])
+def test_decode_infinities_d256(max_len, paged, nL):
+    """head_dim 256, where operands are split into pieces: a key whose logit is
+    -inf has weight 0 (the output is the attention over the other slots), one
+    whose logit is +inf makes its head NaN, an infinite value stays infinite in
+    its dimension and touches no other. Unsplit, few and many chunks."""
+    import paper_2606_26631_gb300 as prcr
+    H, Hq, D, dim, slot = 2, 6, 256, 37, max_len - 30
+    P, g = D // 2, Hq // H
+    inp = make_decode_inputs(1, nL, H, Hq, D, max_len, paged, device=DEV, seed=12)
+    ck, cv, bt = inp["cache_k"], inp["cache_v"], inp["block_table"]
+
+    def put(cache, h, d, x):
+        if paged:
+            cache[:, int(bt[0, slot // 16]), slot % 16, h, d] = x
+        else:
+            cache[0, :, slot, h, d] = x
+
+    cfg = prcr.rope_cfg(nL, H, D, (48, 40, 40), 1e6)
+    cd = prcr.cache_paged(ck, cv, bt) if paged else prcr.cache_contiguous(ck, cv)
+    p, l = int(inp["q_pos"][0]), nL - 1
+    qv = _f64(inp["q"])[0, l]
+    K, V = (x[:, l] for x in _cache_rows(ck, cv, bt, 0, max_len, paged))
+    others = np.arange(max_len) != slot
+    full = O.decode_attention(qv, p, K, V, D, (48, 40, 40), 1e6)
+    without = O.decode_attention(qv, p, K[others], V[others], D, (48, 40, 40), 1e6)
+    angle = p * 1e6 ** (-2.0 * dim / D)
+    rot = qv[:, dim] * np.cos(angle) - qv[:, dim + P] * np.sin(angle)  # the query's component that meets the infinite key
+    vmax = np.abs(V).max()
+    for sign in (-1.0, 1.0):
+        kept = ck.clone()
+        put(ck, 0, dim, sign * float("inf"))
+        out, st = _run_decode(cfg, cd, inp["q"], inp["q_pos"], inp["seq_len"], max_len)
+        ck.copy_(kept)
+        got = out[0, l].cpu().numpy()
+        assert st == 0
+        for h in range(Hq):
+            if h < g and sign * rot[h] > 0:
+                assert np.all(np.isnan(got[h])), h
+            else:
+                assert np.abs(got[h] - (without if h < g else full)[h]).max() <= 8e-6 * vmax, h
+    kept = cv.clone()
+    put(cv, 1, 200, float("-inf"))
+    out, st = _run_decode(cfg, cd, inp["q"], inp["q_pos"], inp["seq_len"], max_len)
+    cv.copy_(kept)
+    got = out[0, l].cpu().numpy()
+    assert st == 0 and np.all(np.isneginf(got[g:, 200]))
+    got[g:, 200] = full[g:, 200]
+    assert np.abs(got - full).max() <= 8e-6 * vmax

@@ -315,3 +315,34 @@ def test_select_raw_sizes(B, M, k, H, Hq, D):
         assert (np.abs(got[b] - ref) / ref).max() <= 1e-4
     for b in range(B):
         assert np.array_equal(sel[b], _topk_by(got[b].astype(np.float64), k)), b
+
+
+@pytest.mark.parametrize("M", [70, 9000])  # one kernel, and two
+def test_select_infinite_key_d256(M):
+    """head_dim 256, where the keys are split into pieces: a key whose logit is
+    -inf has relevance 0 and leaves the others as they are without it."""
+    import paper_2606_26631_gb300 as prcr
+    D, P, m, k, sec = 256, 128, 41, 9, (48, 40, 40)
+    g = torch.Generator(device=DEV).manual_seed(7)
+    store_k = torch.randn((1, 1, M, 1, D), device=DEV, generator=g).to(torch.bfloat16)
+    coords = torch.randint(0, 60, (1, M, 3), device=DEV, generator=g, dtype=torch.int32)
+    q = torch.randn((1, 1, D), device=DEV, generator=g).to(torch.bfloat16)
+    q_pos = torch.full((1,), 700, dtype=torch.int64, device=DEV)
+    qv = O.bf16_bits_to_f64(q.view(torch.int16).cpu().numpy())[0]
+    kv, cv = store_k[0, 0].view(torch.int16).cpu().numpy(), coords[0].cpu().numpy()
+    others = np.arange(M) != m
+    ref = O.ads_relevance(qv, 700, kv[others], cv[others], D, sec, 1e6)
+    for i in range(P):  # a pair both of whose turned components meet the query with one sign
+        angle = float(cv[m, 0 if i < 48 else 1 if i < 88 else 2] - 700) * 1e6 ** (-2.0 * i / D)
+        x, y = qv[0, i] * np.cos(angle), qv[0, i + P] * np.sin(angle)
+        if x * y > 1e-3:
+            break
+    store_k[0, 0, m, 0, i] = -float("inf") if x > 0 else float("inf")
+    idx, sro, rto = (torch.zeros(n, dtype=torch.int32, device=DEV) for n in (k, 2, 2))
+    score = torch.full((1, M), -1.0, dtype=torch.float32, device=DEV)
+    ws = torch.empty(prcr.select_workspace_size(1, 1, M), dtype=torch.uint8, device=DEV)
+    prcr.select_topk(prcr.rope_cfg(1, 1, D, sec, 1e6), prcr.store_desc(store_k, store_k, coords), 0, q, q_pos, k, idx, sro, rto, ws, score)
+    got = score[0].cpu().numpy()
+    assert got[m] == 0.0
+    assert (np.abs(got[others] - ref) / ref).max() <= 1e-4
+    assert np.array_equal(idx.cpu().numpy(), _topk_by(got.astype(np.float64), k))
