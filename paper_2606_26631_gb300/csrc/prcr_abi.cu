@@ -846,10 +846,14 @@ int prcr_select_topk_cached(const prcr_rope_cfg* cfg, const prcr_cache_desc* cac
     a.block_size = cache->kind == PRCR_CACHE_PAGED ? cache->block_size : 1;
     a.n_blocks = cache->n_blocks;
     a.cache_kind = cache->kind;
-    // a cache without a single row may be no memory at all: the workspace (1 KB at
-    // least) stands in for it
-    const bool rows = a.cache_capacity > 0 && (cache->kind == PRCR_CACHE_CONTIGUOUS || cache->n_blocks > 0);
-    a.no_row = rows ? a.cache_k : static_cast<const uint16_t*>(workspace);
+    a.cache_head_stride = cfg->head_dim;
+    if (a.cache_capacity == 0 || (cache->kind == PRCR_CACHE_PAGED && cache->n_blocks == 0)) {
+        // a cache without a single row may be no memory at all: the workspace (1 KB
+        // at least) stands in for its first row at every layer and head
+        a.cache_k = static_cast<const uint16_t*>(workspace);
+        a.cache_layer_stride = 0;
+        a.cache_head_stride = 0;
+    }
     a.img_slot0 = img_slot0;
     a.status = status;
     int dev = 0;

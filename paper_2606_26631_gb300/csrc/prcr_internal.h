@@ -331,13 +331,13 @@ struct SelectArgs {
     int64_t cache_layer_stride;
     int64_t cache_block_stride; // paged
     int64_t cache_slot_stride;
+    int32_t cache_head_stride;  // head_dim
     int64_t cache_capacity;     // slots per sequence
     const int32_t* block_table;
     int32_t bt_stride;
     int32_t block_size;
     int32_t n_blocks;
     int32_t cache_kind;
-    const uint16_t* no_row;     // head_dim readable elements, read for a token without a cache row
     const int32_t* img_slot0;   // [B] first slot of each sequence's image tokens
     uint32_t* status;
     uint64_t turn_freq[kMaxPairs];  // pair i: round(inv_freq_i / (2 pi) * 2^64)

@@ -497,18 +497,18 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
 
     // the items of this warp: warp, warp + NW, ... of (tile, KV head), heads fastest
     uint4 k[NR][RL];
-    const uint16_t* kb = CACHED ? a.cache_k + int64_t(a.layer) * a.cache_layer_stride + kh0 * D + 8 * tq
+    const uint16_t* kb = CACHED ? a.cache_k + int64_t(a.layer) * a.cache_layer_stride + kh0 * a.cache_head_stride + 8 * tq
                                 : a.store_k + int64_t(b) * a.store_seq_stride + int64_t(m_beg) * a.store_token_stride +
                                       int64_t(a.layer) * a.store_layer_stride + kh0 * D + 8 * tq;
     // this lane's two token rows (gid and gid + 8 of the tile) at KV head kh; a
-    // token past the end reads the last one, one without a row what no_row
-    // points to (their logits are not stored, or are -inf)
+    // token past the end reads the last one, one without a row the cache's
+    // first row (their logits are not stored, or are -inf)
     auto rows = [&](int tile, int kh, const uint16_t* (&r)[2]) {
         const int ta = min(16 * tile + gid, nt - 1), tb = min(16 * tile + gid + 8, nt - 1);
         if constexpr (CACHED) {
             const int64_t ra = row_s[ta], rb = row_s[tb];
-            r[0] = ra < 0 ? a.no_row + 8 * tq : kb + ra + kh * D;
-            r[1] = rb < 0 ? a.no_row + 8 * tq : kb + rb + kh * D;
+            r[0] = kb + (ra < 0 ? 0 : ra) + kh * a.cache_head_stride;
+            r[1] = kb + (rb < 0 ? 0 : rb) + kh * a.cache_head_stride;
         } else {
             r[0] = kb + int64_t(ta) * a.store_token_stride + kh * D;
             r[1] = kb + int64_t(tb) * a.store_token_stride + kh * D;

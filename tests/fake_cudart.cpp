@@ -34,8 +34,8 @@ extern "C" {
 
 // launches since the last call, one per line: kernel, grid, block, dynamic
 // shared memory, and of a decode its splits, chunk and team, of a rebind the
-// CTAs that prefetch rows, of a selection whether a token without a cache row
-// reads the cache's first row
+// CTAs that prefetch rows, of a cached selection whether keys are read from
+// the cache (not the workspace)
 __attribute__((visibility("default"))) size_t fake_log(char* out, size_t n) {
     std::lock_guard<std::mutex> g(st().mu);
     std::snprintf(out, n, "%s", st().log.c_str());
@@ -107,7 +107,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
         std::snprintf(line + n, sizeof line - size_t(n), " %d", static_cast<const prcr::RebindArgs*>(args[0])->early_ctas);
     } else if (name.find("select_fused") != std::string::npos || name.find("select_logits") != std::string::npos) {
         const auto* a = static_cast<const prcr::SelectArgs*>(args[0]);
-        std::snprintf(line + n, sizeof line - size_t(n), " %d", a->no_row && a->no_row == a->cache_k);
+        std::snprintf(line + n, sizeof line - size_t(n), " %d", a->cache_k && a->cache_k != reinterpret_cast<const uint16_t*>(a->logits));
     }
     st().log += std::string(line) + "\n";
     return cudaSuccess;
