@@ -358,8 +358,9 @@ cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaS
 cudaError_t launch_select_fused(const SelectArgs& a, bool cached, int n_seqs, int sms, cudaStream_t stream, bool* done);
 // the logits of the cached-key selection
 cudaError_t launch_select_cached_logits(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream);
-// the steps after the logits: normalisers, relevances, top-k
-cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream);
+// the steps after the logits: normalisers, relevances, top-k (fine: logits of
+// float32's accuracy)
+cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, bool fine, cudaStream_t stream);
 
 // The dynamic shared-memory limit of a kernel on the current device, raised to
 // `smem` where it is lower. It belongs to the kernel, not to a launch, so it is

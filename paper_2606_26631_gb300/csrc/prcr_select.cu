@@ -555,7 +555,7 @@ cudaError_t launch_select(const SelectArgs& a, int n_seqs, int sms, cudaStream_t
                              : launch_logits<16>(a, n_seqs, sms, stream));
     }
     if (e != cudaSuccess) return e;
-    return launch_select_tail(a, n_seqs, stream);
+    return launch_select_tail(a, n_seqs, !mma, stream);
 }
 
 cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
@@ -564,7 +564,7 @@ cudaError_t launch_select_cached(const SelectArgs& a, int n_seqs, int sms, cudaS
     if (e != cudaSuccess || done) return e;
     e = launch_select_cached_logits(a, n_seqs, sms, stream);
     if (e != cudaSuccess) return e;
-    return launch_select_tail(a, n_seqs, stream);
+    return launch_select_tail(a, n_seqs, false, stream);
 }
 
 }  // namespace prcr

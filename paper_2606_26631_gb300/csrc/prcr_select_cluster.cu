@@ -80,7 +80,7 @@ struct SelectShared {
 // to the CTA), which each CTA writes into all of them. Also sets up the search's
 // shared state. The caller has arrived at the cluster barrier once at its start:
 // its completion here means that every peer is running.
-template <int NT>
+template <int NT, bool FINE>
 __device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, int rank, SelectShared& sh) {
     const int c = threadIdx.x & (kMaxCluster - 1);
     cluster_wait();
@@ -99,7 +99,7 @@ __device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, int rank
         float m = v.x;
 #pragma unroll
         for (int o = kMaxCluster / 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-        float z = v.x == -INFINITY ? 0.0f : v.y * __expf(v.x - m);
+        float z = v.x == -INFINITY ? 0.0f : v.y * exp_term<FINE>(v.x - m);
 #pragma unroll
         for (int o = kMaxCluster / 2; o; o >>= 1) z += __shfl_xor_sync(kAll, z, o);
         // no finite logit (no readable token, or a query position out of
@@ -275,22 +275,24 @@ __device__ __forceinline__ void select_topk(const SelectArgs& a, int b, int C, i
     }
 }
 
-// (max, sum of exp) of 16 logits (-inf where there is none) into a running one.
-__device__ __forceinline__ void stats16(const float (&x)[16], float& mx, float& z) {
-    float cm = mx;
+// (max, sum of exp) of N logits (-inf where there is none) into a running one.
+template <bool FINE, int N>
+__device__ __forceinline__ void stats_of(const float (&x)[N], float& mx, float& z) {
+    float cm = x[0];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) cm = fmaxf(cm, x[u]);
+    for (int u = 1; u < N; ++u) cm = fmaxf(cm, x[u]);
     if (cm == -INFINITY) return;
+    cm = fmaxf(cm, mx);
     float cz = 0.0f;
 #pragma unroll
-    for (int u = 0; u < 16; ++u) cz += __expf(x[u] - cm);
-    z = (mx == -INFINITY ? 0.0f : z * __expf(mx - cm)) + cz;
+    for (int u = 0; u < N; ++u) cz += exp_term<FINE>(x[u] - cm);
+    z = (mx == -INFINITY ? 0.0f : z * exp_term<FINE>(mx - cm)) + cz;
     mx = cm;
 }
 
 // The statistics of a CTA's nt tokens, a warp per query head, from logits in
 // global memory.
-template <int NW>
+template <int NW, bool FINE>
 __device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int nt, bool vec, SelectShared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int hq = warp; hq < Hq; hq += NW) {
@@ -307,23 +309,29 @@ __device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int n
                     float* y = x[u / 4] + 4 * (u % 4);
                     y[0] = v.x; y[1] = v.y; y[2] = v.z; y[3] = v.w;
                 }
-                stats16(x[0], mx, z);
-                stats16(x[1], mx, z);
+                if (nt <= 128) {  // one load each
+                    const float x4[4] = {x[0][0], x[0][1], x[0][2], x[0][3]};
+                    stats_of<FINE>(x4, mx, z);
+                } else {
+                    stats_of<FINE>(x[0], mx, z);
+                    stats_of<FINE>(x[1], mx, z);
+                }
             }
         } else {
             for (int i = lane; i - lane < nt; i += 512) {
                 float x[16];
 #pragma unroll
                 for (int u = 0; u < 16; ++u) x[u] = i + 32 * u < nt ? row[i + 32 * u] : -INFINITY;
-                stats16(x, mx, z);
+                stats_of<FINE>(x, mx, z);
             }
         }
+        float m = mx;
 #pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const float m2 = __shfl_xor_sync(kAll, mx, o), z2 = __shfl_xor_sync(kAll, z, o);
-            merge_max_sum(mx, z, m2, z2);
-        }
-        if (lane == 0) sh.stat[hq] = make_float2(mx, z);
+        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
+        z = mx == -INFINITY ? 0.0f : z * exp_term<FINE>(mx - m);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(kAll, z, o);
+        if (lane == 0) sh.stat[hq] = make_float2(m, z);
     }
 }
 
@@ -339,6 +347,7 @@ __device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int n
 constexpr int kTailThreads = 1024;
 constexpr int kTailMinTokens = 64;  // per CTA
 
+template <bool FINE>
 __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __grid_constant__ SelectArgs a) {
     pdl_allow();
     constexpr int NT = kTailThreads, NW = NT / 32;
@@ -354,9 +363,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
     cluster_arrive();
     pdl_wait();
 
-    tail_stats<NW>(lg, M, Hq, nt, vec, sh);
+    tail_stats<NW, FINE>(lg, M, Hq, nt, vec, sh);
     __syncthreads();
-    merge_stats<NT>(a, C, rank, sh);
+    merge_stats<NT, FINE>(a, C, rank, sh);
     uint32_t lo = 0xffffffffu, hi = 0u;
     auto seen = [&](float r) {
         lo = min(lo, __float_as_uint(r));
@@ -369,10 +378,10 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
             float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             auto add = [&](const float4& x, int h) {
                 const float2 n = sh.norm[h];
-                r.x = fmaf(__expf(x.x - n.x), n.y, r.x);
-                r.y = fmaf(__expf(x.y - n.x), n.y, r.y);
-                r.z = fmaf(__expf(x.z - n.x), n.y, r.z);
-                r.w = fmaf(__expf(x.w - n.x), n.y, r.w);
+                r.x = fmaf(exp_term<FINE>(x.x - n.x), n.y, r.x);
+                r.y = fmaf(exp_term<FINE>(x.y - n.x), n.y, r.y);
+                r.z = fmaf(exp_term<FINE>(x.z - n.x), n.y, r.z);
+                r.w = fmaf(exp_term<FINE>(x.w - n.x), n.y, r.w);
             };
             int h = 0;
             for (; h + 8 <= Hq; h += 8) {  // eight heads' logits requested together
@@ -399,9 +408,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
 #pragma unroll
                 for (int u = 0; u < 16; ++u) x[u] = lg[int64_t(h + u) * M + i];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) r = fmaf(__expf(x[u] - sh.norm[h + u].x), sh.norm[h + u].y, r);
+                for (int u = 0; u < 16; ++u) r = fmaf(exp_term<FINE>(x[u] - sh.norm[h + u].x), sh.norm[h + u].y, r);
             }
-            for (; h < Hq; ++h) r = fmaf(__expf(lg[int64_t(h) * M + i] - sh.norm[h].x), sh.norm[h].y, r);
+            for (; h < Hq; ++h) r = fmaf(exp_term<FINE>(lg[int64_t(h) * M + i] - sh.norm[h].x), sh.norm[h].y, r);
             rel[i] = r;
             seen(r);
             if (a.score_out) a.score_out[int64_t(b) * M + m_beg + i] = r;
@@ -799,7 +808,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     __syncthreads();
     cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
     __syncthreads();
-    merge_stats<NT>(a, C, rank, sh);
+    merge_stats<NT, false>(a, C, rank, sh);
 
     // relevances: `per` lanes share a token (its heads in turn) where the CTA
     // has few tokens
@@ -923,16 +932,17 @@ int tokens_per_cta(int n_tokens, int C) { return ((n_tokens + C - 1) / C + 15) /
 
 }  // namespace
 
-cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, cudaStream_t stream) {
+cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, bool fine, cudaStream_t stream) {
     SelectArgs t = a;
-    const void* k = reinterpret_cast<const void*>(select_tail_kernel);
+    auto kern = fine ? select_tail_kernel<true> : select_tail_kernel<false>;
+    const void* k = reinterpret_cast<const void*>(kern);
     const cudaError_t e = pick_cluster(k, kTailThreads, n_seqs, a.n_tokens, kTailMinTokens, &t.cluster);
     if (e != cudaSuccess) return e;
     t.tok_per_cta = tokens_per_cta(a.n_tokens, t.cluster);
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kTailThreads, t.cluster,
                                                   size_t(t.cluster) * t.tok_per_cta * 4, stream, attr);
-    return cudaLaunchKernelEx(&cfg, select_tail_kernel, t);
+    return cudaLaunchKernelEx(&cfg, kern, t);
 }
 
 // The one-kernel selection, or *done = false where it does not fit or is the

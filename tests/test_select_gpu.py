@@ -346,3 +346,24 @@ def test_select_infinite_key_d256(M):
     assert got[m] == 0.0
     assert (np.abs(got[others] - ref) / ref).max() <= 1e-4
     assert np.array_equal(idx.cpu().numpy(), _topk_by(got.astype(np.float64), k))
+
+
+@pytest.mark.parametrize("B,M,H,Hq,D", [(3, 8192, 4, 32, 256), (2, 4099, 4, 28, 96), (16, 600, 4, 32, 256)])
+def test_select_weights_sum_to_one(B, M, H, Hq, D):
+    """Raw keys where the logits have float32's accuracy (head dims other than
+    64 and 128): the relevances of a sequence sum to 1 within half a unit in the
+    last place, 2^-24. Their rounding errors, and the heads' normalisers', are
+    thousands of independent ones that average out; what would remain is an
+    exp in the denominators that is off to one side."""
+    import paper_2606_26631_gb300 as prcr
+    sec = (D // 8, D // 4, D // 8)
+    g = torch.Generator(device=DEV).manual_seed(M)
+    store_k = torch.randn((B, 1, M, H, D), device=DEV, generator=g).to(torch.bfloat16)
+    coords = torch.randint(0, 60, (B, M, 3), device=DEV, generator=g, dtype=torch.int32)
+    q = torch.randn((B, Hq, D), device=DEV, generator=g).to(torch.bfloat16)
+    q_pos = torch.arange(B, device=DEV, dtype=torch.int64) * 41 + 700
+    idx, sro, rto = (torch.zeros(n, dtype=torch.int32, device=DEV) for n in (B, B + 1, B + 1))
+    score = torch.zeros((B, M), dtype=torch.float32, device=DEV)
+    ws = torch.empty(prcr.select_workspace_size(B, Hq, M), dtype=torch.uint8, device=DEV)
+    prcr.select_topk(prcr.rope_cfg(1, H, D, sec, 1e6), prcr.store_desc(store_k, store_k, coords), 0, q, q_pos, 1, idx, sro, rto, ws, score)
+    assert float((score.double().sum(1) - 1.0).mean().abs()) <= 2.0 ** -24
