@@ -99,7 +99,7 @@ __device__ __forceinline__ void merge_stats(const SelectArgs& a, int C, int rank
         float m = v.x;
 #pragma unroll
         for (int o = kMaxCluster / 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-        float z = v.x == -INFINITY ? 0.0f : v.y * exp_term<FINE>(v.x - m);
+        float z = v.y * (v.x == -INFINITY ? 0.0f : exp_term<FINE>(v.x - m));
 #pragma unroll
         for (int o = kMaxCluster / 2; o; o >>= 1) z += __shfl_xor_sync(kAll, z, o);
         // no finite logit (no readable token, or a query position out of
@@ -275,18 +275,23 @@ __device__ __forceinline__ void select_topk(const SelectArgs& a, int b, int C, i
     }
 }
 
-// (max, sum of exp) of N logits (-inf where there is none) into a running one.
+// (max, sum of exp) of N logits (-inf where there is none) into a running one. A
+// NaN logit makes the sum a NaN, also where no other is finite.
 template <bool FINE, int N>
 __device__ __forceinline__ void stats_of(const float (&x)[N], float& mx, float& z) {
     float cm = x[0];
 #pragma unroll
     for (int u = 1; u < N; ++u) cm = fmaxf(cm, x[u]);
-    if (cm == -INFINITY) return;
+    if (cm == -INFINITY) {  // no logit, unless one is a NaN
+#pragma unroll
+        for (int u = 0; u < N; ++u) z += x[u] == -INFINITY ? 0.0f : x[u];
+        return;
+    }
     cm = fmaxf(cm, mx);
     float cz = 0.0f;
 #pragma unroll
     for (int u = 0; u < N; ++u) cz += exp_term<FINE>(x[u] - cm);
-    z = (mx == -INFINITY ? 0.0f : z * exp_term<FINE>(mx - cm)) + cz;
+    z = z * (mx == -INFINITY ? 0.0f : exp_term<FINE>(mx - cm)) + cz;
     mx = cm;
 }
 
@@ -328,7 +333,7 @@ __device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int n
         float m = mx;
 #pragma unroll
         for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-        z = mx == -INFINITY ? 0.0f : z * exp_term<FINE>(mx - m);
+        z *= mx == -INFINITY ? 0.0f : exp_term<FINE>(mx - m);
 #pragma unroll
         for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(kAll, z, o);
         if (lane == 0) sh.stat[hq] = make_float2(m, z);

@@ -367,3 +367,25 @@ def test_select_weights_sum_to_one(B, M, H, Hq, D):
     ws = torch.empty(prcr.select_workspace_size(B, Hq, M), dtype=torch.uint8, device=DEV)
     prcr.select_topk(prcr.rope_cfg(1, H, D, sec, 1e6), prcr.store_desc(store_k, store_k, coords), 0, q, q_pos, 1, idx, sro, rto, ws, score)
     assert float((score.double().sum(1) - 1.0).mean().abs()) <= 2.0 ** -24
+
+
+@pytest.mark.parametrize("M", [33, 70, 2050, 9000])  # one kernel, and two
+@pytest.mark.parametrize("D", [96, 128, 256])
+def test_select_nan_key(D, M):
+    """A NaN key makes every relevance of its head NaN, wherever it lies."""
+    import paper_2606_26631_gb300 as prcr
+    sec = (D // 8, D // 4, D // 8)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    store_k = torch.randn((1, 1, M, 1, D), device=DEV, generator=g).to(torch.bfloat16)
+    coords = torch.randint(0, 60, (1, M, 3), device=DEV, generator=g, dtype=torch.int32)
+    q = torch.randn((1, 1, D), device=DEV, generator=g).to(torch.bfloat16)
+    q_pos = torch.full((1,), 700, dtype=torch.int64, device=DEV)
+    idx, sro, rto = (torch.zeros(n, dtype=torch.int32, device=DEV) for n in (3, 2, 2))
+    score = torch.zeros((1, M), dtype=torch.float32, device=DEV)
+    ws = torch.empty(prcr.select_workspace_size(1, 1, M), dtype=torch.uint8, device=DEV)
+    for m in (0, M // 2, M - 1):
+        keep = store_k[0, 0, m].clone()
+        store_k[0, 0, m, 0, 3] = float("nan")
+        prcr.select_topk(prcr.rope_cfg(1, 1, D, sec, 1e6), prcr.store_desc(store_k, store_k, coords), 0, q, q_pos, 3, idx, sro, rto, ws, score)
+        store_k[0, 0, m] = keep
+        assert bool(torch.isnan(score).all()) and idx.tolist() == [0, 1, 2], m
