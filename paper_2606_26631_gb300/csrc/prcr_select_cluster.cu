@@ -732,10 +732,6 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
                     va = ((D == 256 ? lead[c] : acc[0][c]) + acc[1][c]) * a.scale;
                     vb = ((D == 256 ? lead[2 + c] : acc[0][2 + c]) + acc[1][2 + c]) * a.scale;
                 }
-                if constexpr (D == 256 && !CACHED) {
-                    if (va != va && ta < nt) va = raw_logit<D>(a, b, kh0 * g + kh * g + 2 * tq + c, m_beg + ta, p, pt.tf, pt.ax);
-                    if (vb != vb && tb < nt) vb = raw_logit<D>(a, b, kh0 * g + kh * g + 2 * tq + c, m_beg + tb, p, pt.tf, pt.ax);
-                }
                 float* dst = lg + (kh * g + 2 * tq + c) * lg_pitch;
                 if (ta < nt) dst[ta] = ok_a ? va : -INFINITY;
                 if (tb < nt) dst[tb] = ok_b ? vb : -INFINITY;
@@ -745,9 +741,10 @@ __device__ __forceinline__ void cta_logits(const SelectArgs& a, const FusedLayou
 }
 
 // (max, sum of exp) per query head of nt tokens' logits in shared memory, two
-// heads of a warp side by side.
+// heads of a warp side by side. True where one of this thread's sums is a NaN.
 template <int NT>
-__device__ __forceinline__ void cta_stats(const float* lg_s, int pitch, int Hq, int nt, float2* stat) {
+__device__ __forceinline__ bool cta_stats(const float* lg_s, int pitch, int Hq, int nt, float2* stat) {
+    bool nan = false;
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int h0 = warp; h0 < Hq; h0 += 2 * NW) {
@@ -778,7 +775,9 @@ __device__ __forceinline__ void cta_stats(const float* lg_s, int pitch, int Hq, 
             stat[h0] = make_float2(ma, za);
             if (two) stat[h0 + NW] = make_float2(mb, zb);
         }
+        nan = nan || za != za || zb != zb;
     }
+    return nan;
 }
 
 // The whole selection in one kernel; the CTA's logits stay in shared memory.
@@ -811,8 +810,21 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     cta_logits<D, CACHED, NT>(a, f, b, 0, a.n_kv_heads, m_beg, nt, smem_raw, pt, lg_s, f.pitch, err);
     if (CACHED && err) atomicOr(a.status, err);
     __syncthreads();
-    cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
-    __syncthreads();
+    const bool nan = cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
+    if constexpr (D == 256 && !CACHED) {
+        if (__syncthreads_or(nan)) {
+            for (int e = tid; e < Hq * nt; e += NT) {
+                const int h = e / nt, t = e - h * nt;
+                float& x = lg_s[h * f.pitch + t];
+                if (x != x) x = raw_logit<D>(a, b, h, m_beg + t, a.q_pos[b], pt.tf, pt.ax);
+            }
+            __syncthreads();
+            cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
+            __syncthreads();
+        }
+    } else {
+        __syncthreads();
+    }
     merge_stats<NT, false>(a, C, rank, sh);
 
     // relevances: `per` lanes share a token (its heads in turn) where the CTA
