@@ -354,7 +354,6 @@ constexpr int kTailMinTokens = 64;  // per CTA
 
 template <bool FINE>
 __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_allow();
     constexpr int NT = kTailThreads, NW = NT / 32;
     __shared__ SelectShared sh;
     extern __shared__ __align__(16) uint32_t keys[];  // [cluster * tok_per_cta] relevances
@@ -370,6 +369,12 @@ __global__ void __launch_bounds__(kTailThreads, 1) select_tail_kernel(const __gr
 
     tail_stats<NW, FINE>(lg, M, Hq, nt, vec, sh);
     __syncthreads();
+    // Only now: released at entry, calls in a row pile up (each kernel releases the
+    // next before its own wait), and the waiting CTAs of 1024 threads crowd the logits
+    // kernel onto few SMs. 8 sequences of 768 tokens x 16 heads of 80 28.0 -> 22.7 us,
+    // 1 of 8192 x 16 heads of 256 36.4 -> 29.7, of 112 21.0 -> 20.7; before the search
+    // the same.
+    pdl_allow();
     merge_stats<NT, FINE>(a, C, rank, sh);
     uint32_t lo = 0xffffffffu, hi = 0u;
     auto seen = [&](float r) {
