@@ -462,26 +462,35 @@ struct PairTables {
     }
 };
 
-// One logit of a raw key by float32 FMAs, for the rare key or query with an
-// infinity or NaN: an infinity's remainder is a NaN, where the product with the whole
-// operand is an infinity (and a logit of -inf a weight of 0).
-template <int D>
-__device__ __noinline__ float raw_logit(const SelectArgs& a, int b, int hq, int m, int64_t p, const uint64_t* tf, const uint8_t* ax) {
+// The NaN logits of a CTA's tokens again, by float32 FMAs: for the rare key or
+// query with an infinity, whose remainder is a NaN, where the product with the whole
+// operand is an infinity (and a logit of -inf a weight of 0). A call: as code in the
+// kernel's path it made a chain with a decode behind it 52.8 -> 55.7 us, though the
+// selections alone were as fast.
+template <int D, int NT>
+__device__ __noinline__ void exact_nans(const SelectArgs& a, int b, int m_beg, int nt, int pitch, float* lg, const uint64_t* tf,
+                                        const uint8_t* ax) {
     constexpr int P = D / 2;
-    const uint16_t* q = a.q + (int64_t(b) * a.n_q_heads + hq) * D;
-    const uint16_t* k = a.store_k + int64_t(b) * a.store_seq_stride + int64_t(a.layer) * a.store_layer_stride +
-                        int64_t(m) * a.store_token_stride + int64_t(hq / (a.n_q_heads / a.n_kv_heads)) * D;
-    const int32_t* crd = a.coords + int64_t(b) * a.coord_seq_stride + 3 * int64_t(m);
+    const int64_t p = a.q_pos[b];
     auto value = [](uint16_t w) { return __uint_as_float(uint32_t(w) << 16); };
-    float sum = 0.0f;
-    for (int i = 0; i < P; ++i) {
-        float sn, cs;
-        sincos_coord(int64_t(crd[ax[i]]) - p, tf[i], &sn, &cs);
-        const float x = value(k[i]), y = value(k[i + P]);
-        sum = fmaf(value(q[i]), fmaf(x, cs, -y * sn), sum);
-        sum = fmaf(value(q[i + P]), fmaf(y, cs, x * sn), sum);
+    for (int e = threadIdx.x; e < a.n_q_heads * nt; e += NT) {
+        const int hq = e / nt, t = e - hq * nt;
+        if (lg[hq * pitch + t] == lg[hq * pitch + t]) continue;
+        const uint16_t* q = a.q + (int64_t(b) * a.n_q_heads + hq) * D;
+        const uint16_t* k = a.store_k + int64_t(b) * a.store_seq_stride + int64_t(a.layer) * a.store_layer_stride +
+                            int64_t(m_beg + t) * a.store_token_stride + int64_t(hq / (a.n_q_heads / a.n_kv_heads)) * D;
+        const int32_t* crd = a.coords + int64_t(b) * a.coord_seq_stride + 3 * int64_t(m_beg + t);
+        float sum = 0.0f;
+        for (int i = 0; i < P; ++i) {
+            float sn, cs;
+            sincos_coord(int64_t(crd[ax[i]]) - p, tf[i], &sn, &cs);
+            const float x = value(k[i]), y = value(k[i + P]);
+            sum = fmaf(value(q[i]), fmaf(x, cs, -y * sn), sum);
+            sum = fmaf(value(q[i + P]), fmaf(y, cs, x * sn), sum);
+        }
+        lg[hq * pitch + t] = sum * a.scale;
     }
-    return sum * a.scale;
+    __syncthreads();
 }
 
 // Logits of tokens m_beg .. m_beg + nt - 1 of sequence b for the query heads of
@@ -815,19 +824,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
     cta_logits<D, CACHED, NT>(a, f, b, 0, a.n_kv_heads, m_beg, nt, smem_raw, pt, lg_s, f.pitch, err);
     if (CACHED && err) atomicOr(a.status, err);
     __syncthreads();
-    const bool nan = cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
     if constexpr (D == 256 && !CACHED) {
-        if (__syncthreads_or(nan)) {
-            for (int e = tid; e < Hq * nt; e += NT) {
-                const int h = e / nt, t = e - h * nt;
-                float& x = lg_s[h * f.pitch + t];
-                if (x != x) x = raw_logit<D>(a, b, h, m_beg + t, a.q_pos[b], pt.tf, pt.ax);
-            }
-            __syncthreads();
-            cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
-            __syncthreads();
-        }
+        for (bool again = true; __syncthreads_or(cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat)) && again; again = false)
+            exact_nans<D, NT>(a, b, m_beg, nt, f.pitch, lg_s, pt.tf, pt.ax);
     } else {
+        cta_stats<NT>(lg_s, f.pitch, Hq, nt, sh.stat);
         __syncthreads();
     }
     merge_stats<NT, false>(a, C, rank, sh);
