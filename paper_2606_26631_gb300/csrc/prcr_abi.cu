@@ -246,23 +246,26 @@ int layers_per_cta(int64_t tiles, int n_layers, int64_t slots) {
 }
 
 // Layers each CTA walks in the kernels that stream rows from HBM (rebind,
-// capture): the fewest, up to `few`, that make one wave; else `few`, so that
-// many short CTAs overlap one another's prologues and end together; `many`
-// where that would still be over 32 waves, whose tail no longer shows. Groups
-// are evened out. Measured, rebind (few 4, many 12; groups picked for full
-// waves before): 5 sequences x ~800 tokens x 10 layers 45.8 -> 38.9 us, 16 x
-// ~512 x 4 37.3 -> 32.0 us; 4 for 16 x 4 x 640 tokens x 36 layers 1697 us, 18
-// 1688 us. Capture (2 and 2): 3 x 768 tokens x 36 layers x 8 heads 158 us at
-// 2, 161 at 4, 165 at 7; one image of 8192 531 us at 2 and 4, 541 before.
-int stream_layers_per_cta(int64_t tiles, int n_layers, int64_t slots, int few, int many) {
-    if (n_layers > 65535) return layers_per_cta(tiles, n_layers, slots);  // grid y
+// capture): the fewest, up to `few`, that make at most `wave` CTAs; else `few`, so
+// that many short CTAs overlap one another's prologues and end together. Groups are
+// evened out. A CTA's cos/sin cost each thread 8 / n_kv_heads sincos, whatever
+// the layers: few heads want longer groups.
+// Rebind (few 4 + 6 / heads; a wave is one and a half CTAs per SM): the best group of
+// 430 drawn revisits is 0.7 % faster on average, than of few 4 and a wave of all
+// resident CTAs 1.8 %; 16 sequences x 4 x 640 tokens x 36 layers x 8 heads 1674 us at
+// 4, 1676 at 6, 1685 at 12, 1689 at 18; with one head of 256 x 21 layers x 2070 tokens groups of 4 take
+// 33, of 11 22 us, with eight of 128 x 22 x 1344 of 4 42.6, of 11 43.5. Capture (few 6
+// / heads, two at least; a wave is all resident CTAs): one head of 128 x 18 layers x
+// 3410 tokens 90 us at 2, 71 at 6; eight x 36 x 768 x 3 images 158 at 2, 161 at 4.
+int stream_layers_per_cta(int64_t tiles, int n_layers, int64_t wave, int few) {
+    if (n_layers > 65535) return layers_per_cta(tiles, n_layers, wave);  // grid y
     auto even = [&](int g) {
         const int groups = (n_layers + g - 1) / g;
         return (n_layers + groups - 1) / groups;
     };
     for (int g = 1; g < few; ++g)
-        if (tiles * ((n_layers + g - 1) / g) <= slots) return even(g);
-    return even(tiles * ((n_layers + few - 1) / few) > 32 * slots ? many : few);
+        if (tiles * ((n_layers + g - 1) / g) <= wave) return even(g);
+    return even(few);
 }
 
 // Arguments and launch shape of the row-moving kernel (rebind or fused).
@@ -317,8 +320,9 @@ int rebind_setup(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
     const int64_t tiles = (b->total_k + T - 1) / T;
     const int64_t slots = int64_t(sm_count(dev)) * blocks_per_sm(dev, block, smem, kernel);
+    const int few = 4 + 6 / cfg->n_kv_heads;
     const int G = kernel == kFused ? layers_per_cta(tiles, cfg->n_layers, slots)
-                                   : stream_layers_per_cta(tiles, cfg->n_layers, slots, 4, 12);
+                                   : stream_layers_per_cta(tiles, cfg->n_layers, slots * 3 / 8, few);
     const int64_t groups = (cfg->n_layers + G - 1) / G;
     a.layers_per_cta = G;
     a.early_ctas = after_plan ? int32_t(slots) : 0;
@@ -403,7 +407,8 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
     if (cudaGetDevice(&dev) != cudaSuccess) return PRCR_ECUDA;
     const int64_t tiles = (int64_t(m_count) + T - 1) / T;
     const int64_t slots = int64_t(sm_count(dev)) * blocks_per_sm(dev, block, smem, kCapture);
-    const int G = stream_layers_per_cta(tiles, n_layers, slots, 2, 2);
+    const int few = std::max(2, 6 / cfg->n_kv_heads);
+    const int G = stream_layers_per_cta(tiles, n_layers, slots, few);
     a.layers_per_cta = G;
     const dim3 grid(unsigned(tiles), unsigned((n_layers + G - 1) / G), 1);
     return launch_capture(a, grid, block, smem, stream) == cudaSuccess ? PRCR_OK : PRCR_ECUDA;

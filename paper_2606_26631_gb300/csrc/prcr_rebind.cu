@@ -14,15 +14,19 @@
 // instead of the ~2e-3 of a float32 product.
 // Each thread owns one (token, head, 16-byte vector v) slot of the row: it
 // loads the 8 bf16 of the first half at v and the 8 bf16 of the second half
-// at v + D/2 (the rotate-half partners), for K and V, and walks the G layers
-// two at a time. Consecutive threads cover consecutive 16-byte vectors of a
+// at v + D/2 (the rotate-half partners), for K and V, and walks the G
+// layers, two in flight. Consecutive threads cover consecutive 16-byte vectors of a
 // row, so every warp-wide load and store is a set of whole 128-byte lines.
 //
-// HBM-bound. The first two layers' loads go out before the cos/sin, whose
-// latency they hide: measured 16 sequences x 4 x 640 tokens x 36 layers x 8
-// heads of 128 (11.5 GB) 1689 -> 1684 us (6.83 TB/s), 8 x ~512 x 28 x 4 (0.47
-// GB) 84.0 -> 82.1 us, the smaller ones mostly from their layer groups. One
-// layer ahead of the one stored instead (72 registers): 97 us for the second.
+// HBM-bound where there are many rows. The first layer's loads go out before the
+// cos/sin, whose latency they hide. 64 registers, four CTAs of 256 threads per SM:
+// with two layers requested ahead (75 registers, three CTAs) few heads or few layers,
+// whose cos/sin weigh most, were slower than with none. Whole revisits in us, no
+// layer ahead | two | one (each with its own rule for the groups of layers, the last
+// stream_layers_per_cta's): 8 sequences x ~512 tokens x 28 layers x 4 heads of 128
+// (0.47 GB) 84.4 | 81.5 | 80.5, 3 x ~650 x 6 x 8 14.3 | 16.0 | 13.1, 3 x ~3700 x 5 x 3
+// 19.4 | 23.7 | 17.9, 9 x ~320 x 21 x 1 of 256 33.3 | 43.9 | 29.2; 16 x 4 x 640 x 36 x
+// 8 (11.5 GB) 1684 | 1680 | 1674 (6.9 TB/s).
 //
 // The kernel is launched with programmatic dependent launch behind the plan
 // kernel and waits on it (griddepcontrol.wait) before touching the plan; its
@@ -64,7 +68,7 @@ __device__ __forceinline__ void prefetch_rows(const RebindArgs& a) {
     }
 }
 
-__global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ RebindArgs a) {
+__global__ void __launch_bounds__(512, 2) rebind_kernel(const __grid_constant__ RebindArgs a) {
     extern __shared__ __align__(16) float smem[];
     pdl_allow();
     if (int64_t(blockIdx.y) * gridDim.x + blockIdx.x < a.early_ctas) prefetch_rows(a);
@@ -92,23 +96,15 @@ __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ Reb
     const int64_t sls = a.store_layer_stride;
     const int64_t cls = a.cache_layer_stride;
     const int64_t s_off = (dst < 0 ? 0 : a.plan_src[my_tok]) + int64_t(l0) * sls + off;
-    const uint16_t* sk = a.store_k + s_off;
-    const uint16_t* sv = a.store_v + s_off;
-    // two layers' vectors (K and its rotate-half partner, V likewise), the
-    // first two requested before the cos/sin
-    uint4 x[2][4];
-    auto load = [&](int n) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (u < n) {
-                x[u][0] = ld_stream(sk + u * sls);
-                x[u][1] = ld_stream(sk + u * sls + P);
-                x[u][2] = ld_stream(sv + u * sls);
-                x[u][3] = ld_stream(sv + u * sls + P);
-            }
-        }
-    };
-    if (dst >= 0) load(l1 - l0);
+    // the first layer's vectors (K and its rotate-half partner, V likewise),
+    // requested before the cos/sin
+    uint4 x[4];
+    if (dst >= 0) {
+        x[0] = ld_stream(a.store_k + s_off);
+        x[1] = ld_stream(a.store_k + s_off + P);
+        x[2] = ld_stream(a.store_v + s_off);
+        x[3] = ld_stream(a.store_v + s_off + P);
+    }
 
     for (int q = threadIdx.x; q < T * P; q += blockDim.x) {
         const int t = q / P;
@@ -135,23 +131,16 @@ __global__ void __launch_bounds__(512) rebind_kernel(const __grid_constant__ Reb
         s[0] = s0.x; s[1] = s0.y; s[2] = s0.z; s[3] = s0.w;
         s[4] = s1.x; s[5] = s1.y; s[6] = s1.z; s[7] = s1.w;
     }
-    uint16_t* ck = a.cache_k + dst + int64_t(l0) * cls + off;
-    uint16_t* cv = a.cache_v + dst + int64_t(l0) * cls + off;
-    for (int l = l0; l < l1; l += 2) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (l + u < l1) {
-                uint4 o0, o1;
-                rotate_vec(x[u][0], x[u][1], c, s, o0, o1);
-                st_row(ck + u * cls, o0);
-                st_row(ck + u * cls + P, o1);
-                st_row(cv + u * cls, x[u][2]);
-                st_row(cv + u * cls + P, x[u][3]);
-            }
-        }
-        sk += 2 * sls; sv += 2 * sls; ck += 2 * cls; cv += 2 * cls;
-        load(l1 - l - 2);
-    }
+    const int64_t c_off = dst + int64_t(l0) * cls + off;
+    uint16_t* ck = a.cache_k + c_off;
+    uint16_t* cv = a.cache_v + c_off;
+    uint4 o0, o1;
+    rotate_vec(x[0], x[1], c, s, o0, o1);
+    st_row(ck, o0);
+    st_row(ck + P, o1);
+    st_row(cv, x[2]);
+    st_row(cv + P, x[3]);
+    stream_layers(a.store_k + s_off + sls, a.store_v + s_off + sls, ck + cls, cv + cls, sls, cls, P, l1 - l0 - 1, c, s);
 }
 
 }  // namespace

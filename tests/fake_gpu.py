@@ -92,3 +92,10 @@ def paged(c, seqs, blocks_per_seq, block, n_blocks=1024):
     row = c.n_kv_heads * c.head_dim
     return B.CacheDesc(kind=1, block_size=block, k=FAKE, v=FAKE, seq_stride=0, layer_stride=1024 * block * row, block_stride=block * row,
                        slot_stride=row, block_table=FAKE, bt_stride=blocks_per_seq, n_blocks=n_blocks, max_slots=0, n_seqs=seqs)
+
+
+def capture(c, tokens):
+    st, ca = store(c, 1, tokens), contiguous(c, 1, tokens)
+    row = c.n_kv_heads * c.head_dim
+    return lib().prcr_prefill_capture(C.byref(c), C.byref(st), C.byref(ca), 0, 0, c.n_layers, 0, tokens, 0, FAKE, FAKE, tokens * row, row,
+                                      FAKE, FAKE, None)

@@ -106,3 +106,17 @@ def test_cached_selection_of_a_cache_without_rows(n_tokens):
         F.launches()
         assert F.select_cached(c, 4, 4, n_tokens, cache) == 0
         assert F.launches()[0][1][5] == first_row
+
+
+def test_few_heads_take_longer_layer_groups():
+    """A CTA's cos/sin cost as much for one KV head as for eight: with few heads
+    a CTA walks more layers (rebind and capture), with eight as few as four and
+    two."""
+    for H, D, L, tokens, rebind, capture in ((1, 256, 21, 2916, 3, None), (2, 128, 23, 20000, 4, None), (8, 128, 36, 4000, 9, None),
+                                             (1, 128, 18, 3410, None, 3), (2, 128, 12, 6048, None, 4), (8, 128, 12, 6048, None, 6)):
+        c = F.cfg(L, H, D)
+        F.launches()
+        if rebind:
+            assert F.revisit(c, 1, tokens) == 0 and F.launches()[1][1][1] == rebind, (H, D)
+        else:
+            assert F.capture(c, tokens) == 0 and F.launches()[0][1][1] == capture, (H, D)
