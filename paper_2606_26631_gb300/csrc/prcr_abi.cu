@@ -444,10 +444,16 @@ int do_capture(const prcr_rope_cfg* cfg, const prcr_store_desc* store,
 // layers x 4 heads of up to 4096 slots 205 | 213 | 208 | 208 | 200, of up to 8192
 // 404 | 404 | 394 | 384 | 390, 6 of up to 4096 180 | 175 | 169 | 169 | 166; 16 x 36
 // x 8 of up to 4096 851 | 856 | 833 | 828 | 826; 16 x 28 x 4 of up to 900 103 | 94;
-// teams of six and twelve 174 and 169 for the third. head_dim 64: one warp on 512
+// teams of six and twelve 174 and 169 for the third. Two or three sequences of few
+// waves, whose last one shows: half those chunks, where the group is at most 4 query
+// heads (the partials are in proportion to it): 2 sequences x 36 layers x 8 heads, 4096
+// and 2976 slots 177 us at 2048 slots per chunk, 169 at 1024 (161 with CTAs looping over
+// the KV heads, before the teams), 6000 and 4025 242 | 234 (226), 3 x 36 x 8 of up to
+// 3000 with seven draws of lengths 5.6 % less; six sequences of 36 x 4 up to 4096 lose
+// 5 % by it. head_dim 64: one warp on 512
 // (8 x 28 x 4 of up to 4096 110 us, teams 114; 12 x 28 x 8 326, 333).
 template <int D>
-int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, int* team,
+int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, int group, int* team,
                      int64_t* most) {
     using Sh = DecodeShape<D>;
     constexpr int kPerSm = Sh::kCtas * Sh::kWarps;
@@ -479,6 +485,12 @@ int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, in
         const int64_t longest = Sh::kChunk * std::max(1, *team);
         splits = (max_len + longest - 1) / longest;
         *most = std::max(*most, splits);
+        if (*team && group <= 4 && n_seqs <= 3) {
+            const int64_t n = (4 * int64_t(sms) * (kPerSm / *team) - 1) / units;  // the most chunks under four waves
+            const int64_t halves = (max_len + longest / 2 - 1) / (longest / 2);
+            *most = std::max(*most, std::min(halves, 2 * n));
+            if (splits > 1 && splits <= n) splits = halves;
+        }
         return *team ? (tiles + splits - 1) / splits * 16 : longest;
     }
     // the fewest warps that take as many rounds of tiles
@@ -514,12 +526,12 @@ int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms, int64_t* most
 }
 
 void decode_split(int64_t n_seqs, int n_layers, int64_t max_len, int sms, int n_kv_heads,
-                  int head_dim, int* splits, int* chunk, int* team, int64_t* most) {
+                  int group, int head_dim, int* splits, int* chunk, int* team, int64_t* most) {
     const int64_t units = n_seqs * n_layers * n_kv_heads;
     max_len = std::min<int64_t>(max_len, INT32_MAX);  // a sequence's length is an int32
     *team = 0;
-    int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, team, most)
-                      : head_dim == 128 ? decode_chunk<128>(n_seqs, units, max_len, sms, team, most)
+    int64_t c = head_dim == 64    ? decode_chunk<64>(n_seqs, units, max_len, sms, group, team, most)
+                      : head_dim == 128 ? decode_chunk<128>(n_seqs, units, max_len, sms, group, team, most)
                                         : decode_wide_chunk(units, max_len, sms, most);
     c = std::min<int64_t>(c, 1 << 30);
     *chunk = int(c);
@@ -716,7 +728,7 @@ size_t prcr_decode_workspace_size(const prcr_rope_cfg* cfg, int32_t n_seqs, int3
     if (cudaGetDevice(&dev) == cudaSuccess) sms = sm_count(dev);
     int splits = 1, chunk = 32, team = 0;
     int64_t most = 1;
-    decode_split(n_seqs, cfg->n_layers, max_len, sms, cfg->n_kv_heads, cfg->head_dim,
+    decode_split(n_seqs, cfg->n_layers, max_len, sms, cfg->n_kv_heads, n_q_heads / cfg->n_kv_heads, cfg->head_dim,
                  &splits, &chunk, &team, &most);
     if (most == 1) return 0;
     return size_t(n_seqs) * cfg->n_layers * n_q_heads * most * (cfg->head_dim + 2) * sizeof(float);
@@ -745,7 +757,7 @@ int prcr_decode_attention(const prcr_rope_cfg* cfg, const prcr_cache_desc* cache
     DecodeArgs a = {};
     int64_t most;
     decode_split(n_seqs, cfg->n_layers, max_len, sm_count(dev), cfg->n_kv_heads,
-                 cfg->head_dim, &a.splits, &a.chunk, &a.team, &most);
+                 n_q_heads / cfg->n_kv_heads, cfg->head_dim, &a.splits, &a.chunk, &a.team, &most);
     if (n_seqs > 65535 || cfg->n_layers > 65535) return PRCR_EINVAL;  // grid z and y
     if (a.splits > 1) {
         const size_t need = size_t(n_seqs) * cfg->n_layers * n_q_heads * a.splits *

@@ -120,3 +120,14 @@ def test_few_heads_take_longer_layer_groups():
             assert F.revisit(c, 1, tokens) == 0 and F.launches()[1][1][1] == rebind, (H, D)
         else:
             assert F.capture(c, tokens) == 0 and F.launches()[0][1][1] == capture, (H, D)
+
+
+def test_decode_chunks_of_few_long_sequences():
+    """Two or three long sequences under four waves of teams take chunks of 1024
+    slots, which even out their last wave; more sequences, more waves, or a
+    group of more than 4 query heads 2048."""
+    for L, H, seqs, group, n, want in ((36, 8, 2, 4, 4096, 1024), (36, 8, 3, 4, 3000, 1008), (11, 8, 3, 1, 8192, 1024), (36, 8, 2, 4, 8192, 2048),
+                                       (36, 4, 6, 4, 4096, 2048), (28, 4, 3, 7, 8192, 2048), (36, 8, 16, 4, 4096, 2048)):
+        F.launches()
+        assert F.decode(F.cfg(L, H, 128), seqs, group, n, 1 << 40) == 0
+        assert F.launches()[0][1][6:] == [want, 4], (L, H, seqs, group, n)
