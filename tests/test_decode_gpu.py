@@ -56,11 +56,10 @@ CASES = [  # (B, layers, H, Hq, D, max_len, paged)
     (2, 2, 2, 14, 64, 700, False),
     (2, 2, 4, 4, 256, 1200, True),
     (5, 1, 4, 28, 128, 9000, True),
-    # one sequence of the Table 3 shape (small batch: KV heads split over
-    # CTAs, chunk rows requested into L2 ahead of the tile loop)
+    # one sequence of the Table 3 shape (a team of six warps per KV head, unsplit)
     (1, 36, 8, 32, 128, 933, False),
     (2, 2, 8, 16, 64, 500, True),
-    # the head-split kernel at the ends of the GQA range: 1 and 8 query heads per KV head
+    # teams at the ends of the GQA range: 1 and 8 query heads per KV head
     (1, 2, 8, 8, 128, 500, False),
     (1, 2, 8, 64, 128, 300, True),
 ]
@@ -94,9 +93,8 @@ def test_decode_parity(case):
 def test_decode_empty_and_single_slot(H, Hq, D, paged):
     """A sequence with no slots gets zeros; one with a single slot gets that
     slot's V row exactly (its softmax weight is exactly 1); a longer one
-    beside them still matches the oracle. Covers the head-split kernel
-    (8 KV heads), the one-CTA-per-chunk kernel, head_dim 64 and the
-    head_dim 256 kernel."""
+    beside them still matches the oracle. Head dims 64, 128 and 256; the kernel
+    of one warp per chunk has its own such lengths in test_decode_large."""
     import paper_2606_26631_gb300 as prcr
     B, nL, max_len = 3, 2, 300
     sec = (D // 8, D // 8 + (D // 2 - 3 * (D // 8)) // 2, 0)
@@ -174,8 +172,8 @@ def test_decode_device_errors():
 def test_decode_query_position_range():
     """A query position of 2^31 or more is beyond the fixed-point angle
     reduction: PRCR_ST_POS_RANGE, and that sequence reads no slot (its output
-    is zeros) while the other sequence of the batch matches the oracle.
-    Head-split and one-CTA-per-chunk kernels, split and unsplit sequences."""
+    is zeros) while the other sequence of the batch matches the oracle. Teams
+    of warps, split and unsplit sequences."""
     import paper_2606_26631_gb300 as prcr
     sec = (16, 24, 24)
     for H, Hq, max_len in ((8, 32, 300), (2, 8, 300), (8, 32, 3000)):
@@ -228,8 +226,8 @@ def test_decode_unaligned_query():
                                              (1, 8, 128, True, 7), (5, 5, 128, False, 16), (3, 21, 64, True, 16)])
 @pytest.mark.parametrize("n_layers", [1, 9, 19, 40])
 def test_decode_edges(H, Hq, D, paged, bs, n_layers):
-    """Few layers: teams of warps per chunk (1) or per whole sequence (9 and 19:
-    of 12, 6, 4 and 2), many: one warp per chunk. head_dim 256: every product has 24 significant bits and is summed in
+    """Few layers: teams of warps per chunk (1) or per whole sequence (9, 19 and
+    40: of 12, 6, 4 and 2; head_dim 64 at 40: one warp per chunk). head_dim 256: every product has 24 significant bits and is summed in
     float32, so a logit (sum of ~10 in magnitude over 48 MMAs) is off by about
     sqrt(48) 2^-24 10 = 4e-6 and the output by no more than twice that. Below,
     the file's bar: 16 significant bits per operand, 10 * 2^-17 = 8e-5."""
@@ -262,6 +260,54 @@ def test_decode_edges(H, Hq, D, paged, bs, n_layers):
             K, V = (_f64(inp[x][b, l, :n]) for x in ("cache_k", "cache_v"))
         ref = O.decode_attention(qv[b, l], int(inp["q_pos"][b]), K, V, D, sec, 1e6)
         assert np.abs(got[b, l] - ref).max() / np.abs(V).max() <= (8e-6 if D == 256 else 1e-4), (b, n)
+
+
+# (B, layers, H, Hq, D, max_len, paged), and what the host launches on 152 SMs
+# (warps of a team or 0, chunks of max_len), which test_launch_cpu checks
+LARGE = [
+    ((1, 11, 3, 12, 128, 2000, True), (0, 42)),     # one warp per chunk, the merge of over 32
+    ((16, 23, 5, 10, 128, 600, False), (0, 1)),     # one warp per sequence: more than 12 units per SM, 5 of 8 warps in use
+    ((8, 23, 5, 10, 128, 700, True), (4, 1)),       # a large batch: teams of four, a chunk per sequence
+    ((8, 23, 5, 10, 128, 2049, False), (4, 2)),     # and just over a chunk's 2048
+    ((4, 28, 4, 28, 128, 4100, True), (4, 3)),      # and over two
+    ((3, 25, 8, 8, 128, 4097, False), (4, 5)),      # few long sequences: chunks of 1024 at most
+    ((16, 23, 5, 10, 64, 600, True), (0, 1)),       # head_dim 64
+    ((8, 23, 5, 10, 64, 1100, False), (0, 3)),
+]
+
+
+@pytest.mark.parametrize("case", [c for c, _ in LARGE], ids=["B%dL%dH%dHq%dD%dS%d" % c[:6] for c, _ in LARGE])
+def test_decode_large(case):
+    """Many units or long sequences: sequences of no slot, one, a tile and its
+    neighbours, a chunk of this call's and its neighbours, and max_len, at the
+    first and last layer. The file's bar."""
+    import paper_2606_26631_gb300 as prcr
+    B, nL, H, Hq, D, max_len, paged = case
+    sec = (D // 8, D // 4, D // 8)
+    c = -(-(-(-max_len // 16)) // dict(LARGE)[case][1]) * 16
+    lens = ([max_len, 0, 1, 17, c - 1, c, c + 1, 16] * 2)[:B] if B > 4 else [max_len, c + 1, c, 15][:B]
+    lens = [min(n, max_len) for n in lens]
+    g = torch.Generator(device=DEV).manual_seed(B + max_len)
+    bs, nblk = 16, -(-max_len // 16)
+    shape = (nL, B * nblk, bs, H, D) if paged else (B, nL, max_len, H, D)
+    ck, cv = (torch.randn(shape, device=DEV, generator=g, dtype=torch.bfloat16) for _ in range(2))
+    bt = torch.randperm(B * nblk, device=DEV, generator=g).to(torch.int32).view(B, nblk) if paged else None
+    q = torch.randn((B, nL, Hq, D), device=DEV, generator=g, dtype=torch.bfloat16)
+    q_pos = torch.arange(B, device=DEV, dtype=torch.int64) * 977 + max_len
+    cfg = prcr.rope_cfg(nL, H, D, sec, 1e6)
+    cd = prcr.cache_paged(ck, cv, bt) if paged else prcr.cache_contiguous(ck, cv)
+    out, st = _run_decode(cfg, cd, q, q_pos, torch.tensor(lens, dtype=torch.int32, device=DEV), max_len)
+    assert st == 0
+    got, qv = out.cpu().numpy(), _f64(q)
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert np.all(got[b] == 0.0)
+            continue
+        s = torch.arange(n, device=DEV)
+        for l in (0, nL - 1):
+            K, V = (_f64(x[l][bt[b][s // bs].long(), s % bs] if paged else x[b, l, :n]) for x in (ck, cv))
+            ref = O.decode_attention(qv[b, l], int(q_pos[b]), K, V, D, sec, 1e6)
+            assert np.abs(got[b, l] - ref).max() / np.abs(V).max() <= 1e-4, (b, l, n)
 
 
 def test_inject_then_decode():

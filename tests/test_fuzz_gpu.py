@@ -92,7 +92,7 @@ def _decode_case(i: int):
 
 @pytest.mark.parametrize("i", range(12))
 def test_fuzz_decode(i):
-    """Random decode shapes (chunking, head split, merge kernels and the
+    """Random decode shapes (teams of warps, chunks, merge kernels and the
     head_dim 256 kernel all vary with them) against the oracle."""
     import torch
     import paper_2606_26631_gb300 as prcr

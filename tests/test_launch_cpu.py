@@ -131,3 +131,16 @@ def test_decode_chunks_of_few_long_sequences():
         F.launches()
         assert F.decode(F.cfg(L, H, 128), seqs, group, n, 1 << 40) == 0
         assert F.launches()[0][1][6:] == [want, 4], (L, H, seqs, group, n)
+
+
+def test_decode_large_cases_reach_their_kernels():
+    """The GPU test's shapes take the kernel, the team and the split they name."""
+    from test_decode_gpu import LARGE
+    for (B, layers, H, Hq, D, max_len, _), (team, splits) in LARGE:
+        F.launches()
+        assert F.decode(F.cfg(layers, H, D), B, Hq // H, max_len, 1 << 40) == 0
+        kernel, *merge = F.launches()
+        assert f"decode_kernelILi{D}ELb{int(team > 0)}E" in kernel[0]
+        assert [kernel[1][5], kernel[1][7]] == [splits, team] and len(merge) == (splits > 1), (B, layers, H)
+        if splits > 1:
+            assert ("warp" in merge[0][0]) == (splits <= 32)
