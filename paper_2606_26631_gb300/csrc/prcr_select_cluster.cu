@@ -856,18 +856,22 @@ __global__ void __launch_bounds__(kFusedThreads, 1) select_fused_kernel(const __
 
 // Logits of the cached-key selection to global memory, where it is too large for
 // one cluster per sequence: a CTA takes one (sequence, chunk of tok_per_cta
-// tokens, group of kh_per_item KV heads), two CTAs per SM, so that one's set-up
-// runs beside the other's streaming. DRAM bounds it, with 64 KB of keys in flight
-// per SM; these need lines of L1, so shared memory is kept small (logits staged
+// tokens, group of kh_per_item KV heads), two CTAs per SM (four at head_dim 64,
+// whose items are half as long), so that one's set-up runs beside the other's
+// streaming. DRAM bounds it, with 64 KB of keys in flight per SM; these need lines of L1, so shared memory is kept small (logits staged
 // there for whole-line stores and statistics, 200 KB per SM, made it 2 to 3
 // times slower). Measured against a kernel whose warps each looked up their rows
 // per item and loaded 64 bytes per lane (half a sector per load), whole selections:
 // 16 sequences of 8192 tokens x 8 heads of 128 66.8 -> 63.1 us, 32 of 16,384 212.6
-// -> 206.0 us, 16 of 4096 40.1 -> 36.6 us, 7 of 8192 40.3 -> 36.0 us.
+// -> 206.0 us, 16 of 4096 40.1 -> 36.6 us, 7 of 8192 40.3 -> 36.0 us. Head_dim
+// 64, 32 sequences of 8192 x 8 heads, before | two | three | four | five CTAs per SM:
+// 71.9 | 76.3 | 61.6 | 59.8 | 73.6.
 constexpr int kSplitThreads = 256;
+template <int D>
+constexpr int kSplitCtas = D == 64 ? 4 : 2;  // per SM
 
 template <int D>
-__global__ void __launch_bounds__(kSplitThreads, 2) select_logits_kernel(const __grid_constant__ SelectArgs a) {
+__global__ void __launch_bounds__(kSplitThreads, kSplitCtas<D>) select_logits_kernel(const __grid_constant__ SelectArgs a) {
     constexpr int NT = kSplitThreads;
     __shared__ PairTables<D, true, NT> pt;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -998,15 +1002,15 @@ cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t str
     return cudaLaunchKernelEx(&cfg, kern, t);
 }
 
-// Chunks of the cached-key logits: as many per sequence as make one wave of two
-// CTAs per SM, of at least kSplitMinTokens tokens and at most kSplitMaxTokens.
+// Chunks of the cached-key logits: as many per sequence as make one wave of
+// kSplitCtas CTAs per SM, of at least kSplitMinTokens tokens and at most kSplitMaxTokens.
 template <int D>
 cudaError_t launch_logits_split(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream) {
     SelectArgs t = a;
     const int H = a.n_kv_heads, g = a.n_q_heads / H;
     t.kh_per_item = H < 1024 / D ? H : 1024 / D;  // 32 KB of query fragments at most
     const int64_t per = int64_t(n_seqs) * ((H + t.kh_per_item - 1) / t.kh_per_item);
-    const int64_t n = std::max<int64_t>(1, 2 * int64_t(sms) / per);
+    const int64_t n = std::max<int64_t>(1, kSplitCtas<D> * int64_t(sms) / per);
     const int64_t T = std::min<int64_t>(kSplitMaxTokens, std::max<int64_t>(kSplitMinTokens, (a.n_tokens + n - 1) / n));
     t.tok_per_cta = int((T + 15) / 16 * 16);
     const size_t smem = fused_layout(D, true, t.kh_per_item, t.kh_per_item * g, t.tok_per_cta, 0, false).total;

@@ -144,3 +144,14 @@ def test_decode_large_cases_reach_their_kernels():
         assert [kernel[1][5], kernel[1][7]] == [splits, team] and len(merge) == (splits > 1), (B, layers, H)
         if splits > 1:
             assert ("warp" in merge[0][0]) == (splits <= 32)
+
+
+@pytest.mark.parametrize("D,ctas", [(64, 4), (128, 2), (256, 2)])
+def test_cached_logits_fill_the_gpu_once(D, ctas):
+    """A large cached selection's logits: one wave of four CTAs per SM at
+    head_dim 64 (whose rows are half as long), of two above."""
+    F.launches()
+    assert F.select_cached(F.cfg(1, 4, D), 8, 4, 16384) == 0
+    logits, tail = F.launches()
+    assert "select_logits" in logits[0] and "select_tail" in tail[0]
+    assert 0.9 * 152 * ctas < logits[1][0] <= 152 * ctas
