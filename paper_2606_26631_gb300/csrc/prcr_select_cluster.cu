@@ -908,7 +908,6 @@ cudaLaunchConfig_t cluster_config(int grid, int block, int C, size_t smem, cudaS
 }
 
 constexpr int kFusedMinTokens = 32;  // per CTA
-constexpr int kFusedRowsRaw = 640, kFusedRowsCached = 1152;
 constexpr int kSplitMinTokens = 64, kSplitMaxTokens = 2048;  // per CTA of the logits kernel
 constexpr size_t kMaxDynSmem = 192 * 1024;  // beside the static shared memory, within 227 KB
 
@@ -974,15 +973,25 @@ cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, bool fine, cudaS
 
 // The one-kernel selection, or *done = false where it does not fit or is the
 // slower path. It leaves SMs idle (a cluster per sequence, and clusters do not
-// fill every GPC), so its time grows with the rows (token, KV head) of a CTA,
-// that of a logits kernel and select_tail_kernel with all rows over all SMs,
-// on top of ~6 us more for the second kernel. Measured (us, fused | two
-// kernels), raw keys, 8 heads of 128: 1 sequence of 1024 tokens (512 rows per
-// CTA) 13.0 | 15.2, of 2048 17.7 | 16.3, of 4096 27.8 | 18.1; 7 of 2048 (1024
-// rows) 19.1 | 27.1, of 4096 29.4 | 32.8, of 8192 61.9 | 43.8; 16 of 1024 21.0
-// | 28.9, of 2048 34.3 | 34.7. Cached keys: 1 of 1024 12.4 | 16.2, of 2048
-// 15.3 | 17.5, of 4096 20.0 | 19.0; 7 of 4096 22.5 | 25.5, of 8192 35.9 | 36.6; 16
-// of 2048 23.7 | 24.7, of 4096 40.3 | 36.6. The line below lies between them.
+// fill every GPC), so its time grows with the work of a CTA, that of a logits
+// kernel and select_tail_kernel with all work over all SMs, on top of a few us more
+// for the second kernel. Work is counted in key rows (token, KV head), to which raw
+// keys add about three per token for its cos/sin; the second path grows with their
+// number per SM, at first faster (its grids fill) than in proportion. The constants are
+// fitted per head_dim to 41,871 drawn calls timed both ways (1..48 sequences of
+// 128..16,384 tokens, 1..8 KV heads, groups of 1..7): the chosen path is 0.1 to 0.4 %
+// behind the better one on average; with one line for all head dims, linear, in rows of
+// 128, 0.6 to 2.6 % and twice as slow at worst. Some of them, us, fused | two kernels: raw
+// keys, 8 heads of 128, 1 sequence of 1024 tokens 12.2 | 12.9, of 1536 14.2 | 13.3; 7 of
+// 4096 27.5 | 30.2; 40 of 2048 x 8 heads of 64 46.0 | 36.2, 7 of 8192 37.1 | 29.9; 1 of
+// 1024 x 8 of 256 18.0 | 26.3. Cached keys, 8 heads of 128, 1 of 2048 13.3 | 13.7, of
+// 3072 15.8 | 14.7; 7 of 4096 18.8 | 19.8; 16 of 4096 43 | 35; 8 heads of 256, 7 of 1536
+// 16.6 | 17.2, of 3072 24.4 | 22.9.
+struct FusedLine {
+    double rows, linear, root;
+};
+constexpr FusedLine kFusedLine[2][3] = {{{500, 0.45, 55}, {330, 0.2, 55}, {370, 1.7, 43}},   // raw keys: head_dim 64, 128, 256
+                                        {{740, 0.15, 34}, {600, 0.65, 17}, {280, 0.7, 17}}};  // cached keys
 template <int D, bool CACHED>
 cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream, bool* done) {
     auto kern = select_fused_kernel<D, CACHED>;
@@ -992,10 +1001,10 @@ cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t str
     if (e != cudaSuccess) return e;
     t.tok_per_cta = tokens_per_cta(a.n_tokens, t.cluster);
     const FusedLayout f = fused_layout(D, CACHED, a.n_kv_heads, a.n_q_heads, t.tok_per_cta, t.cluster);
-    const int64_t rows = int64_t(t.tok_per_cta) * a.n_kv_heads * D / 128;
-    const int64_t spread = int64_t(n_seqs) * a.n_tokens * a.n_kv_heads * D / 128 / sms;
-    // (the other path's logits kernel for raw keys of head_dim 256 takes ~3 times as long)
-    if (f.total > kMaxDynSmem || rows > (CACHED ? kFusedRowsCached : kFusedRowsRaw) + spread * (D == 256 && !CACHED ? 3 : 1)) return cudaSuccess;
+    const int64_t per_token = a.n_kv_heads + (CACHED ? 0 : 3);
+    const double spread = double(n_seqs) * a.n_tokens * per_token / sms;
+    const FusedLine c = kFusedLine[CACHED][D / 128];
+    if (f.total > kMaxDynSmem || double(t.tok_per_cta * per_token) > c.rows + c.linear * spread + c.root * std::sqrt(spread)) return cudaSuccess;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kFusedThreads, t.cluster, f.total, stream, attr);
     *done = true;
