@@ -505,9 +505,9 @@ int64_t decode_chunk(int64_t n_seqs, int64_t units, int64_t max_len, int sms, in
 // CTAs per SM with chunks of at least kWideMinChunk slots; where that is less
 // than two waves, one wave. Chunks are whole rounds of the CTA's warps, so a
 // longer max_len may be split into fewer; *most bounds what any up to it is.
-// Measured: 16 sequences x 26 layers x 4 heads of up to 4096 slots 822 us at 8
-// waves, 852 us at 16; 4 sequences of up to 2000 slots 162 us at 576 slots,
-// 178 us at 384.
+// Measured (before the logits' sums were shortened): 16 sequences x 26 layers x 4
+// heads of up to 4096 slots 822 us at 8 waves, now 797, 852 us at 16; 4 sequences of
+// up to 2000 slots 162 us at 576 slots, 178 us at 384.
 constexpr int64_t kWideMinChunk = 576;
 int64_t decode_wide_chunk(int64_t units, int64_t max_len, int sms, int64_t* most) {
     constexpr int64_t round = 16 * kDecodeWideWarps, longest = kDecodeMaxChunk / round * round;
@@ -548,7 +548,7 @@ bool decode_shape_ok(const prcr_rope_cfg* cfg, int32_t n_q_heads) {
 }
 
 // Checks and fills what both selection entry points share: heads, k, the
-// output pointers and the workspace, laid out for token tiles of `tile`.
+// output pointers and the workspace; `tile`: tokens per tile of the logits kernel.
 int select_common(const prcr_rope_cfg* cfg, int32_t n_seqs, int32_t layer, int32_t n_q_heads,
                   int32_t n_tokens, const void* q, const int64_t* q_pos, int32_t k,
                   int32_t* idx_out, int32_t* seq_rev_off, int32_t* rev_tok_off, float* score_out,

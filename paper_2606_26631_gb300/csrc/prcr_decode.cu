@@ -5,10 +5,10 @@
 //
 // The step is memory-bound: every cached K/V row is read once. Warps take
 // chunks of slots of one KV head of one (sequence, layer) and stream them in
-// tiles of 16 slots through tensor cores: one warp a chunk at head_dim 64 and
-// 128 (decode_kernel), three at 256 (decode_wide_kernel). Chunks of one
-// (sequence, layer) are merged by a further kernel from (max, sum, accumulator)
-// partials when the sequence is split.
+// tiles of 16 slots through tensor cores: at head_dim 64 and 128 (decode_kernel)
+// a team of 2 to 12 warps a chunk, or one warp, by decode_chunk's rule; at 256
+// (decode_wide_kernel) three. Chunks of one (sequence, layer) are merged by a
+// further kernel from (max, sum, accumulator) partials when the sequence is split.
 #include <cmath>
 
 #include <cuda_bf16.h>
@@ -66,9 +66,10 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
 // are bf16 already and enter exactly. A tile's P V is summed from zero and
 // added to the running accumulator by the FMA that rescales it.
 // TEAM: a CTA of up to kDecodeMaxTeam warps takes one unit, its warps the chunk's
-// tiles in turn, and merges their (max, sum, accumulator) in shared memory, so
-// that a small batch needs no chunks and no merge kernel (29.2 -> 25.2 us for one
-// sequence of 933 slots x 36 layers x 8 heads; the rule is decode_chunk's).
+// tiles in turn, and merges their (max, sum, accumulator) in shared memory. A small
+// batch mostly needs no chunks and no merge kernel that way (29.2 -> 25.2 us for one
+// sequence of 933 slots x 36 layers x 8 heads); a large one at head_dim 128 takes
+// teams of four on longer chunks, a quarter of the partials to merge.
 // DRAM bounds it: an SM's 12 warps keep ~100 KB in flight (~2.2 us at its share
 // of the copy rate). Measured, before | now (before: a CTA looping over the KV
 // heads with K in registers for large batches, CTAs of four heads each for

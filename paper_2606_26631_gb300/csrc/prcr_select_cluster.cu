@@ -346,9 +346,9 @@ __device__ __forceinline__ void tail_stats(const float* lg, int M, int Hq, int n
 // us: statistics 13k cycles, relevances 11k, the two exchanges 7k, search 6k,
 // output 3k. Measured against the three kernels it replaced (normaliser,
 // relevance, a top-k of one CTA per sequence counting two bits a round), whole
-// selections: that shape 262 -> 244 us, 16 x 8192 cached 72.8 -> 66.9 us, one
-// sequence of 16,384 43.9 -> 35.4 us; one of 64 tokens, where the chain of
-// exchanges shows, 10.5 -> 14 us of GPU time but 21 -> 16 us with its launches.
+// selections: that shape 262 -> 243.5 us, one sequence of 16,384 43.9 -> 36 us; one of
+// 64 tokens x 4 heads of 112, where the chain of exchanges shows, 19.0 -> 13.6 us in a
+// row, as a CUDA graph 12.8 | 12.8.
 constexpr int kTailThreads = 1024;
 constexpr int kTailMinTokens = 64;  // per CTA
 
