@@ -28,7 +28,8 @@
 namespace prcr {
 namespace {
 
-__global__ void __launch_bounds__(512) capture_kernel(const __grid_constant__ CaptureArgs a) {
+template <int THREADS, int CTAS, bool AHEAD>
+__global__ void __launch_bounds__(THREADS, CTAS) capture_kernel(const __grid_constant__ CaptureArgs a) {
     extern __shared__ __align__(16) float smem[];
     const int D = a.head_dim;
     const int P = D >> 1;
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(512) capture_kernel(const __grid_constant__ Ca
     };
     pdl_allow();
     pdl_wait();
-    if (act) load();
+    if (AHEAD && act) load();
 
     for (int t = threadIdx.x; t < T; t += blockDim.x) {
         const int j = tok0 + t;
@@ -120,10 +121,11 @@ __global__ void __launch_bounds__(512) capture_kernel(const __grid_constant__ Ca
     uint16_t* ck = a.cache_k + c_off;
     uint16_t* cv = a.cache_v + c_off;
     for (int l = l0; l < l1; ++l) {
+        if (!AHEAD) load();
         const uint4 x0 = k0, x1 = k1, y0 = v0, y1 = v1;
         sk += a.src_layer_stride;
         sv += a.src_layer_stride;
-        if (l + 1 < l1) load();
+        if (AHEAD && l + 1 < l1) load();
         st_row(rk, x0);
         st_row(rk + P, x1);
         st_row(rv, y0);
@@ -143,13 +145,23 @@ __global__ void __launch_bounds__(512) capture_kernel(const __grid_constant__ Ca
 
 }  // namespace
 
+namespace {
+
+// Rows of more than 384 threads (n_kv_heads x head_dim > 6144): without a layer
+// ahead, in 64 registers, or the CTA is alone on its SM. 64 heads of 128, 2 images of 5920 tokens x 2 layers 402
+// -> 350 us, one of 1600 x 24 605 -> 554; up to 384 threads two CTAs fit as they are.
+using CaptureKernel = void (*)(CaptureArgs);
+CaptureKernel capture_for(int block) { return block > 384 ? capture_kernel<512, 2, false> : capture_kernel<384, 1, true>; }
+
+}  // namespace
+
 cudaError_t capture_blocks_per_sm(int block, size_t smem, int* out) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, capture_kernel, block, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, capture_for(block), block, smem);
 }
 
 cudaError_t launch_capture(const CaptureArgs& a, dim3 grid, int block, size_t smem,
                            cudaStream_t stream) {
-    return launch_pdl(capture_kernel, grid, dim3(unsigned(block)), smem, stream, a);
+    return launch_pdl(capture_for(block), grid, dim3(unsigned(block)), smem, stream, a);
 }
 
 }  // namespace prcr

@@ -206,3 +206,31 @@ def test_prefill_capture_interleaved_layout():
     assert np.array_equal(pu.bits(_rows(cv, bt, 0, slots, layers, False)), v_want)
     e = pu.k_error(pu.bits(_rows(ck, bt, 0, slots, layers, False)), k_want, k_raw)
     assert e["max_err"] <= pu.K_TOL, e
+
+
+@pytest.mark.parametrize("H,D", [(64, 128), (32, 256), (48, 128)])
+@pytest.mark.parametrize("n_layers", [1, 3])
+def test_prefill_capture_wide_rows(H, D, n_layers):
+    """Rows of 512 threads (the kernel without a layer ahead) and of 384."""
+    import paper_2606_26631_gb300 as prcr
+    import parity_util as pu
+    M, first, sec = 37, 5, (D // 8, D // 8, D // 4)
+    g = torch.Generator(device=DEV).manual_seed(H)
+    k, v = (torch.randn((n_layers, M, H, D), device=DEV, generator=g).to(torch.bfloat16) for _ in range(2))
+    coords = torch.randint(0, 900, (M, 3), device=DEV, generator=g, dtype=torch.int32)
+    store_k, store_v = (torch.zeros((1, n_layers, M, H, D), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    ck, cv = (torch.full((1, n_layers, M + 9, H, D), CANARY_BITS, dtype=torch.int16, device=DEV).view(torch.bfloat16) for _ in range(2))
+    got = torch.zeros((1, M, 3), dtype=torch.int32, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    prcr.prefill_capture(prcr.rope_cfg(n_layers, H, D, sec, 1e6), prcr.store_desc(store_k, store_v, got), prcr.cache_contiguous(ck, cv), 0, 0, 0,
+                         first, k, v, coords, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(got[0], coords)
+    assert torch.equal(store_k[0], k) and torch.equal(store_v[0], v)
+    k_raw, v_raw = pu.bits(k.transpose(0, 1)), pu.bits(v.transpose(0, 1))
+    _, _, k_want, v_want = O.prefill_capture(k_raw, v_raw, coords.cpu().numpy(), D, sec, 1e6)
+    rows = slice(first, first + M)
+    assert np.array_equal(pu.bits(cv[0, :, rows].transpose(0, 1)), v_want)
+    assert pu.k_error(pu.bits(ck[0, :, rows].transpose(0, 1)), k_want, k_raw)["max_err"] <= pu.K_TOL
+    for c in (ck, cv):
+        assert bool((c.view(torch.int16)[0, :, :first] == CANARY_BITS).all()) and bool((c.view(torch.int16)[0, :, first + M:] == CANARY_BITS).all())

@@ -155,3 +155,11 @@ def test_cached_logits_fill_the_gpu_once(D, ctas):
     logits, tail = F.launches()
     assert "select_logits" in logits[0] and "select_tail" in tail[0]
     assert 0.9 * 152 * ctas < logits[1][0] <= 152 * ctas
+
+
+def test_capture_of_wide_rows_keeps_two_ctas_per_sm():
+    """A row of 512 threads takes the capture kernel of 64 registers a thread."""
+    for H, D, wide in ((8, 128, False), (32, 128, False), (48, 128, False), (64, 128, True), (32, 256, True)):
+        F.launches()
+        assert F.capture(F.cfg(2, H, D), 900) == 0
+        assert ("capture_kernelILi512E" in F.launches()[0][0]) == wide, (H, D)
