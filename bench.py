@@ -45,9 +45,9 @@ SPEC_HBM_GBS = 8000.0
 # workload, from an ncu capture; valid only for the kernel source it was
 # measured on (its sha256 prefix), reported as null otherwise.
 TRAFFIC = {
-    # captured on the stress shape cut to 2 sequences (8,192 tokens: 1,202,836,992 B
-    # read + 1,150,053,632 B written) and scaled by the 16x more tokens of a full launch
-    ("stress", "06ba5c35f9d5221d"): 37646249984,
+    # captured on the stress shape cut to 2 sequences (8,192 tokens: 1,203,277,312 B
+    # read + 1,150,387,200 B written) and scaled by the 16x more tokens of a full launch
+    ("stress", "df5ffd89c9a19a1b"): 37658632192,
 }
 
 # the Table 3 shapes (Qwen3-VL-8B dimensions, a 768-token image, K = 32 and

@@ -45,7 +45,10 @@ constexpr int kEarlyLayers = 4;
 // Hints only: nothing read here is used for anything else, so indices or offsets
 // that are wrong cost time alone; what is prefetched lies in the store whatever
 // they hold. The plan takes ~8 us,
-// of which the lookups here leave a few. Only the first wave's CTAs are there by
+// of which the lookups here, three dependent loads a token, leave a few: two tokens a
+// warp at most (a CTA of few short heads has up to 256 tokens, and all of them made 9
+// sequences x ~290 tokens x 21 layers x 3 heads of 16 12.8 -> 16.2 us, 12 x ~600 x 8 x
+// 1 of 32 16.5 -> 25.8; now 13.3 and 15.2). Only the first wave's CTAs are there by
 // then. Measured (calls in a row, without | 2 layers | 4 | 12): 3 x 267 tokens x 8
 // layers x 8 heads of 128 32.2 | 31.9 | 31.1 | 31.1 us, 5 x 443 x 32 x 5 41.2 | 40.6
 // | 39.9 | 39.9, 12 x 201 x 11 x 5 of 256 49.9 | 49.9 | 49.0 | 49.0, 8 x ~512 x 28
@@ -56,7 +59,7 @@ __device__ __forceinline__ void prefetch_rows(const RebindArgs& a) {
     const int l = int(blockIdx.y) * a.layers_per_cta + (lane >> 1);
     const int n = min(kEarlyLayers, a.layers_per_cta);
     const uint32_t bytes = uint32_t(a.lanes) * 32;  // of a row
-    for (int t = warp; t < a.tok_per_cta; t += nw) {
+    for (int t = warp; t < min(a.tok_per_cta, 2 * nw); t += nw) {
         const int64_t j = int64_t(blockIdx.x) * a.tok_per_cta + t;
         if (j >= a.total_k) break;
         const int m = a.idx[j];
