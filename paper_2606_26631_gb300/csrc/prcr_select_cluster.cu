@@ -979,19 +979,20 @@ cudaError_t launch_select_tail(const SelectArgs& a, int n_seqs, bool fine, cudaS
 // keys add about three per token for its cos/sin; the second path grows with their
 // number per SM, at first faster (its grids fill) than in proportion. The constants are
 // fitted per head_dim to 41,871 drawn calls timed both ways (1..48 sequences of
-// 128..16,384 tokens, 1..8 KV heads, groups of 1..7): the chosen path is 0.1 to 0.4 %
-// behind the better one on average; with one line for all head dims, linear, in rows of
-// 128, 0.6 to 2.6 % and twice as slow at worst. Some of them, us, fused | two kernels: raw
+// 128..16,384 tokens, 1..8 KV heads, groups of 1..7) and 7080 of 9..64 KV heads: the
+// chosen path is 0.1 to 0.4 % behind the better one on average, with more heads 0.5 to
+// 1 % (3.6 % cached at 256); with one line for all head dims, linear, in rows of 128,
+// 0.6 to 2.6 %, 1.3 to 13 %, and twice as slow at worst. Some of them, us, fused | two kernels: raw
 // keys, 8 heads of 128, 1 sequence of 1024 tokens 12.2 | 12.9, of 1536 14.2 | 13.3; 7 of
 // 4096 27.5 | 30.2; 40 of 2048 x 8 heads of 64 46.0 | 36.2, 7 of 8192 37.1 | 29.9; 1 of
 // 1024 x 8 of 256 18.0 | 26.3. Cached keys, 8 heads of 128, 1 of 2048 13.3 | 13.7, of
 // 3072 15.8 | 14.7; 7 of 4096 18.8 | 19.8; 16 of 4096 43 | 35; 8 heads of 256, 7 of 1536
 // 16.6 | 17.2, of 3072 24.4 | 22.9.
 struct FusedLine {
-    double rows, linear, root;
+    double rows, heads, linear, root;
 };
-constexpr FusedLine kFusedLine[2][3] = {{{500, 0.45, 55}, {330, 0.2, 55}, {370, 1.7, 43}},   // raw keys: head_dim 64, 128, 256
-                                        {{740, 0.15, 34}, {600, 0.65, 17}, {280, 0.7, 17}}};  // cached keys
+constexpr FusedLine kFusedLine[2][3] = {{{590, 10, 0.33, 52}, {330, 0, 0.2, 55}, {490, 7, 1.5, 27}},   // raw keys: head_dim 64, 128, 256
+                                        {{850, 37, 0.16, 30}, {600, 5, 0.75, 9}, {280, 0, 0.7, 17}}};  // cached keys
 template <int D, bool CACHED>
 cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t stream, bool* done) {
     auto kern = select_fused_kernel<D, CACHED>;
@@ -1004,7 +1005,8 @@ cudaError_t try_fused(const SelectArgs& a, int n_seqs, int sms, cudaStream_t str
     const int64_t per_token = a.n_kv_heads + (CACHED ? 0 : 3);
     const double spread = double(n_seqs) * a.n_tokens * per_token / sms;
     const FusedLine c = kFusedLine[CACHED][D / 128];
-    if (f.total > kMaxDynSmem || double(t.tok_per_cta * per_token) > c.rows + c.linear * spread + c.root * std::sqrt(spread)) return cudaSuccess;
+    const double line = c.rows + c.heads * per_token + c.linear * spread + c.root * std::sqrt(spread);
+    if (f.total > kMaxDynSmem || double(t.tok_per_cta * per_token) > line) return cudaSuccess;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = cluster_config(n_seqs * t.cluster, kFusedThreads, t.cluster, f.total, stream, attr);
     *done = true;

@@ -163,3 +163,15 @@ def test_capture_of_wide_rows_keeps_two_ctas_per_sm():
         F.launches()
         assert F.capture(F.cfg(2, H, D), 900) == 0
         assert ("capture_kernelILi512E" in F.launches()[0][0]) == wide, (H, D)
+
+
+def test_selection_takes_the_faster_path():
+    """Points where one kernel and two were measured at least a tenth apart."""
+    for cached, D, H, g, seqs, tokens, one in ((False, 128, 8, 4, 1, 768, True), (False, 128, 8, 4, 1, 4096, False), (False, 64, 8, 4, 1, 4096, False),
+                                               (False, 64, 8, 4, 7, 1536, True), (False, 64, 8, 4, 40, 2048, False), (False, 256, 8, 4, 1, 1024, True),
+                                               (True, 64, 8, 4, 40, 3072, False), (True, 64, 32, 3, 1, 214, True), (True, 64, 64, 1, 8, 311, True),
+                                               (True, 128, 8, 4, 1, 1024, True), (True, 128, 8, 4, 16, 4096, False), (True, 128, 2, 4, 1, 8192, False),
+                                               (True, 256, 8, 4, 7, 512, True), (True, 256, 8, 4, 16, 2048, False)):
+        F.launches()
+        assert (F.select_cached if cached else F.select_raw)(F.cfg(1, H, D), seqs, g, tokens) == 0
+        assert ("select_fused" in F.launches()[0][0]) == one, (cached, D, H, g, seqs, tokens)
