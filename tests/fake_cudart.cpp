@@ -89,7 +89,9 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* c) {
-    *n = 152 / int(c->gridDim.x);
+    // as a GB300 answers for one CTA per SM: clusters do not fill every GPC
+    static const int held[17] = {0, 152, 70, 46, 36, 28, 23, 15, 15, 15, 13, 8, 8, 7, 7, 7, 7};
+    *n = held[c->gridDim.x];
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
